@@ -60,6 +60,16 @@ size_t sched_bytes(const gdn_desc* d)
     return sizeof(gdn::SchedHeader) + round256((size_t)(d->num_seqs > 0 ? d->num_seqs : 1) * sizeof(int32_t));
 }
 
+// The operand ring that the tensor-core path uses for calls with few chains (in host-memory mode: for its smallest groups of
+// requests); nothing for other calls.  It is the last part of the workspace: a workspace without it still serves.
+size_t ring_bytes(const gdn_desc* d)
+{
+    const bool tc = d->io_dtype == GDN_BF16 && d->head_k_dim == 128 && d->head_v_dim == 128 && d->kernel != GDN_KERNEL_FP32_SIMT;
+    int64_t chains = (int64_t)d->num_seqs * d->num_v_heads;
+    if (d->memory == GDN_MEM_HOST && chains > gdn::kRingClusters) chains = gdn::kRingClusters;
+    return tc && chains <= gdn::kRingClusters ? round256((size_t)chains * gdn::kRingSlots * gdn::kRingSlotBytes) : 0;
+}
+
 // Scheduler + forward kernel of one (sub-)batch on `stream`; sets the launch count of this thread.
 int32_t run_kernels(gdn::Problem& p, gdn::Sched sched, bool use_tc, int32_t kernel, int32_t io_dtype, cudaStream_t stream)
 {
@@ -131,7 +141,7 @@ int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, 
     const bool tc_shape = d->io_dtype == GDN_BF16 && d->head_k_dim == 128 && d->head_v_dim == 128;
     if (d->kernel == GDN_KERNEL_TCGEN05 && !tc_shape) return GDN_ERR_UNSUPPORTED;
     if (d->num_seqs == 0) return GDN_OK;
-    const size_t need = gdn_workspace_size(d);
+    const size_t ring = ring_bytes(d), need = gdn_workspace_size(d) - ring;
     if (!d->workspace || d->workspace_bytes < need) return GDN_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(d->workspace) & 255u) != 0) return GDN_ERR_INVALID_ARG;
     if (d->memory == GDN_MEM_HOST) {
@@ -147,6 +157,7 @@ int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, 
     sched.header = (gdn::SchedHeader*)ws;
     sched.order = (int32_t*)(ws + sizeof(gdn::SchedHeader));
     ws += sched_bytes(d);
+    sched.ring = ring && d->workspace_bytes >= need + ring ? (uint8_t*)d->workspace + need : nullptr;
 
     gdn::Problem p;
     memset(&p, 0, sizeof p);
@@ -255,7 +266,7 @@ extern "C" {
 size_t gdn_workspace_size(const gdn_desc* d)
 {
     if (!desc_shape_ok(d)) return 0;
-    size_t total = sched_bytes(d);
+    size_t total = sched_bytes(d) + ring_bytes(d);
     if (d->memory == GDN_MEM_HOST) {
         const Sizes s = sizes_of(d);
         total += round256(s.cu) + 2 * round256(s.qk) + round256(s.v) + 2 * round256(s.gb) +

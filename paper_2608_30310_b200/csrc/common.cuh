@@ -26,6 +26,11 @@ struct Problem {
 
 constexpr float kNormEps = 1.0e-6f;   // added to the squared norm of q and k rows in the fused input stage
 
+// Operand ring of the tensor-core path for few chains (see gdn_tc.cu): slots per cluster, and the largest number of
+// clusters (four CTAs each), hence of chains, that it is used for.
+constexpr uint32_t kRingSlots = 9, kRingSlotBytes = 32768 + 512;
+constexpr int64_t kRingClusters = 37;
+
 // Scheduler scratch at the head of the workspace.
 struct SchedHeader {
     uint32_t next_item;       // dynamic work counter, reset by the scheduler kernel
@@ -39,6 +44,8 @@ struct Sched {
     SchedHeader* header;
     int32_t* order;           // [N] request indices, longest first; null: the requests in the order given (the
                               // tensor-core path with a single request, which then needs no scheduler kernel)
+    uint8_t* ring;            // kRingSlots * kRingSlotBytes per chain, for calls of up to kRingClusters chains on the
+                              // tensor-core path; null: none (the call then runs without clusters)
 };
 
 cudaError_t launch_scheduler(const int32_t* cu, int32_t num_seqs, const Sched& s, cudaStream_t stream);

@@ -7,40 +7,37 @@
 //
 //   G_t   = cumsum(g) inside the chunk;  Gam[t,s] = exp(G_t - G_s) (t >= s)
 //   Gram  = [K;Q] K^T                        (MMA, 128 x 64: rows 0-63 K K^T, rows 64-127 Q K^T)
-//   A     = strict_lower(beta_t Gam (K K^T)) and X = (I + A)^-1 enter as T' = X diag(beta), T'' = X diag(beta e^G).
-//           With beta moved to the columns, A^ = strict_lower(Gam (K K^T)) diag(beta) and P^ = (I + A^)^-1 (8 x 8
-//           diagonal blocks by substitution in fp32, block merges on mma.sync bf16 with ldmatrix-fed fragments), one
-//           has T' = diag(beta) P^ and T'' = diag(beta) P^ diag(e^G): P^ itself and its column-scaled copy
-//           P^ diag(e^G) are the two MMA operands, and the common row factor beta moves behind the products
+//   A^    = strict_lower(Gam (K K^T)) diag(beta),  P^ = (I + A^)^-1.  With A = strict_lower(beta_t Gam (K K^T)) and
+//           X = (I + A)^-1 one has X diag(beta) = diag(beta) P^: P^ itself and its column-scaled copy P^ diag(e^G) are the
+//           MMA operands T' and T'', and the common row factor beta moves behind the products
 //   P     = lower_incl(Gam (Q K^T)) diag(beta)    (beta on the columns here as well)
 //   W~^T  = K^T (P^ diag(e^G))^T              (MMA, 128(dk) x 64)
 //   Dl~^T = V^T P^^T - S0 W~^T                (two MMAs into one accumulator, second negated; Delta = Dl~ diag(beta))
 //   O^T   = (S0 Q^T) diag(e^G) + Dl~^T P^T    (two MMAs, combined in the epilogue)
 //   S     = e^{G_C} S0 + (Dl~ diag(beta e^{G_C - G}))^T K   (MMA accumulating in place: tensor memory holds S / c with
-//                                              c the running product of the chunk decays, folded into the
-//                                              per-token factors; rescaled before c drops below 2^-40)
+//                                              c the running product of the chunk decays; rescaled before c drops
+//                                              below 2^-40)
 //
-// The CTA is warp-specialised and software-pipelined over the chunks of all chains it owns (28 warps):
-//   warp 0       TMA producer: K/Q tiles two chunks ahead (3 slots), V one chunk ahead (1 slot)
-//   warp 1       issues the chain MMAs (U^T, S0 W^T, the state update, then S0 Q^T and Dl~^T P^T)
-//   warp 2       issues the Gram MMAs, ahead of the chain (fused input stage: also the query norms of the chunk)
-//   warp 3       decay warp: loads g and beta up to three chunks ahead, scans the log-decay and publishes the
-//                per-chunk decay factors
-//   warps 4-11   group G1 (two warps per TMEM lane window): Gram post-processing of chunk k+1 (A^ straight into the
-//                chunk's T' buffer, P into its P buffer, both in MMA operand layout), then the W^T epilogue of chunk k
-//   warps 12-19  chain group: Delta epilogue, state conversion (and rescaling when due), start states from
-//                init_state, final states
-//   warps 20-23  group G2, two teams of two warps that take alternate chunks: the triangular solve in place in the T'
-//                buffer, then the column-scaled copy T''; the team then issues the W^T MMA itself
-//   warps 24-27  output group: output epilogue of chunk j, off the chain's critical path
-// Every per-chunk loop is kept rolled with 16-column TMEM accesses: straight-line code larger than the
-// instruction caches runs at a fraction of the issue rate, so the static footprint matters as much as the
-// instruction count.
-// Chains (request, v-head) are ordered longest-first by the scheduler kernel and dealt to CTAs in
-// snake order, so each role can walk its CTA's chunk sequence without any broadcast.  Padding rows
-// of a ragged last chunk get beta = 0 and a cumulative decay that makes their rows of A^ and P vanish, which keeps
-// them inert whatever (finite) values follow the request in memory; their outputs are not stored.
-// Every mbarrier wait is bounded: on expiry the CTA records GDN_ERR_TIMEOUT and unwinds.
+// Only the last four lines depend on the state.  The kernel has two forms (CL):
+//
+// Few chains (request, v-head), CL = true: the work of a chain is split over the CTAs of a thread-block cluster:
+//   rank 0        "chain CTA": walks the chunks one after the other with the state resident in tensor memory
+//   ranks 1..R    "prep CTAs": chunk j is prepared by rank 1 + j % R.  Three teams of four warps take a prep CTA's chunks in
+//                 turn; each carries a chunk from its K/Q tiles to the finished operands W~^T, T', P (32 KB, in MMA
+//                 operand layout), which travel to the chain CTA through a small ring in global memory that stays in L2: a
+//                 bulk store out of the prep CTA (30 bytes per cycle), a bulk load into the chain CTA (60-80).  Copies from
+//                 CTA to CTA reach 18 bytes per cycle (25 from three sources), and less beside the chain CTA's own loads.
+// Flow control: the CTAs of a cluster run at the same time, so they signal each other with remote mbarrier arrivals: a
+// chunk's operands are in the ring (prep -> chain), a ring slot has been read (chain -> prep).
+//
+// Many chains, CL = false ("fused CTA"): one CTA per SM does both parts of a chain, with two prep teams and everything in its
+// own shared memory.  Its period per chunk is longer (the parts compete for the SM's issue slots), but no SM waits.
+//
+// Chains are ordered longest-first by the scheduler kernel and dealt to clusters (CTAs) in snake order, so each role can walk
+// its cluster's chunk sequence without any broadcast.  Padding rows of a ragged last chunk get beta = 0 and a cumulative
+// decay that makes their rows of A^ and P vanish, which keeps them inert whatever (finite) values follow the request
+// in memory; their outputs are not stored.  Every mbarrier wait is bounded: on expiry the CTA records
+// GDN_ERR_TIMEOUT and unwinds.
 #include <cuda.h>
 #include "common.cuh"
 #include "ptx.cuh"
@@ -50,139 +47,174 @@ namespace {
 
 using namespace ptx;
 
-constexpr int LDM = 40;                       // bf16 row stride of the merge scratch (80 B: conflict-free ldmatrix)
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr int kThreads = 896;      // 28 warps, see the role table above (at most 72 registers per thread)
+template <bool CL> constexpr int kThreads = CL ? 640 : 768;      // 20 warps (up to 96 registers a thread) / 24 warps (80)
+constexpr uint32_t NT = 3;                    // prep teams per prep CTA
+constexpr uint32_t NSLOT = 3;                 // operand slots in the chain CTA
+constexpr uint32_t OPS_BYTES = 32768;         // W~^T 16 KB, T' 8 KB, P 8 KB
+constexpr uint32_t OPS_W = 0, OPS_TP = 16384, OPS_P = 24576;
+constexpr uint32_t NORM_BYTES = 512;          // fused input stage: 1 / norms of the chunk's key and query rows
+static_assert(OPS_BYTES + NORM_BYTES == kRingSlotBytes, "");
+constexpr uint32_t kClusterCtas = 4;          // of a cluster: one chain CTA, three prep CTAs
 
-// ---- shared memory map (bytes from a 1024-aligned base) ---------------------------------------
-constexpr uint32_t SM_KQ = 0;                 // 3 slots x {2 halves x [128 rows: K 0-63, Q 64-127] x 128 B}  96 KB
-constexpr uint32_t KQ_SLOT = 32768;
-constexpr uint32_t NKQ = 3;
-constexpr uint32_t SM_V = SM_KQ + NKQ * KQ_SLOT;   // 2 halves x [64 rows] x 128 B                          16 KB
-constexpr uint32_t SM_WT = SM_V + 16384;      // W^T [dk][t] bf16, 128 rows x 128 B                          16 KB
-constexpr uint32_t SM_TP = SM_WT + 16384;     // 3 x T' [t][s] bf16: A^ from the post-processing, inverted in place  24 KB
-constexpr uint32_t SM_TPP = SM_TP + 3 * 8192; // T'' [t][s] bf16 (one buffer)                                  8 KB
-constexpr uint32_t SM_P = SM_TPP + 8192;      // 3 x P [t][s] bf16                                           24 KB
-constexpr uint32_t SM_MH = SM_P + 3 * 8192;   // merge scratch of the solve, bf16 [32][LDM]
-constexpr uint32_t MH_BYTES = 32 * LDM * 2;   // one per solve team
-constexpr uint32_t SM_MISC = ((SM_MH + 2 * MH_BYTES + 15) / 16) * 16;
+// ---- shared memory of a chain CTA (bytes from a 1024-aligned base) -----------------------------
+constexpr uint32_t C_OPS = 0;                              // NSLOT operand slots                             96 KB
+constexpr uint32_t C_KQ = C_OPS + NSLOT * OPS_BYTES;       // 2 x {K, Q}, each 2 halves x [64 rows] x 128 B  64 KB
+constexpr uint32_t C_V = C_KQ + 2 * 32768;                 // 2 halves x [64 rows] x 128 B                     16 KB
+constexpr uint32_t C_O = C_V + 16384;                      // 2 x outputs of a chunk on their way out, layout of V  32 KB
+constexpr uint32_t C_MISC = C_O + 2 * 16384;
+// ---- shared memory of a prep CTA: per team K/Q 32 KB | operands 32 KB (same layout as a slot) | T'' 8 KB ------------
+constexpr uint32_t P_TEAM = 32768 + OPS_BYTES + 8192;
+constexpr uint32_t P_OPS = 32768, P_TPP = 32768 + OPS_BYTES;
+constexpr uint32_t P_MISC = NT * P_TEAM;
+// ---- shared memory of a fused CTA: two prep teams and the chain --------------------------------------------------------
+constexpr uint32_t F_KQ = 0;                               // 4 x K/Q tiles; the outputs of a chunk replace its Q   128 KB
+constexpr uint32_t F_W = F_KQ + 4 * 32768;                 // per team W~^T; its first half holds T'' before         32 KB
+constexpr uint32_t F_TP = F_W + 2 * 16384;                 // per team T'                                            16 KB
+constexpr uint32_t F_P = F_TP + 2 * 8192;                  // 3 x P                                                  24 KB
+constexpr uint32_t F_V = F_P + 3 * 8192;                   // V                                                      16 KB
+constexpr uint32_t F_MISC = F_V + 16384;
+static_assert(P_MISC % 1024 == 0 && C_MISC <= P_MISC && F_MISC <= P_MISC, "");
 
-enum Bar {
-    B_FULL_KQ0 = 0, B_FULL_KQ1, B_FULL_KQ2, B_FULL_V, B_GRAM_DONE, B_W_DONE0, B_W_DONE1, B_U_DONE, B_MMA1_DONE,
-    B_MMA3_DONE, B_STATE_DONE, B_KQ_FREE0, B_KQ_FREE1, B_KQ_FREE2, B_P_FREE0, B_P_FREE1, B_P_FREE2,
-    B_TP_FREE0, B_TP_FREE1, B_TP_FREE2,
-    B_GRAM_READ, B_WACC_READ,
-    B_PRE_DONE0, B_PRE_DONE1, B_D_READY, B_SBF_READY, B_ACC23_FREE, B_SQ_DONE,
-    B_DECAY_READY0, B_DECAY_READY1, B_DECAY_READY2, B_DECAY_READY3,
-    B_DECAY_FREE0, B_DECAY_FREE1, B_DECAY_FREE2, B_DECAY_FREE3,
-    B_A_READY0, B_A_READY1, B_A_READY2, B_TP_READY0, B_TP_READY1, B_TP_READY2,
-    B_RQ_READY0, B_RQ_READY1, B_RQ_READY2, B_RQ_READY3, NUM_BARS
+enum ChainBar {
+    CB_OPS_FULL0 = 0, CB_KQ_FULL0 = 3, CB_U = 5, CB_DONE0 = 6, CB_MMA1 = 10, CB_STATE0, CB_STATE1, CB_OUT0, CB_OUT1,
+    CB_ACC_FREE0, CB_ACC_FREE1, CB_DECAY_READY0, CB_DECAY_FREE0 = CB_DECAY_READY0 + 4, CB_RING0 = CB_DECAY_FREE0 + 4,
+    CB_NUM = CB_RING0 + kRingSlots
+};
+enum FusedBar {
+    FB_KQ_FULL0 = 0, FB_KQ_FREE0 = 4, FB_V_FULL = 8, FB_U0, FB_GRAM0 = FB_U0 + 2, FB_W0 = FB_GRAM0 + 2, FB_OPS0 = FB_W0 + 2, FB_MMA1_0 = FB_OPS0 + 2,
+    FB_STATE0 = FB_MMA1_0 + 2, FB_OUT = FB_STATE0 + 2, FB_DONE0, FB_ACC_FREE = FB_DONE0 + 4, FB_DECAY_READY0, FB_DECAY_FREE0 = FB_DECAY_READY0 + 4,
+    FB_NUM = FB_DECAY_FREE0 + 4
+};
+enum PrepBar {
+    PB_KQ_FULL0 = 0, PB_GRAM0 = 3, PB_W0 = 6, PB_OPS0 = 9, PB_SENT0 = 12, PB_DECAY_READY0 = 15, PB_DECAY_FREE0 = 19, PB_CREDIT0 = 23,
+    PB_NUM = PB_CREDIT0 + NT
 };
 
-// Per-chunk decay factors.  The fp32 state lives in tensor memory divided by a running factor c (the product of
-// the chunk decays since the last rescale), so that a chunk update is a plain accumulation; c is folded into
-// the factors below, and the state is rescaled (c back to 1) before c leaves [2^-40, 1].
-//   G2    log2-domain inclusive cumulative decay,  beta
-//   colfb 2^(G2[31] - G2[s]) beta[s] for s < 32: column factors of the purely off-diagonal quadrant of Gam
-//   eG    e^G c_prev         (column factors of T'', so that W^T comes out multiplied by c_prev, as
-//                             S0 = c_prev * stored state; also the output epilogue's factor of (stored state) q)
+// Per-chunk factors.  The fp32 state lives in tensor memory divided by a running factor c (the product of the chunk decays
+// since the last rescale), so that a chunk update is a plain accumulation; c is folded into the factors below, and the
+// state is rescaled (c back to 1) before c leaves [2^-40, 1].
+//   eG    e^G c_prev         (column factors of T'', so that W~^T comes out multiplied by c_prev, as S0 = c_prev * stored
+//                            state; also the output epilogue's factor of (stored state) q)
+// Chain CTA:
 //   bRest beta e^(G_C - G) / c   (Delta' = Delta~ diag(bRest) accumulates onto the stored state)
-//   eGk   the column factors of T'' (= eG; the fused input stage folds the key norms into this copy)
-//   rq    fused input stage only: 1 / norm of the query rows, written by the Gram warp (the outputs are linear in q,
-//         so the query norms multiply the finished output rows)
+//   rq    fused input stage: 1 / norm of the query rows (the outputs are linear in q)
 //   rescale / wb: this chunk starts from a rescaled state: the previous chunk's state epilogue multiplies the
 //   stored state by wb = c_prev e^(G_C) first;  cfin = c after this chunk (final state = cfin * stored state)
-struct __align__(16) Decay { float G2[64], beta[64], eG[64], bRest[64], colfb[32], eGk[64], rq[64]; float wb; float G2mid; float cfin; int rescale; int pad[3]; };
-static_assert(sizeof(Decay) % 16 == 0, "the decay ring is read with 16-byte vector loads");
+// Prep CTA:
+//   G2    log2-domain inclusive cumulative decay, beta;  colfb  2^(G2[31] - G2[s]) beta[s] for s < 32 (column factors of
+//   the quadrant of Gam below the diagonal quadrants);  norms  fused input stage: 1 / norms of the key and query rows
+struct __align__(16) ChainDecay { float eG[64], bRest[64], rq[64]; float wb, cfin; int rescale; int pad; };
+struct __align__(16) PrepDecay { float G2[64], beta[64], eG[64], colfb[32], norms[128]; float G2mid; int pad[3]; };
+struct ChainMisc {
+    ChainDecay decay[4];
+    float norms[NSLOT][128];           // fused input stage: norms of the slot's chunk (copied with the operands)
+};
+struct PrepMisc { PrepDecay decay[4]; };
+// Fused CTA: both in one record.  eGk: eG times the key norms (fused input stage)
+struct __align__(16) FusedDecay { float G2[64], beta[64], eG[64], colfb[32], norms[128]; float G2mid, wb, cfin; int rescale; float bRest[64], eGk[64]; };
+struct FusedMisc { FusedDecay decay[4]; };
 struct Misc {
-    float rk[64];                      // fused input stage: 1 / norm of the chunk's key rows (group G1)
-    Decay decay[4];                    // per-chunk decay factors, ring of 4 (decay warp writes; pre and chain read)
-    unsigned long long bars[NUM_BARS];
+    unsigned long long bars[40];
     uint32_t tmem_base;
     volatile uint32_t abort;
     unsigned long long timeout_ns;
+    union { ChainMisc c; PrepMisc p; FusedMisc f; };
 };
-constexpr uint32_t SM_TOTAL = SM_MISC + ((sizeof(Misc) + 15) / 16) * 16;
-constexpr uint32_t SMEM_BYTES = SM_TOTAL + 1008;   // slack for the manual 1024-byte alignment of a 16-byte aligned base
-static_assert(NKQ == 3, "the K/Q barriers are enumerated per slot");
-static_assert(B_FULL_KQ0 == 0 && B_FULL_V == NKQ && NUM_BARS <= 64, "barrier set-up: the producer's four first, one thread each for the rest");
+static_assert(CB_NUM <= 40 && PB_NUM <= 40 && FB_NUM <= 40, "");
+// the part of the records that a prep team reads / that the chain's epilogues read (CL: the split over a cluster)
+template <bool CL> __device__ __forceinline__ auto& prep_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->p.decay[i]; else return m->f.decay[i]; }
+template <bool CL> __device__ __forceinline__ auto& chain_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->c.decay[i]; else return m->f.decay[i]; }
+__device__ __forceinline__ const float* query_norms(const ChainDecay& dc) { return dc.rq; }
+__device__ __forceinline__ const float* query_norms(const FusedDecay& dc) { return dc.norms + 64; }
+static_assert(offsetof(Misc, c) % 16 == 0, "");
+constexpr uint32_t SM_MISC = P_MISC;         // the same place in every kind of CTA
+constexpr uint32_t SMEM_BYTES = SM_MISC + ((sizeof(Misc) + 15) / 16) * 16 + 1008;   // slack: manual 1024-byte alignment
 static_assert(SMEM_BYTES <= 232448, "exceeds the 227 KB shared memory of one CTA");
 
-// ---- TMEM column map (512 columns x 128 lanes x 32 bit) ----------------------------------------
+// ---- TMEM columns of a chain CTA (512 columns x 128 lanes x 32 bit) ----------------------------------------
 constexpr uint32_t TM_S32 = 0;      // fp32 state S (dv x dk), 128 columns
 constexpr uint32_t TM_SBF = 128;    // bf16 copy of the chunk-start state, 64 columns
 constexpr uint32_t TM_ACC1 = 192;   // Delta^T accumulator (U^T - S0 W^T), 64 columns
-constexpr uint32_t TM_ACC2 = 256;   // S0 Q^T, 64 columns
-constexpr uint32_t TM_ACC3 = 320;   // Delta^T P^T, 64 columns
-constexpr uint32_t TM_GRAM = 384;   // Gram accumulator, 64 columns
-constexpr uint32_t TM_WACC = 448;   // W^T accumulator, 64 columns
+constexpr uint32_t TM_ACC2 = 256;   // 2 x S0 Q^T, 64 columns
+constexpr uint32_t TM_ACC3 = 384;   // 2 x Delta^T P^T, 64 columns
 // The bf16 A operands Delta^T and Delta'^T replace the fp32 accumulator they are computed from, in place: the 16
 // fp32 columns of tokens [16 s, 16 s + 16) become 8 columns of Delta^T followed by 8 columns of Delta'^T.
-constexpr uint32_t TM_DBF = TM_ACC1;        // + 16 s
-constexpr uint32_t TM_DPBF = TM_ACC1 + 8;   // + 16 s
+constexpr uint32_t TM_DBF = 0, TM_DPBF = 8;      // offsets in the Delta accumulator, + 16 s
+// ---- TMEM columns of a prep team: Gram 64, W~^T 64 ----
+constexpr uint32_t TM_TEAM = 128, TM_GRAM = 0, TM_WACC = 64;
+// ---- TMEM columns of a fused CTA: state as in a chain CTA, one accumulator of each kind; each team has 64 columns that
+// hold first its Gram tile, then its W~^T accumulator ----
+constexpr uint32_t TM_F_ACC3 = 320, TM_F_TEAM = 384;
+template <bool CL> __device__ __forceinline__ uint32_t tm_acc2(uint32_t j) { return TM_ACC2 + (CL ? (j & 1u) * 64 : 0u); }
+template <bool CL> __device__ __forceinline__ uint32_t tm_acc3(uint32_t j) { return CL ? TM_ACC3 + (j & 1u) * 64 : TM_F_ACC3; }
 
 constexpr uint32_t ID_GRAM = idesc_bf16(128, 64, 0, 0, 0);    // [K;Q] (K-major) x K (K-major)
 constexpr uint32_t ID_WU = idesc_bf16(128, 64, 1, 0, 0);      // K^T or V^T (M-major) x T (K-major)
 constexpr uint32_t ID_SW = idesc_bf16(128, 64, 0, 1, 1);      // -S0 (TMEM) x W^T (N-major)
 constexpr uint32_t ID_SQ = idesc_bf16(128, 64, 0, 0, 0);      // S0 (TMEM) x Q (K-major)
 constexpr uint32_t ID_DP = idesc_bf16(128, 64, 0, 0, 0);      // Delta^T (TMEM) x P (K-major)
-constexpr uint32_t ID_DK = idesc_bf16(128, 128, 0, 1, 0);     // Delta'^T (TMEM) x K (N-major)
+constexpr uint32_t ID_DK = idesc_bf16(128, 64, 0, 1, 0);      // Delta'^T (TMEM) x half of K (N-major)
 
 struct TcParams {
     Problem p;
     Sched s;
     unsigned long long wait_timeout_ns;   // bound of every device-side wait
     int32_t skip_kq_load;         // testing aid: chunk whose K/Q copy is left out (-1: none)
+    uint32_t csize;               // CTAs per cluster (1 chain CTA + R prep CTAs)
+    uint32_t ring;                // slots of a cluster's operand ring, a multiple of NT * R: a ring slot and its credits belong
+                                  // to one team, so that no wait looks more than one phase ahead
 };
 
-// Walks the chunk sequence of one CTA: chains dealt in snake order over the longest-first list,
+// Walks the chunk sequence of one cluster: chains dealt in snake order over the longest-first list,
 // chunks of 64 rows inside each chain.  Every role keeps its own cursor(s).
 struct ChunkCursor {
-    const Problem* p;
-    const int32_t* order;
+    const TcParams* prm;
     int r, h, hq, row_begin, row_end, nchunks, c;
     bool valid;
 
-    __device__ void init(const Problem* pp, const int32_t* ord)
+    __device__ void init(const TcParams* pp)
     {
-        p = pp; order = ord; r = -1;
+        prm = pp; r = -1;
         next_chain();
     }
-    __device__ static uint32_t item_of(int round)
+    __device__ static uint32_t item_of(const TcParams* prm, int round)
     {
-        const uint32_t G = gridDim.x, b = blockIdx.x;
+        const uint32_t G = gridDim.x / prm->csize, b = blockIdx.x / prm->csize;
         return (uint32_t)round * G + ((round & 1) ? (G - 1 - b) : b);
     }
-    // The next work item of this CTA after round r that has at least one chunk, kept out of line (integer divisions,
+    // The next work item of this cluster after round r that has at least one chunk, kept out of line (integer divisions,
     // dependent global loads and a loop over empty requests, needed once per chain by every role; everything goes and
     // comes back in registers): x = first row, y = end row, z = v-head | q/k head << 16, w = its round, or -1 when
-    // the CTA's items are exhausted.
-    __device__ __noinline__ static int4 find_chain(const Problem* p, const int32_t* order, int r)
+    // the cluster's items are exhausted.
+    __device__ __noinline__ static int4 find_chain(const TcParams* prm, int r)
     {
-        const uint32_t num_items = (uint32_t)p->num_seqs * (uint32_t)p->Hv;
+        const Problem& p = prm->p;
+        const uint32_t num_items = (uint32_t)p.num_seqs * (uint32_t)p.Hv;
         for (;;) {
             ++r;
-            const uint32_t item = item_of(r);
+            const uint32_t item = item_of(prm, r);
             if (item >= num_items) return make_int4(0, 0, 0, -1);
-            const int n = order ? order[item / p->Hv] : (int)(item / p->Hv);   // no order list: requests as given
-            const int h = item % p->Hv;
-            const int hq = h / (p->Hv / p->Hq);
-            const int a = p->cu[n], b = p->cu[n + 1];
+            const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);   // no order list: requests as given
+            const int h = item % p.Hv;
+            const int hq = h / (p.Hv / p.Hq);
+            const int a = p.cu[n], b = p.cu[n + 1];
             if (b - a > 0) return make_int4(a, b, h | (hq << 16), r);
         }
     }
     // Row range and heads of one work item: x = first row, y = end row, z = v-head | q/k head << 16, w = request index.
-    __device__ __noinline__ static int4 lookup(const Problem* p, const int32_t* order, uint32_t item)
+    __device__ __noinline__ static int4 lookup(const TcParams* prm, uint32_t item)
     {
-        const int n = order ? order[item / p->Hv] : (int)(item / p->Hv);
-        const int h = item % p->Hv;
-        const int hq = h / (p->Hv / p->Hq);
-        return make_int4(p->cu[n], p->cu[n + 1], h | (hq << 16), n);
+        const Problem& p = prm->p;
+        const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);
+        const int h = item % p.Hv;
+        const int hq = h / (p.Hv / p.Hq);
+        return make_int4(p.cu[n], p.cu[n + 1], h | (hq << 16), n);
     }
     // moves to the next chain that has at least one chunk
     __device__ void next_chain()
     {
-        const int4 ci = find_chain(p, order, r);
+        const int4 ci = find_chain(prm, r);
         r = ci.w;
         valid = ci.w >= 0;
         row_begin = ci.x; row_end = ci.y; h = ci.z & 0xffff; hq = ci.z >> 16;
@@ -192,6 +224,12 @@ struct ChunkCursor {
     __device__ void advance()
     {
         if (++c >= nchunks) next_chain();
+    }
+    __device__ void advance(int n)
+    {
+        int over = c + n;
+        while (valid && over >= nchunks) { over -= nchunks; next_chain(); }
+        c = over;
     }
     __device__ int row0() const { return row_begin + c * 64; }
     __device__ int nvalid() const { return min(64, row_end - row0()); }
@@ -206,27 +244,50 @@ struct Ctx {
     __device__ uint32_t bar(int i) const { return sb + SM_MISC + (uint32_t)offsetof(Misc, bars) + 8u * i; }
     __device__ bool stop() const { return __shfl_sync(0xffffffffu, misc->abort, 0) != 0u; }
     // Bounded wait.  On expiry it raises the CTA-wide abort flag; from then on no wait blocks any more, so
-    // every role still runs through its (data-independent) loop structure, keeps meeting its warpgroup
+    // every role still runs through its (data-independent) loop structure, keeps meeting its named
     // barriers and reaches the end of the kernel; the results are garbage and the host sees the status word.
-    __device__ bool wait(int i, uint32_t parity) const
+    // (A ready barrier costs a few cycles; a try_wait that has to wait suspends the warp in hardware, without polling, and
+    // returns about 90 cycles after the last arrival.)
+    __device__ __forceinline__ void wait(int i, uint32_t parity) const
     {
         const uint32_t b = bar(i);
-        if (mbar_try_wait(b, parity)) return true;
-        return wait_slow(b, parity, misc);
+        if (!mbar_try_wait(b, parity)) wait_slow(b, parity, misc);
     }
-    // kept out of line: the kernel has some sixty wait sites and its static code size matters
-    __device__ __noinline__ static bool wait_slow(uint32_t b, uint32_t parity, Misc* misc)
+    // kept out of line: the kernel has many wait sites and its static code size matters
+    __device__ __noinline__ static void wait_slow(uint32_t b, uint32_t parity, Misc* misc)
     {
-        if (misc->abort) return true;
-        const uint64_t t0 = globaltimer_ns();
-        for (;;) {
-            // suspended in hardware until the phase completes (or ~20 us pass): no polling instructions
-            if (mbar_try_wait_hint(b, parity, 20000u)) return true;
-            if (misc->abort) return true;
-            if (globaltimer_ns() - t0 > misc->timeout_ns) { misc->abort = 1u; return true; }
+        uint64_t t0 = 0;
+        while (!mbar_try_wait(b, parity)) {
+            if (misc->abort) return;
+            const uint64_t t = globaltimer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > misc->timeout_ns) { misc->abort = 1u; return; }
+        }
+    }
+    // for barriers that the other CTAs of the cluster arrive on
+    __device__ __forceinline__ void wait_cluster(int i, uint32_t parity) const
+    {
+        const uint32_t b = bar(i);
+        if (!mbar_try_wait_cluster(b, parity)) wait_cluster_slow(b, parity, misc);
+    }
+    __device__ __noinline__ static void wait_cluster_slow(uint32_t b, uint32_t parity, Misc* misc)
+    {
+        uint64_t t0 = 0;
+        while (!mbar_try_wait_cluster(b, parity)) {
+            if (misc->abort) return;
+            const uint64_t t = globaltimer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > misc->timeout_ns) { misc->abort = 1u; return; }
         }
     }
 };
+
+// Hand-overs from the epilogue warps of a chain CTA to its MMA warp, on named barriers (a hardware barrier wakes its
+// waiter sooner than an mbarrier does, and these sit on the serial path of a chain).  The waits cannot outlast
+// the bounded mbarrier waits: the arriving warps run through their loop whatever happens.
+enum HandOver { HB_SBF0 = 8, HB_SBF1 = 9, HB_DP = 10, HB_D = 11 };
+template <int WARPS> __device__ __forceinline__ void hand_over_arrive(int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(WARPS * 32 + 32) : "memory"); }
+template <int WARPS> __device__ __forceinline__ void hand_over_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(WARPS * 32 + 32) : "memory"); }
 
 // One arrival per warp: every lane has fenced its own TMEM / shared-memory accesses, the warp converges,
 // lane 0 arrives.  (A full-warp arrive is 32 serialized shared-memory atomics on one address.)
@@ -235,22 +296,29 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);
 }
-// ---- small bf16 tensor-core helpers for the block merges of the triangular solve --------------------
-// Four 8x8 bf16 matrices of the 16 x 16 tile at (row0, col0) of a row-major shared-memory matrix:
-// plain -> A fragment {a0..a3}; transposed -> B fragments {b0, b1} of the two 8-column halves.
-__device__ __forceinline__ uint32_t tile_addr(uint32_t base, int ld, int row0, int col0, int lane)
-{
-    return base + (uint32_t)(((row0 + (lane & 7) + ((lane >> 3) & 1) * 8) * ld + col0 + (lane >> 4) * 8) * 2);
-}
+// ---- small bf16 tensor-core helpers for the triangular solve ----------------------------------------
 __device__ __forceinline__ void ldm_x4(uint32_t (&r)[4], uint32_t addr)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void ldm_x4_trans(uint32_t (&r)[4], uint32_t addr)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldm_x2(uint32_t (&r)[2], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldm_x2_trans(uint32_t (&r)[2], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+// stores four 8 x 8 matrices transposed: lane 8 m + i gives the address of the row that receives column i of matrix m
+__device__ __forceinline__ void stm_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
@@ -258,686 +326,715 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// same four 8 x 8 matrices of a 64 x 64 bf16 tile kept in MMA operand layout: 128-byte rows, 16-byte chunk
-// index XORed with (row & 7)
-__device__ __forceinline__ uint32_t sw_off(int row, int col)
-{
-    return (uint32_t)(row * 128 + ((((col >> 3) ^ (row & 7))) << 4) + (col & 7) * 2);
-}
-__device__ __forceinline__ uint32_t tile_addr_sw(uint32_t base, int row0, int col0, int lane)
-{
-    return base + sw_off(row0 + (lane & 7) + ((lane >> 3) & 1) * 8, col0 + (lane >> 4) * 8);
-}
-// c (16 x 16, two 8-column halves) += A tile * B tile, each given by its per-lane ldmatrix address
-__device__ __forceinline__ void tile16_mma_at(float (&c)[2][4], uint32_t a_addr, uint32_t b_addr)
-{
-    uint32_t a[4], b[4];
-    ldm_x4(a, a_addr);
-    ldm_x4_trans(b, b_addr);
-    mma_bf16(c[0], a, b[0], b[1]);
-    mma_bf16(c[1], a, b[2], b[3]);
-}
-// stores sign * c as bf16 at D[r0.., n0..+16) (row-major, ld elements)
-__device__ __forceinline__ void tile16_store(const float (&c)[2][4], float sign, uint8_t* D, int ld, int r0, int n0, int lane)
-{
-    const int g = lane >> 2, t4 = lane & 3;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        *reinterpret_cast<uint32_t*>(D + ((r0 + g) * ld + n0 + 8 * h + 2 * t4) * 2) = pack_bf16x2(sign * c[h][0], sign * c[h][1]);
-        *reinterpret_cast<uint32_t*>(D + ((r0 + g + 8) * ld + n0 + 8 * h + 2 * t4) * 2) = pack_bf16x2(sign * c[h][2], sign * c[h][3]);
-    }
-}
-// 8 x 8 variants for the first merge level (two independent 8 x 8 problems per instruction pair)
-__device__ __forceinline__ void ldm_x2(uint32_t (&r)[2], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
-__device__ __forceinline__ void ldm_x2_trans(uint32_t (&r)[2], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
 // rows 0-7 of (A[8 x 8] * B[8 x 8]) in c[0], c[1] (row lane / 4, columns 2 (lane % 4) + {0, 1})
 __device__ __forceinline__ void mma_8x8(float (&c)[4], uint32_t a0, uint32_t b0)
 {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(0u), "r"(b0));
 }
-__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
+// transpose of an 8 x 8 bf16 matrix held one row pair per lane quad: accumulator layout -> B operand layout
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t a)
 {
     uint32_t d;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
     return d;
+}
+// byte offset in a 64 x 64 bf16 tile in MMA operand layout: 128-byte rows, 16-byte chunk index XORed with (row & 7)
+__device__ __forceinline__ uint32_t sw_off(int row, int col)
+{
+    return (uint32_t)(row * 128 + ((((col >> 3) ^ (row & 7))) << 4) + (col & 7) * 2);
+}
+// ldmatrix address of the four 8 x 8 matrices of the 16 x 16 tile at (row0, col0), A fragment order
+__device__ __forceinline__ uint32_t tile_addr_sw(uint32_t base, int row0, int col0, int lane)
+{
+    return base + sw_off(row0 + (lane & 7) + ((lane >> 3) & 1) * 8, col0 + (lane >> 4) * 8);
 }
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
-// ================================================================================================
-// warp 0: TMA producer.  Its first tile copies are issued before the CTA-wide start-up barrier (begin), so that they
-// are in flight while tensor memory is allocated, the other barriers are set up and the other roles find their work.
-// ================================================================================================
-struct Producer {
-    ChunkCursor ckq, cv;                 // K/Q runs two chunks ahead of V
-    uint32_t jkq;
-
-    __device__ void load_kq(const Ctx& cx, const TcParams& prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
-    {
-        const uint32_t slot = jkq % NKQ, dst = cx.sb + SM_KQ + slot * KQ_SLOT, bar = cx.bar(B_FULL_KQ0 + slot);
-        if ((int32_t)jkq != prm.skip_kq_load) {           // testing aid: the skipped tile never arrives
-            if (elect_one()) {
-                mbar_arrive_expect_tx(bar, 32768u);
-                tma_load_2d(dst, tm_k, ckq.hq * 128, ckq.row0(), bar);
-                tma_load_2d(dst + 16384, tm_k, ckq.hq * 128 + 64, ckq.row0(), bar);
-                tma_load_2d(dst + 8192, tm_q, ckq.hq * 128, ckq.row0(), bar);
-                tma_load_2d(dst + 24576, tm_q, ckq.hq * 128 + 64, ckq.row0(), bar);
-            }
-            __syncwarp();
-        }
-        ckq.advance();
-        ++jkq;
-    }
-    // needs only the barriers of the K/Q slots
-    __device__ void begin(const Ctx& cx, const TcParams& prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
-    {
-        ckq.init(&prm.p, prm.s.order);
-        cv = ckq;
-        jkq = 0;
-        while (jkq < NKQ - 1 && ckq.valid) load_kq(cx, prm, tm_q, tm_k);
-    }
-    __device__ void run(const Ctx& cx, const TcParams& prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
-                        const CUtensorMap* tm_v)
-    {
-#pragma unroll 1
-        for (uint32_t j = 0; cv.valid && !cx.stop(); ++j) {
-            // V(j): the single slot is free once U^T MMA of chunk j-1 has completed
-            if (j >= 1) cx.wait(B_U_DONE, (j - 1) & 1u);
-            const uint32_t bar = cx.bar(B_FULL_V);
-            if (elect_one()) {
-                mbar_arrive_expect_tx(bar, 16384u);
-                tma_load_2d(cx.sb + SM_V, tm_v, cv.h * 128, cv.row0(), bar);
-                tma_load_2d(cx.sb + SM_V + 8192, tm_v, cv.h * 128 + 64, cv.row0(), bar);
-            }
-            __syncwarp();
-            cv.advance();
-            // K/Q(j+2): its slot held chunk j-1, free once the state-update MMA of chunk j-1 has completed
-            if (ckq.valid) {
-                if (jkq >= NKQ) cx.wait(B_KQ_FREE0 + jkq % NKQ, ((jkq / NKQ) - 1u) & 1u);
-                load_kq(cx, prm, tm_q, tm_k);
-            }
-        }
-    }
-};
-
 // advances the start-address field of a shared-memory descriptor by a byte offset
 __device__ __forceinline__ uint64_t desc_add(uint64_t d, uint32_t bytes) { return d + (uint64_t)(bytes >> 4); }
 
-// Fused input stage, Gram warp's part (inlined into the warp's fused-stage instance only): 1 / norm of the query rows of
-// chunk j from its Q tile, for the output epilogue, which scales the finished output rows with them (the
-// outputs are linear in q).  The warp has just issued the chunk's Gram MMAs and has nothing else to do until the
-// next tiles land, and nothing upstream of the output epilogue waits for these numbers.
-__device__ __forceinline__ void query_norms(const Ctx& cx, uint32_t j, int lane)
+// The tensor maps are three-dimensional, [half head][row][64 values], so that one copy brings the 128 values of 64 rows as two
+// 64-value halves (a TMA instruction costs its issuer some 130 cycles).
+// One tile: 2 halves x [64 rows] x 128 bytes
+__device__ __forceinline__ void load_tile(uint32_t dst, const CUtensorMap* tm, int head, int row, uint32_t bar)
 {
-    const uint8_t* qt = cx.sm + SM_KQ + (j % NKQ) * KQ_SLOT + 8192;      // Q rows of the two 64-column halves
-    float s0 = 0.f, s1 = 0.f;
-#pragma unroll 1
-    for (int i = 0; i < 16; ++i) {
-        // 16-byte pieces of the rows in an order that spreads the lanes over the banks (the sum does not care)
-        const uint32_t off = (uint32_t)(i >> 3) * 16384u + (uint32_t)(((i + lane) & 7) << 4);
-        const uint4 x0 = *reinterpret_cast<const uint4*>(qt + off + lane * 128);
-        const uint4 x1 = *reinterpret_cast<const uint4*>(qt + off + (lane + 32) * 128);
-        const uint32_t w0[4] = {x0.x, x0.y, x0.z, x0.w}, w1[4] = {x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            s0 = fmaf(bf_lo(w0[e]), bf_lo(w0[e]), s0); s0 = fmaf(bf_hi(w0[e]), bf_hi(w0[e]), s0);
-            s1 = fmaf(bf_lo(w1[e]), bf_lo(w1[e]), s1); s1 = fmaf(bf_hi(w1[e]), bf_hi(w1[e]), s1);
-        }
-    }
-    const float rq0 = rsqrtf(s0 + kNormEps), rq1 = rsqrtf(s1 + kNormEps);     // tokens lane and lane + 32
-    // the ring slot is this chunk's once its decay factors are published (the decay warp waits for the slot's last reader)
-    cx.wait(B_DECAY_READY0 + (j & 3u), (j >> 2) & 1u);
-    cx.misc->decay[j & 3u].rq[lane] = rq0;
-    cx.misc->decay[j & 3u].rq[lane + 32] = rq1;
-    warp_arrive(cx.bar(B_RQ_READY0 + (j & 3u)), lane);
-    // the Q tile has been read: second arrival (after the chain's) that releases the K/Q slot in this mode
-    if (lane == 0) mbar_arrive(cx.bar(B_KQ_FREE0 + j % NKQ));
+    tma_load_3d(dst, tm, 0, row, 2 * head, bar);
+}
+// K and Q tiles of a chunk as the Gram product takes them: 2 halves x [64 rows of K, 64 rows of Q] x 128 bytes (the boxes of
+// these maps are one half wide)
+__device__ __forceinline__ void load_kq_tiles(uint32_t dst, const CUtensorMap* tm_q, const CUtensorMap* tm_k, int head, int row, uint32_t bar)
+{
+    mbar_arrive_expect_tx(bar, 32768u);
+    tma_load_3d(dst, tm_k, 0, row, 2 * head, bar);
+    tma_load_3d(dst + 16384, tm_k, 0, row, 2 * head + 1, bar);
+    tma_load_3d(dst + 8192, tm_q, 0, row, 2 * head, bar);
+    tma_load_3d(dst + 24576, tm_q, 0, row, 2 * head + 1, bar);
 }
 
-// ================================================================================================
-// warp 2: Gram MMAs.  Gram(j) needs the K/Q tiles of chunk j and the accumulator read by chunk j-1.
-// ================================================================================================
+// log-decay (log2 domain) and beta of one token from the raw input values; ok = false for rows past the end
 template <bool RAW>
-__device__ void role_mma_gram(const Ctx& cx, const TcParams& prm)
+__device__ __forceinline__ void token_inputs(float& g, float& b, bool ok)
 {
-    const int lane = threadIdx.x & 31;
-    ChunkCursor cc;
-    cc.init(&prm.p, prm.s.order);
-#pragma unroll 1
-    for (uint32_t j = 0; cc.valid; ++j, cc.advance()) {
-        const uint32_t slot = j % NKQ;
-        const uint64_t d_kq = smem_desc_sw128(cx.sb + SM_KQ + slot * KQ_SLOT, 16, 1024);   // [K;Q] rows, K-major
-        cx.wait(B_FULL_KQ0 + slot, (j / NKQ) & 1u);
-        if (j >= 1) cx.wait(B_GRAM_READ, (j - 1) & 1u);
-        tc_fence_after();
-        if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const uint64_t d = desc_add(d_kq, (ks >> 2) * 16384 + (ks & 3) * 32);
-                mma_ss(cx.tmem + TM_GRAM, d, d, ID_GRAM, ks > 0);
-            }
-            mma_commit(cx.bar(B_GRAM_DONE));
-        }
-        __syncwarp();
-        if (RAW) query_norms(cx, j, lane);
+    if (RAW) {
+        // fused input stage: alpha = sigmoid(gate), i.e. log2 alpha = -log2(1 + e^-gate);  beta = sigmoid(b)
+        g = ok ? -__log2f(1.f + ex2_approx(-kLog2e * g)) : 0.f;
+        b = ok ? __frcp_rn(1.f + ex2_approx(-kLog2e * b)) : 0.f;
+    } else {
+        g *= kLog2e;
     }
+    g = fmaxf(g, -1.0e5f);    // g = -inf (alpha = 0) keeps every difference of cumulative sums finite; 2^-1e5 is still 0
+}
+// inclusive scan over the 64 tokens of a chunk (token lane in G0, token lane + 32 in G1)
+__device__ __forceinline__ void scan64(float& G0, float& G1, int lane)
+{
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float u0 = __shfl_up_sync(0xffffffffu, G0, off), u1 = __shfl_up_sync(0xffffffffu, G1, off);
+        if (lane >= off) { G0 += u0; G1 += u1; }
+    }
+    G1 += __shfl_sync(0xffffffffu, G0, 31);
+}
+struct TokenLoad { float g0, g1, b0, b1; int nvalid; };
+__device__ __forceinline__ TokenLoad load_tokens(const Problem& p, const ChunkCursor& cc, int lane)
+{
+    TokenLoad t;
+    t.nvalid = cc.nvalid();
+    const size_t off = (size_t)(cc.row0() + lane) * p.Hv + cc.h, off1 = off + (size_t)32 * p.Hv;
+    const bool ok0 = lane < t.nvalid, ok1 = lane + 32 < t.nvalid;
+    t.g0 = ok0 ? p.g[off] : 0.f; t.g1 = ok1 ? p.g[off1] : 0.f;
+    t.b0 = ok0 ? p.beta[off] : 0.f; t.b1 = ok1 ? p.beta[off1] : 0.f;
+    return t;
 }
 
-// ================================================================================================
-// warp 1: chain MMAs
-// ================================================================================================
-__device__ void role_mma_chain(const Ctx& cx, const TcParams& prm)
+// The decay warp of either kind of CTA: walks every chunk of the cluster's sequence (the running factor c depends on all of them)
+// and hands the lane's two tokens (lane, lane + 32) to publish(j, first, cumulative decays G0, G1, betas, number of valid rows,
+// G_C, c_prev, c, rescale)
+// The loads run three chunks ahead (strided 4-byte loads from DRAM take up to 2,000 cycles, a chunk takes 1,500).
+template <bool RAW, typename F>
+__device__ __forceinline__ void walk_decays(const TcParams* prm, int lane, F publish)
 {
-    ChunkCursor cc;
-    cc.init(&prm.p, prm.s.order);
-    const bool has_init = prm.p.init_state != nullptr;
-    const uint64_t d_v = smem_desc_sw128(cx.sb + SM_V, 8192, 1024);     // V tile as M-major operand (V^T)
-    const uint64_t d_wt = smem_desc_sw128(cx.sb + SM_WT, 16, 1024);     // W^T rows [dk][t], N-major operand
+    ChunkCursor cc, cl;                                       // current chunk, next chunk to load
+    cc.init(prm);
+    cl = cc;
+    float c = 1.f;
+    TokenLoad t0 = {}, t1 = {}, t2 = {};
+    if (cl.valid) { t0 = load_tokens(prm->p, cl, lane); cl.advance(); }
+    if (cl.valid) { t1 = load_tokens(prm->p, cl, lane); cl.advance(); }
+    if (cl.valid) { t2 = load_tokens(prm->p, cl, lane); cl.advance(); }
 #pragma unroll 1
-    for (uint32_t j = 0; cc.valid; ++j, cc.advance()) {
-        const uint32_t kq = cx.sb + SM_KQ + (j % NKQ) * KQ_SLOT;
-        const uint64_t d_q = smem_desc_sw128(kq + 8192, 16, 1024);      // Q rows, K-major
-        const uint64_t d_kn = smem_desc_sw128(kq, 16384, 1024);         // K tile as N-major operand
-        const uint64_t d_p = smem_desc_sw128(cx.sb + SM_P + (j % 3u) * 8192, 16, 1024);
-        const uint64_t d_tp = smem_desc_sw128(cx.sb + SM_TP + (j % 3u) * 8192, 16, 1024);
-        const bool has_state = !cc.first() || has_init;     // a zero start state is skipped, not multiplied
-        cx.wait(B_TP_READY0 + j % 3u, (j / 3u) & 1u);
-        cx.wait(B_FULL_V, j & 1u);
-        tc_fence_after();
-        // U^T = V^T T'^T -> ACC1 (free: the Delta operands of chunk j-1 in it were read by MMAs issued before
-        // these).  Issued ahead of the wait for the W^T operand, which is the last piece of the set to arrive.
-        if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ss(cx.tmem + TM_ACC1, desc_add(d_v, ks * 2048), desc_add(d_tp, ks * 32), ID_WU, ks > 0);
-            mma_commit(cx.bar(B_U_DONE));
-            mma_commit(cx.bar(B_TP_FREE0 + j % 3u));
-        }
-        __syncwarp();
-        cx.wait(B_PRE_DONE0 + (j & 1u), (j >> 1) & 1u);
-        // start state of this chunk: the previous chunk's state converted, or, at a chain start, the previous chain's
-        // state read out and this chain's start state (if any) written
-        cx.wait(B_SBF_READY, j & 1u);
-        tc_fence_after();
-        if (has_state && elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                mma_ts(cx.tmem + TM_ACC1, cx.tmem + TM_SBF + ks * 8, desc_add(d_wt, ks * 2048), ID_SW, 1u);
-        }
-        __syncwarp();
-        // Delta^T is complete: its epilogue starts now
-        if (elect_one()) mma_commit(cx.bar(B_MMA1_DONE));
-        __syncwarp();
-        // The state update only needs the Delta epilogue: it goes first, so that the chain never queues behind the
-        // output accumulators.
-        cx.wait(B_D_READY, j & 1u);
-        tc_fence_after();
-        if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ts(cx.tmem + TM_S32, cx.tmem + TM_DPBF + ks * 16, desc_add(d_kn, ks * 2048), ID_DK,
-                       (has_state || ks > 0) ? 1u : 0u);
-            mma_commit(cx.bar(B_STATE_DONE));
-        }
-        __syncwarp();
-        // The two output products need the accumulators back from the output epilogue of chunk j-1.  S0 Q^T is the last
-        // reader of the bf16 state: the state epilogue waits for it (SQ_DONE) before it overwrites that copy.
-        if (j >= 1) cx.wait(B_ACC23_FREE, (j - 1) & 1u);
-        tc_fence_after();
-        if (elect_one()) {
-            if (has_state) {
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ts(cx.tmem + TM_ACC2, cx.tmem + TM_SBF + ks * 8,
-                           desc_add(d_q, (ks >> 2) * 16384 + (ks & 3) * 32), ID_SQ, ks > 0);
-            }
-            mma_commit(cx.bar(B_SQ_DONE));
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ts(cx.tmem + TM_ACC3, cx.tmem + TM_DBF + ks * 16, desc_add(d_p, ks * 32), ID_DP, ks > 0);
-            mma_commit(cx.bar(B_MMA3_DONE));
-            mma_commit(cx.bar(B_P_FREE0 + j % 3u));
-            mma_commit(cx.bar(B_KQ_FREE0 + j % NKQ));           // K and Q of this chunk have been read
-        }
-        __syncwarp();
-    }
-}
-
-// ================================================================================================
-// warp 3: decay warp.  Runs up to three chunks ahead of the consumers (ring of four slots), which hides the
-// DRAM latency of the strided g / beta loads.
-// ================================================================================================
-template <bool RAW>
-__device__ void role_decay(const Ctx& cx, const TcParams& prm)
-{
-    const Problem& p = prm.p;
-    const int lane = threadIdx.x & 31;
-    ChunkCursor cc;
-    cc.init(&p, prm.s.order);
-    float c = 1.f;                                            // running scale of the stored state (see Decay)
-#pragma unroll 1
-    for (uint32_t j = 0; cc.valid; ++j, cc.advance()) {
-        const int row0 = cc.row0(), nvalid = cc.nvalid(), h = cc.h;
+    for (uint32_t j = 0; cc.valid; ++j) {
         const bool first = cc.first();
-        const bool ok0 = lane < nvalid, ok1 = lane + 32 < nvalid;
-        float g0 = ok0 ? p.g[(size_t)(row0 + lane) * p.Hv + h] : 0.f;
-        float g1 = ok1 ? p.g[(size_t)(row0 + lane + 32) * p.Hv + h] : 0.f;
-        float b0 = ok0 ? p.beta[(size_t)(row0 + lane) * p.Hv + h] : 0.f;
-        float b1 = ok1 ? p.beta[(size_t)(row0 + lane + 32) * p.Hv + h] : 0.f;
-        if (RAW) {
-            // fused input stage: alpha = sigmoid(gate), i.e. log alpha = -log(1 + e^-gate) (the gate of a padded row is 0,
-            // its beta is set to 0 below);  beta = sigmoid(b)
-            g0 = -0.6931471805599453f * __log2f(1.f + ex2_approx(-kLog2e * g0));
-            g1 = -0.6931471805599453f * __log2f(1.f + ex2_approx(-kLog2e * g1));
-            b0 = ok0 ? __frcp_rn(1.f + ex2_approx(-kLog2e * b0)) : 0.f;
-            b1 = ok1 ? __frcp_rn(1.f + ex2_approx(-kLog2e * b1)) : 0.f;
-            g0 = ok0 ? g0 : 0.f; g1 = ok1 ? g1 : 0.f;
-        }
-        // clamped so that g = -inf (alpha = 0) keeps every difference of cumulative sums finite; 2^-1e5 is still 0
-        float G0 = fmaxf(g0 * kLog2e, -1.0e5f), G1 = fmaxf(g1 * kLog2e, -1.0e5f);
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float u0 = __shfl_up_sync(0xffffffffu, G0, off), u1 = __shfl_up_sync(0xffffffffu, G1, off);
-            if (lane >= off) { G0 += u0; G1 += u1; }
-        }
-        G1 += __shfl_sync(0xffffffffu, G0, 31);
+        const int nvalid = t0.nvalid;
+        float G0 = t0.g0, G1 = t0.g1, b0 = t0.b0, b1 = t0.b1;
+        cc.advance();
+        t0 = t1; t1 = t2;
+        if (cl.valid) { t2 = load_tokens(prm->p, cl, lane); cl.advance(); }
+        token_inputs<RAW>(G0, b0, lane < nvalid);
+        token_inputs<RAW>(G1, b1, lane + 32 < nvalid);
+        scan64(G0, G1, lane);
         const float GC = __shfl_sync(0xffffffffu, G1, 31);
         const float cprev = first ? 1.f : c;
         const float eGC = ex2_approx(GC);
         const bool rescale = first || !(cprev * eGC >= 9.094947e-13f);       // 2^-40; also catches NaN
         c = rescale ? 1.f : cprev * eGC;
-        const float cinv = rescale ? 1.f : __frcp_rn(c);
-        const float e0 = ex2_approx(G0) * cprev, e1 = ex2_approx(G1) * cprev;
-        // the slot was last read by the chain group's output epilogue of chunk j - 4
-        if (j >= 4) cx.wait(B_DECAY_FREE0 + (j & 3u), ((j >> 2) - 1u) & 1u);
-        Decay& dc = cx.misc->decay[j & 3u];
+        publish(j, G0, G1, b0, b1, nvalid, GC, eGC, cprev, c, rescale);
+    }
+}
+
+// ================================================================================================
+// Prep CTA
+// ================================================================================================
+// warp 0: K/Q tiles of the CTA's chunks, one buffer per team, refilled as soon as the team's W~^T product has read it
+__device__ void prep_producer(const Ctx& cx, const TcParams* prm, uint32_t rank, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
+{
+    const int R = (int)prm->csize - 1;
+    ChunkCursor cc;
+    cc.init(prm);
+    cc.advance((int)rank - 1);
+#pragma unroll 1
+    for (uint32_t i = 0; cc.valid && !cx.stop(); ++i, cc.advance(R)) {
+        const uint32_t team = i % NT, use = i / NT;
+        if (use >= 1) cx.wait(PB_W0 + (int)team, (use - 1) & 1u);
+        if ((int32_t)(i * R + rank - 1) != prm->skip_kq_load) {           // testing aid: the skipped tile never arrives
+            if (elect_one()) load_kq_tiles(cx.sb + team * P_TEAM, tm_q, tm_k, cc.hq, cc.row0(), cx.bar(PB_KQ_FULL0 + team));
+            __syncwarp();
+        }
+    }
+}
+
+// warps 16-18: finished operands into the cluster's ring, one warp per team (a store takes 1-2 us until it is complete)
+template <bool RAW>
+__device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, uint32_t team)
+{
+    const uint32_t R = prm->csize - 1, own = prm->ring / R;            // ring slots of this CTA (kRingSlots / 3 or kRingSlotsPair)
+    ChunkCursor cc;
+    cc.init(prm);
+    cc.advance((int)(rank - 1 + team * R));
+    uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
+#pragma unroll 1
+    for (uint32_t i = team; cc.valid; i += NT, cc.advance((int)(R * NT))) {
+        const uint32_t j = rank - 1 + i * R, slot = j % prm->ring;
+        cx.wait(PB_OPS0 + (int)team, (i / NT) & 1u);
+        if (i >= own) cx.wait_cluster(PB_CREDIT0 + (int)(i % own), (i / own - 1u) & 1u);
+        if (elect_one()) {
+            uint8_t* dst = ring + (size_t)slot * kRingSlotBytes;
+            bulk_store(dst, cx.sb + team * P_TEAM + P_OPS, OPS_BYTES);
+            if (RAW) bulk_store(dst + OPS_BYTES, smem_u32(cx.misc->p.decay[i & 3u].norms), NORM_BYTES);
+            bulk_commit();
+            bulk_wait();                                               // in L2, where the bulk load finds it; source buffers free
+            mbar_arrive_remote_release(map_to_rank(cx.bar(CB_RING0 + (int)slot), 0u));
+            mbar_arrive(cx.bar(PB_SENT0 + (int)team));
+            mbar_arrive(cx.bar(PB_DECAY_FREE0 + (int)(i & 3u)));
+        }
+        __syncwarp();
+    }
+}
+
+// warp 2: factors of the CTA's chunks
+template <bool RAW>
+__device__ void prep_decay(const Ctx& cx, const TcParams* prm, uint32_t rank, int lane)
+{
+    const uint32_t R = prm->csize - 1;
+    uint32_t i = 0;
+    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float, float, float cprev, float, bool) {
+        if (j % R != rank - 1) return;
+        if (i >= 4) cx.wait(PB_DECAY_FREE0 + (int)(i & 3u), ((i >> 2) - 1u) & 1u);
+        PrepDecay& dc = cx.misc->p.decay[i & 3u];
+        const float G31 = __shfl_sync(0xffffffffu, G0, 31);
         // rows past the end of the request (whose k, q, v may be anything finite) get a hugely negative cumulative
         // decay: every Gam[t, .] of such a row underflows to zero, so its A^ and P rows vanish
-        dc.G2[lane] = ok0 ? G0 : -1.0e30f; dc.G2[lane + 32] = ok1 ? G1 : -1.0e30f;
+        dc.G2[lane] = lane < nvalid ? G0 : -1.0e30f; dc.G2[lane + 32] = lane + 32 < nvalid ? G1 : -1.0e30f;
         dc.beta[lane] = b0; dc.beta[lane + 32] = b1;
-        dc.eG[lane] = e0; dc.eG[lane + 32] = e1;
-        dc.eGk[lane] = e0; dc.eGk[lane + 32] = e1;
-        dc.bRest[lane] = b0 * (ex2_approx(GC - G0) * cinv); dc.bRest[lane + 32] = b1 * (ex2_approx(GC - G1) * cinv);
-        const float G31 = __shfl_sync(0xffffffffu, G0, 31);
+        dc.eG[lane] = ex2_approx(G0) * cprev; dc.eG[lane + 32] = ex2_approx(G1) * cprev;
         dc.colfb[lane] = ex2_approx(G31 - G0) * b0;
-        if (lane == 0) { dc.wb = cprev * eGC; dc.G2mid = G31; dc.cfin = c; dc.rescale = rescale ? 1 : 0; }
-        warp_arrive(cx.bar(B_DECAY_READY0 + (j & 3u)), lane);
-    }
+        if (lane == 0) dc.G2mid = G31;
+        warp_arrive(cx.bar(PB_DECAY_READY0 + (int)(i & 3u)), lane);
+        ++i;
+    });
 }
 
-// Number of 64-row chunks this CTA processes over all of its chains.
-__device__ __noinline__ uint32_t count_chunks(const TcParams& prm)
+// One team of four warps (w = 0..3, TMEM lane window w): chunk after chunk from the K/Q tiles to the operands W~^T, T', P.
+template <bool RAW, bool CL>
+__device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uint32_t team, int w, int lane)
 {
+    const int R = CL ? (int)prm->csize - 1 : 1;
+    const uint32_t NTEAM = CL ? NT : 2u;
+    const uint32_t o_w = CL ? team * P_TEAM + P_OPS + OPS_W : F_W + team * 16384;
+    const uint32_t o_tp = CL ? team * P_TEAM + P_OPS + OPS_TP : F_TP + team * 8192;
+    const uint32_t o_tpp = CL ? team * P_TEAM + P_TPP : o_w;
+    uint8_t* const TP = cx.sm + o_tp;                         // A^, inverted in place
+    uint8_t* const TPP = cx.sm + o_tpp;                       // T'' = T' diag(e^G)
+    const uint32_t xs = cx.sb + o_tp;
+    const uint32_t tm_gram = cx.tmem + (CL ? team * TM_TEAM + TM_GRAM : TM_F_TEAM + team * 64);
+    const uint32_t tm_wacc = cx.tmem + (CL ? team * TM_TEAM + TM_WACC : TM_F_TEAM + team * 64);
+    const uint32_t lane_win = (uint32_t)(w * 32) << 16;
+    auto team_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); };
+    const int t = ((w & 1) << 5) + lane;                      // this thread's row of the Gram tile
+    const bool isA = w < 2;                                   // windows 0, 1 hold K K^T rows, 2, 3 hold Q K^T rows
+    const bool lower_rows = (w & 1) != 0;                     // rows 32-63
+
     ChunkCursor cc;
-    cc.init(&prm.p, prm.s.order);
-    uint32_t n = 0;
-    while (cc.valid) { n += (uint32_t)cc.nchunks; cc.next_chain(); }
-    return n;
-}
-
-// Fused input stage, group G1's part (inlined into the group's fused-stage instance only).  The squared norms of the chunk's
-// key rows are the diagonal of K K^T, which sits in the Gram accumulator: one warp per lane window of the K rows reads
-// them, the group meets, 64 of its threads fold 1 / |k_s| into the per-token factors that multiply key s wherever it
-// enters (columns of A^ and P, columns of T'', the state update), the group meets again.  Returns what a row of A^
-// adds to its row decay: log2(1 / |k_t|) (0 for rows of P: the query norms multiply the finished output rows instead).
-__device__ __forceinline__ float key_norms(const Ctx& cx, Misc* misc, uint32_t c, uint32_t tl, int wtid, int t, bool isA, int hf)
-{
-    Decay& dc = misc->decay[c & 3u];
-    if (isA && hf == 0) {
-        // the diagonal entry of this lane's row lies in the first (lanes 0-15) or second (lanes 16-31) 16-column block of
-        // the warp's rows (the address is the same for all lanes): both are read, then a select tree on the lane bits
-        uint32_t lo[16], hi[16];
-        tmem_ld16(tl + TM_GRAM + (uint32_t)(t & 32), lo);
-        tmem_ld16(tl + TM_GRAM + (uint32_t)(t & 32) + 16u, hi);
-        tmem_ld_wait();
-        uint32_t x8[8], x4[4];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const uint32_t a = (t & 8) ? lo[e + 8] : lo[e], b = (t & 8) ? hi[e + 8] : hi[e];
-            x8[e] = (t & 16) ? b : a;
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) x4[e] = (t & 4) ? x8[e + 4] : x8[e];
-        const uint32_t y0 = (t & 2) ? x4[2] : x4[0], y1 = (t & 2) ? x4[3] : x4[1];
-        const float dg = __uint_as_float((t & 1) ? y1 : y0);
-        misc->rk[t] = rsqrtf(dg + kNormEps);
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (wtid < 64) {
-        const float r = misc->rk[wtid];
-        dc.beta[wtid] *= r; dc.bRest[wtid] *= r; dc.eGk[wtid] *= r;
-        if (wtid < 32) dc.colfb[wtid] *= r;
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    return isA ? __log2f(misc->rk[t]) : 0.f;
-}
-
-// ================================================================================================
-// warps 4-11: group G1.  Per iteration k: Gram post-processing of chunk k+1 (writes A^ for the solve and the
-// operand P), then the W^T epilogue of chunk k.
-// ================================================================================================
-template <bool RAW>
-__device__ void role_g1(const Ctx& cx, const TcParams& prm, int wtid)
-{
-    const int lane = wtid & 31, pw = wtid >> 5;          // pw = 0..7
-    const int w4 = pw & 3, hf = pw >> 2;                 // TMEM lane window, column half
-    const uint32_t tl = cx.tmem + ((uint32_t)(w4 * 32) << 16);
-    Misc* misc = cx.misc;
-    const uint32_t J = count_chunks(prm);
-
-    // ---- Gram tile of chunk c -> A (bf16 scratch for the solve) and P (bf16 operand), 16 columns at a time
-    auto post = [&](uint32_t c) {
-        const Decay& dc = misc->decay[c & 3u];
-        cx.wait(B_DECAY_READY0 + (c & 3u), (c >> 2) & 1u);       // decay factors of this chunk are published
-        // this thread's row of the Gram tile: lane windows 0,1 hold K K^T rows, 2,3 hold Q K^T rows
-        const int t = ((w4 & 1) << 5) + lane;
-        const bool isA = w4 < 2;
-        float G2t = dc.G2[t];
-        // the solve works on A^ = strict_lower(Gam (K K^T)) diag(beta) (beta on the columns): its inverse P^ gives
-        // T' = diag(beta) P^ and T'' = diag(beta) P^ diag(e^G), and the common row factor beta moves into the
-        // Delta epilogue, so that P^ itself is one MMA operand and its column-scaled copy the other
-        // (P carries beta on its columns as well, so that the output product takes Delta~ as it is)
-        const float* __restrict__ colscale = dc.beta;
-        const float* __restrict__ colfac = dc.colfb;
-        const int t_lim = isA ? t : t + 1;                      // keep columns s < t_lim
-        cx.wait(B_GRAM_DONE, c & 1u);
-        tc_fence_after();
-        if (RAW) G2t += key_norms(cx, misc, c, tl, wtid, t, isA, hf);
-        // buffers: P and T' of chunk c were last read by the MMAs of chunk c-3
-        if (c >= 3) {
-            cx.wait(B_P_FREE0 + c % 3u, ((c / 3u) - 1u) & 1u);
-            cx.wait(B_TP_FREE0 + c % 3u, ((c / 3u) - 1u) & 1u);
-        }
-        // this thread's row of the operand tile it writes: A^ into T' (where the solve inverts it in place), or P
-        uint8_t* prow = cx.sm + (isA ? SM_TP : SM_P) + (c % 3u) * 8192 + t * 128;
-        // column blocks are dealt so that each warp of a lane window gets one block that touches the
-        // diagonal and one that does not: half 0 -> blocks {0, 2}, half 1 -> blocks {1, 3}
-        const bool lower_rows = (w4 & 1) != 0;                  // rows 32-63
-        const float rowf = lower_rows ? ex2_approx(G2t - dc.G2mid) : 0.f;
+    cc.init(prm);
+    cc.advance((CL ? (int)rank - 1 : 0) + R * (int)team);
 #pragma unroll 1
-        for (int g = 0; g < 2; ++g) {
-            const int cb = hf + 2 * g, c0 = 16 * cb;
-            if (c0 > ((w4 & 1) << 5) + 31) {                    // block entirely above the diagonal (warp-uniform)
-                continue;                                       // (zero since the start of the kernel)
-            }
-            uint32_t acc[16];
-            tmem_ld16(tl + TM_GRAM + c0, acc);
-            tmem_ld_wait();
-            float vals[16];
-            if (lower_rows && cb < 2) {
-                // every column precedes every row of this warp: Gam = rowf * colf, no mask, no exp
-#pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    const float4 cf = *reinterpret_cast<const float4*>(&colfac[c0 + 4 * i4]);
-                    vals[4 * i4 + 0] = (rowf * cf.x) * __uint_as_float(acc[4 * i4 + 0]);
-                    vals[4 * i4 + 1] = (rowf * cf.y) * __uint_as_float(acc[4 * i4 + 1]);
-                    vals[4 * i4 + 2] = (rowf * cf.z) * __uint_as_float(acc[4 * i4 + 2]);
-                    vals[4 * i4 + 3] = (rowf * cf.w) * __uint_as_float(acc[4 * i4 + 3]);
-                }
-            } else {
-#pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    const float4 gs = *reinterpret_cast<const float4*>(&dc.G2[c0 + 4 * i4]);
-                    const float4 cs = *reinterpret_cast<const float4*>(&colscale[c0 + 4 * i4]);
-                    const float gss[4] = {gs.x, gs.y, gs.z, gs.w}, css[4] = {cs.x, cs.y, cs.z, cs.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int i = 4 * i4 + e;
-                        // masked entries may overflow to inf / NaN before the select discards them
-                        const float f = ex2_approx(G2t - gss[e]) * css[e];
-                        vals[i] = (c0 + i < t_lim) ? f * __uint_as_float(acc[i]) : 0.f;
-                    }
-                }
-            }
-            uint4 u[2];
-#pragma unroll
-            for (int c8 = 0; c8 < 2; ++c8) {
-                u[c8].x = pack_bf16x2(vals[c8 * 8 + 0], vals[c8 * 8 + 1]);
-                u[c8].y = pack_bf16x2(vals[c8 * 8 + 2], vals[c8 * 8 + 3]);
-                u[c8].z = pack_bf16x2(vals[c8 * 8 + 4], vals[c8 * 8 + 5]);
-                u[c8].w = pack_bf16x2(vals[c8 * 8 + 6], vals[c8 * 8 + 7]);
-            }
-            *reinterpret_cast<uint4*>(prow + (((2 * cb) ^ (t & 7)) << 4)) = u[0];
-            *reinterpret_cast<uint4*>(prow + (((2 * cb + 1) ^ (t & 7)) << 4)) = u[1];
-        }
-        tc_fence_before();
-        warp_arrive(cx.bar(B_GRAM_READ), lane);                 // the accumulator may take the next Gram tile
-        fence_proxy_async_smem();                               // P is an MMA operand
-        // A^ of chunk c is complete: the solve may start.  (Barriers that follow a T' buffer are kept per buffer: the
-        // buffer's reuse then bounds how far an arrival can run ahead of a waiter, which a parity wait needs.)
-        warp_arrive(cx.bar(B_A_READY0 + c % 3u), lane);
-    };
-
-    // ---- W^T epilogue of chunk c: bf16 rows [dk][t] as the N-major operand of the S0 W^T MMA; completes the
-    // operand set of chunk c (each warp converts 32 columns of its lane window; TMEM lane = key index)
-    auto w_epilogue = [&](uint32_t c) {
-        cx.wait(B_W_DONE0 + (c & 1u), (c >> 1) & 1u);
-        tc_fence_after();
-        // W^T is single-buffered: the S0 W^T MMA of chunk c-1 must have read it
-        if (c >= 1) cx.wait(B_MMA1_DONE, (c - 1) & 1u);
-        const int drow = w4 * 32 + lane;
-        uint8_t* wrow = cx.sm + SM_WT + drow * 128;
-        const int c0 = 32 * hf;
-        uint32_t acc[32];
-        tmem_ld32(tl + TM_WACC + c0, acc);
-        tmem_ld_wait();
-#pragma unroll
-        for (int c8 = 0; c8 < 4; ++c8) {
-            uint4 u;
-            u.x = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 0]), __uint_as_float(acc[c8 * 8 + 1]));
-            u.y = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 2]), __uint_as_float(acc[c8 * 8 + 3]));
-            u.z = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 4]), __uint_as_float(acc[c8 * 8 + 5]));
-            u.w = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 6]), __uint_as_float(acc[c8 * 8 + 7]));
-            *reinterpret_cast<uint4*>(wrow + ((((c0 >> 3) + c8) ^ (drow & 7)) << 4)) = u;
-        }
-        tc_fence_before();
-        warp_arrive(cx.bar(B_WACC_READ), lane);                 // the accumulator may take the next W^T tile
-        fence_proxy_async_smem();
-        warp_arrive(cx.bar(B_PRE_DONE0 + (c & 1u)), lane);
-    };
-
-    // iteration i: Gram post-processing of chunk i, then the W^T epilogue of chunk i-1, whose solve and W^T MMA
-    // ran meanwhile
-#pragma unroll 1
-    for (uint32_t i = 0; i <= J; ++i) {
-        if (i < J) post(i);
-        if (i >= 1) w_epilogue(i - 1);
-    }
-}
-
-// ================================================================================================
-// warps 20-23: group G2 (two teams of two warps on alternate chunks), P^ = (I + A^)^-1 of chunk k.  Each warp of a
-// team inverts one 32 x 32 diagonal half without any cross-warp barrier:
-//   level 0  : its four 8 x 8 diagonal blocks by forward substitution in fp32
-//   level 0.5: 8 -> 16 merges, level 1: the 16 -> 32 merge X[hi][lo] = -X[hi][hi] (A[hi][lo] X[lo][lo]),
-//   level 2  : X[32:64][0:32] = -X22 (A21 X11), two 16 x 16 tiles per warp,
-// the merges on mma.sync with ldmatrix-fed bf16 fragments.  The post-processing has left A^ in the chunk's T' operand
-// buffer (MMA operand layout, which ldmatrix reads just as well), and the inverse replaces it block by block: every
-// block is read by the warp that overwrites it, before it does.  A last pass writes the copy with columns scaled by
-// e^G into the T'' operand buffer.  What lies above the 16 x 16 diagonal blocks of both is zero from the start of
-// the kernel.
-// ================================================================================================
-// stores sign * c of a 16 x 16 accumulator tile (two 8-column halves) at rows r0.., columns n0.. of an operand tile
-__device__ __forceinline__ void tile16_store_sw(const float (&c)[2][4], float sign, uint8_t* T, int r0, int n0, int lane)
-{
-    const int g = lane >> 2, t4 = lane & 3;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        *reinterpret_cast<uint32_t*>(T + sw_off(r0 + g, n0 + 8 * h + 2 * t4)) = pack_bf16x2(sign * c[h][0], sign * c[h][1]);
-        *reinterpret_cast<uint32_t*>(T + sw_off(r0 + g + 8, n0 + 8 * h + 2 * t4)) = pack_bf16x2(sign * c[h][2], sign * c[h][3]);
-    }
-}
-
-__device__ void role_g2(const Ctx& cx, const TcParams& prm, int wtid, int team)
-{
-    const int lane = wtid & 31, pw = wtid >> 5;          // pw = 0, 1
-    uint8_t* MH = cx.sm + SM_MH + team * MH_BYTES;
-    const uint32_t mh = cx.sb + SM_MH + team * MH_BYTES;
-    const uint32_t J = count_chunks(prm);
-    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(3 + team) : "memory"); };
-    // The 16-byte pieces of T'' on and below the diagonal (row t has t / 8 + 1 of them, 288 in all) are dealt evenly
-    // to the team's 64 threads, at most 5 each, instead of one row per thread (whose longest rows have 8): ten bits
-    // per piece (row, piece index, valid), fixed for the whole kernel.
-    unsigned long long tpp_items = 0ull;
-    for (int it = 0; it < 5; ++it) {
-        const int i = it * 64 + wtid;
-        if (i < 288) {
-            int g = 0;
-            while (4 * (g + 1) * (g + 2) <= i) ++g;              // rows 8 g .. 8 g + 7 own pieces [4 g (g + 1), 4 (g + 1)(g + 2))
-            const int r = i - 4 * g * (g + 1);
-            const int t = 8 * g + r / (g + 1), ch = r % (g + 1);
-            tpp_items |= (unsigned long long)(512 | (ch << 6) | t) << (10 * it);
-        }
-    }
-    // team 0 takes the even chunks, team 1 the odd ones: the A, T' and T'' buffers alternate the same way
-#pragma unroll 1
-    for (uint32_t k = (uint32_t)team; k < J; k += 2) {
-        cx.wait(B_A_READY0 + k % 3u, (k / 3u) & 1u);
-        const Decay& dc = cx.misc->decay[k & 3u];
-        uint8_t* TP = cx.sm + SM_TP + (k % 3u) * 8192;           // holds A^; becomes the inverse
-        const uint32_t xs = cx.sb + SM_TP + (k % 3u) * 8192;
-        {
-            const int bb = 4 * pw + (lane >> 3), b = 8 * bb, jj = lane & 7;
-            uint4 rows[7];
-#pragma unroll
-            for (int r = 1; r < 8; ++r) rows[r - 1] = *reinterpret_cast<const uint4*>(TP + sw_off(b + r, b));
-            __syncwarp();                                       // every row is in registers before any is overwritten
-            float x[8];
-#pragma unroll
-            for (int r = 0; r < 8; ++r) x[r] = (r == jj) ? 1.f : 0.f;
-#pragma unroll
-            for (int r = 1; r < 8; ++r) {
-                const uint32_t wds[4] = {rows[r - 1].x, rows[r - 1].y, rows[r - 1].z, rows[r - 1].w};
-                float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-                for (int s2 = 0; s2 < r; ++s2) {
-                    const float a = (s2 & 1) ? bf_hi(wds[s2 >> 1]) : bf_lo(wds[s2 >> 1]);
-                    if (s2 & 1) acc1 = fmaf(a, x[s2], acc1); else acc0 = fmaf(a, x[s2], acc0);
-                }
-                x[r] = (r > jj) ? -(acc0 + acc1) : x[r];
-            }
-            // this thread's column of the diagonal block, zeros above the diagonal included
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-                *reinterpret_cast<__nv_bfloat16*>(TP + sw_off(b + r, b + jj)) = __float2bfloat16_rn(x[r]);
-        }
-        __syncwarp();
-        {
-            const int i = (lane >> 3) & 1, rr = lane & 7, b16 = 32 * pw + 16 * i;
-            const int g = lane >> 2, t4 = lane & 3;
-            uint32_t a[2], bx[2];
-            ldm_x2(a, xs + sw_off(b16 + 8 + rr, b16));                            // A21 of both blocks
-            ldm_x2_trans(bx, xs + sw_off(b16 + rr, b16));                         // X11 of both blocks
-            float m0[4] = {0.f, 0.f, 0.f, 0.f}, m1[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_8x8(m0, a[0], bx[0]);
-            mma_8x8(m1, a[1], bx[1]);
-            *reinterpret_cast<uint32_t*>(MH + ((16 * pw + g) * LDM + 2 * t4) * 2) = pack_bf16x2(m0[0], m0[1]);
-            *reinterpret_cast<uint32_t*>(MH + ((16 * pw + 8 + g) * LDM + 2 * t4) * 2) = pack_bf16x2(m1[0], m1[1]);
-            __syncwarp();
-            uint32_t a2[2], bm[2];
-            ldm_x2(a2, xs + sw_off(b16 + 8 + rr, b16 + 8));                       // X22 of both blocks
-            ldm_x2_trans(bm, mh + ((16 * pw + 8 * i + rr) * LDM) * 2);           // M of both blocks
-            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_8x8(d0, a2[0], bm[0]);
-            mma_8x8(d1, a2[1], bm[1]);
-            const int c0b = 32 * pw, c1b = 32 * pw + 16;
-            *reinterpret_cast<uint32_t*>(TP + sw_off(c0b + 8 + g, c0b + 2 * t4)) = pack_bf16x2(-d0[0], -d0[1]);
-            *reinterpret_cast<uint32_t*>(TP + sw_off(c1b + 8 + g, c1b + 2 * t4)) = pack_bf16x2(-d1[0], -d1[1]);
-        }
-        __syncwarp();
-        {
-            const int lo = 32 * pw, hi = 32 * pw + 16;
-            float m[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-            tile16_mma_at(m, tile_addr_sw(xs, hi, lo, lane), tile_addr_sw(xs, lo, lo, lane));          // A[hi][lo] X[lo][lo]
-            tile16_store(m, 1.f, MH, LDM, 16 * pw, 0, lane);
-            __syncwarp();
-            float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-            tile16_mma_at(d, tile_addr_sw(xs, hi, hi, lane), tile_addr(mh, LDM, 16 * pw, 0, lane));   // X[hi][hi] M
-            tile16_store_sw(d, -1.f, TP, hi, lo, lane);
-        }
-        pair_sync();
-        // level 2: warp pw owns block row mt = pw of X[32:64][0:32] (it alone reads and then overwrites those rows);
-        // its two 16 x 16 tiles are independent, so their ldmatrix / mma chains are written side by side
-        {
-            const int mt = pw;
-            float m0[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, m1[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-            // X11 is lower triangular: block column nt starts at block row nt
-            tile16_mma_at(m0, tile_addr_sw(xs, 32 + 16 * mt, 0, lane), tile_addr_sw(xs, 0, 0, lane));
-            tile16_mma_at(m1, tile_addr_sw(xs, 32 + 16 * mt, 16, lane), tile_addr_sw(xs, 16, 16, lane));
-            tile16_mma_at(m0, tile_addr_sw(xs, 32 + 16 * mt, 16, lane), tile_addr_sw(xs, 16, 0, lane));
-            tile16_store(m0, 1.f, MH, LDM, 16 * mt, 0, lane);
-            tile16_store(m1, 1.f, MH, LDM, 16 * mt, 16, lane);
-            pair_sync();
-            float d0[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, d1[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-            // X22 is lower triangular: block row mt ends at block column mt
-            tile16_mma_at(d0, tile_addr_sw(xs, 32 + 16 * mt, 32, lane), tile_addr(mh, LDM, 0, 0, lane));
-            tile16_mma_at(d1, tile_addr_sw(xs, 32 + 16 * mt, 32, lane), tile_addr(mh, LDM, 0, 16, lane));
-            if (mt == 1) {
-                tile16_mma_at(d0, tile_addr_sw(xs, 48, 48, lane), tile_addr(mh, LDM, 16, 0, lane));
-                tile16_mma_at(d1, tile_addr_sw(xs, 48, 48, lane), tile_addr(mh, LDM, 16, 16, lane));
-            }
-            tile16_store_sw(d0, -1.f, TP, 32 + 16 * mt, 0, lane);
-            tile16_store_sw(d1, -1.f, TP, 32 + 16 * mt, 16, lane);
-        }
-        fence_proxy_async_smem();                               // T' is an MMA operand
-        warp_arrive(cx.bar(B_TP_READY0 + k % 3u), lane);
-        pair_sync();                                            // the whole inverse is in place
-        // T'' = T' diag(e^G): this thread's share of the 16-byte pieces up to the diagonal.  The one T'' buffer was last read by
-        // the W^T MMA of chunk k-1 (the other team's; consecutive phases of its barrier are observed chunk after chunk).
-        if (k >= 1) cx.wait(B_W_DONE0 + ((k - 1) & 1u), ((k - 1) >> 1) & 1u);
-        {
-#pragma unroll 1
-            for (int it = 0; it < 5; ++it) {
-                const uint32_t code = (uint32_t)(tpp_items >> (10 * it)) & 1023u;
-                if (code & 512u) {
-                    const int t = (int)(code & 63u), ch = (int)((code >> 6) & 7u);
-                    const uint32_t off = (uint32_t)t * 128u + (uint32_t)((ch ^ (t & 7)) << 4);
-                    const uint4 v = *reinterpret_cast<const uint4*>(TP + off);
-                    const float4 e0 = *reinterpret_cast<const float4*>(&dc.eGk[8 * ch]);
-                    const float4 e1 = *reinterpret_cast<const float4*>(&dc.eGk[8 * ch + 4]);
-                    uint4 o;
-                    o.x = mul_bf16x2(v.x, pack_bf16x2(e0.x, e0.y)); o.y = mul_bf16x2(v.y, pack_bf16x2(e0.z, e0.w));
-                    o.z = mul_bf16x2(v.z, pack_bf16x2(e1.x, e1.y)); o.w = mul_bf16x2(v.w, pack_bf16x2(e1.z, e1.w));
-                    *reinterpret_cast<uint4*>(cx.sm + SM_TPP + off) = o;
-                }
-            }
-        }
-        fence_proxy_async_smem();                               // T'' is an MMA operand
-        pair_sync();                                            // both warps' rows of T'' are in place
-        // W~^T = K^T T''^T, issued from here: needs the accumulator read by the W^T epilogue of chunk k-1
-        if (pw == 0) {
-            const uint64_t d_kt = smem_desc_sw128(cx.sb + SM_KQ + (k % NKQ) * KQ_SLOT, 16384, 1024);   // K^T, M-major
-            const uint64_t d_tpp = smem_desc_sw128(cx.sb + SM_TPP, 16, 1024);
-            if (k >= 1) cx.wait(B_WACC_READ, (k - 1) & 1u);
+    for (uint32_t k = 0; cc.valid; ++k, cc.advance(R * (int)NTEAM)) {
+        const uint32_t par = k & 1u, i = k * NTEAM + team;        // position in the CTA's chunk sequence
+        const uint32_t o_kq = CL ? team * P_TEAM : F_KQ + (i & 3u) * 32768, kq = cx.sb + o_kq;
+        const uint32_t o_p = CL ? team * P_TEAM + P_OPS + OPS_P : F_P + (i % 3u) * 8192;
+        const int b_kq = CL ? PB_KQ_FULL0 + (int)team : FB_KQ_FULL0 + (int)(i & 3u);
+        const uint32_t kq_par = CL ? par : (i >> 2) & 1u;
+        auto& dc = prep_rec<CL>(cx.misc, i & 3u);
+        if (w == 0) {
+            // ---- Gram = [K;Q] K^T
+            cx.wait(b_kq, kq_par);
             tc_fence_after();
             if (elect_one()) {
+                const uint64_t d_kq = smem_desc_sw128(kq, 16, 1024);
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_ss(cx.tmem + TM_WACC, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * 32), ID_WU, ks > 0);
-                mma_commit(cx.bar(B_W_DONE0 + (k & 1u)));
+                for (int ks = 0; ks < 8; ++ks) {
+                    const uint64_t d = desc_add(d_kq, (ks >> 2) * 16384 + (ks & 3) * 32);
+                    mma_ss(tm_gram, d, d, ID_GRAM, ks > 0);
+                }
+                mma_commit(cx.bar((CL ? PB_GRAM0 : FB_GRAM0) + (int)team));
             }
             __syncwarp();
         }
+        if (CL) {
+            if (k >= 1) cx.wait(PB_SENT0 + (int)team, (k - 1) & 1u);        // the operands of the team's last chunk are in the ring
+        } else {
+            // T' and P were last read by U^T of chunk i - 2 and the outputs of chunk i - 3
+            if (i >= 2) cx.wait(FB_U0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
+            if (i >= 3) cx.wait(FB_DONE0 + (int)((i - 3) & 3u), ((i - 3) >> 2) & 1u);
+        }
+        cx.wait((CL ? PB_DECAY_READY0 : FB_DECAY_READY0) + (int)(i & 3u), (i >> 2) & 1u);
+        cx.wait((CL ? PB_GRAM0 : FB_GRAM0) + (int)team, par);
+        tc_fence_after();
+        float G2t = dc.G2[t];
+        float* col_eG = dc.eG;                                  // column factors of T''
+        if constexpr (RAW && !CL) col_eG = dc.eGk;
+        if (RAW) {
+            // fused input stage: the squared norms of the key rows are the diagonal of K K^T; 1 / |k_s| is folded into the
+            // factors that multiply key s wherever it enters (columns of A^ and P, columns of T''; rows of A^ below).
+            // The query norms multiply the finished output rows.
+            float ss;
+            if (isA) {
+                uint32_t lo[16], hi[16];
+                tmem_ld16(tm_gram + lane_win + (uint32_t)(t & 32), lo);
+                tmem_ld16(tm_gram + lane_win + (uint32_t)(t & 32) + 16u, hi);
+                tmem_ld_wait();
+                uint32_t x8[8], x4[4];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t a = (t & 8) ? lo[e + 8] : lo[e], b = (t & 8) ? hi[e + 8] : hi[e];
+                    x8[e] = (t & 16) ? b : a;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x4[e] = (t & 4) ? x8[e + 4] : x8[e];
+                const uint32_t y0 = (t & 2) ? x4[2] : x4[0], y1 = (t & 2) ? x4[3] : x4[1];
+                ss = __uint_as_float((t & 1) ? y1 : y0);
+            } else {
+                cx.wait(b_kq, kq_par);
+                ss = 0.f;
+#pragma unroll 1
+                for (int i = 0; i < 16; ++i) {
+                    // 16-byte pieces of the row in an order that spreads the lanes over the banks (the sum does not care)
+                    const uint4 x = *reinterpret_cast<const uint4*>(cx.sm + o_kq + 8192 + (uint32_t)(i >> 3) * 16384u + t * 128 + (((i + lane) & 7) << 4));
+                    const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { ss = fmaf(bf_lo(xw[e]), bf_lo(xw[e]), ss); ss = fmaf(bf_hi(xw[e]), bf_hi(xw[e]), ss); }
+                }
+            }
+            const float rn = rsqrtf(ss + kNormEps);
+            dc.norms[(isA ? 0 : 64) + t] = rn;
+            team_sync();
+            if (isA) {
+                dc.beta[t] *= rn; col_eG[t] *= rn;
+                if constexpr (!CL) dc.bRest[t] *= rn;
+                if (t < 32) dc.colfb[t] *= rn;
+                G2t += __log2f(rn);
+            }
+            team_sync();
+        }
+
+        // ---- Gram tile -> A^ (into the T' buffer, where the solve inverts it) and P, 16 columns at a time
+        {
+            uint8_t* prow = (isA ? TP : cx.sm + o_p) + t * 128;
+            const float rowf = lower_rows ? ex2_approx(G2t - dc.G2mid) : 0.f;
+#pragma unroll 1
+            for (int cb = 0; cb < (lower_rows ? 4 : 2); ++cb) {       // (blocks above the diagonal: zero since the start)
+                const int c0 = 16 * cb;
+                uint32_t acc[16];
+                tmem_ld16(tm_gram + lane_win + c0, acc);
+                uint32_t u[8];
+                if (lower_rows && cb < 2) {
+                    // every column precedes every row of this warp: Gam = rowf * colf, no mask, no exp
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i4 = 0; i4 < 4; ++i4) {
+                        const float4 cf = *reinterpret_cast<const float4*>(&dc.colfb[c0 + 4 * i4]);
+                        float f0 = cf.x, f1 = cf.y, f2 = cf.z, f3 = cf.w;
+                        mul_f32x2(f0, f1, rowf, rowf);
+                        mul_f32x2(f2, f3, rowf, rowf);
+                        mul_f32x2(f0, f1, __uint_as_float(acc[4 * i4]), __uint_as_float(acc[4 * i4 + 1]));
+                        mul_f32x2(f2, f3, __uint_as_float(acc[4 * i4 + 2]), __uint_as_float(acc[4 * i4 + 3]));
+                        u[2 * i4] = pack_bf16x2(f0, f1);
+                        u[2 * i4 + 1] = pack_bf16x2(f2, f3);
+                    }
+                } else {
+                    // the two blocks that hold diagonals: columns below lim are kept (of the packed pairs; what is masked may
+                    // have overflowed to inf or NaN)
+                    const int lim = (lane - 16 * (cb & 1)) + (isA ? 0 : 1);
+                    float f[16];
+#pragma unroll
+                    for (int i4 = 0; i4 < 4; ++i4) {
+                        const float4 gs = *reinterpret_cast<const float4*>(&dc.G2[c0 + 4 * i4]);
+                        const float4 cs = *reinterpret_cast<const float4*>(&dc.beta[c0 + 4 * i4]);
+                        f[4 * i4] = ex2_approx(G2t - gs.x); f[4 * i4 + 1] = ex2_approx(G2t - gs.y);
+                        f[4 * i4 + 2] = ex2_approx(G2t - gs.z); f[4 * i4 + 3] = ex2_approx(G2t - gs.w);
+                        mul_f32x2(f[4 * i4], f[4 * i4 + 1], cs.x, cs.y);
+                        mul_f32x2(f[4 * i4 + 2], f[4 * i4 + 3], cs.z, cs.w);
+                    }
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        mul_f32x2(f[2 * i], f[2 * i + 1], __uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1]));
+                        const uint32_t keep = lim >= 2 * i + 2 ? 0xffffffffu : lim == 2 * i + 1 ? 0xffffu : 0u;
+                        u[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]) & keep;
+                    }
+                }
+                *reinterpret_cast<uint4*>(prow + (((2 * cb) ^ (t & 7)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
+                *reinterpret_cast<uint4*>(prow + (((2 * cb + 1) ^ (t & 7)) << 4)) = make_uint4(u[4], u[5], u[6], u[7]);
+            }
+            tc_fence_before();
+        }
+        // T'' of a fused CTA takes the first half of the W~^T buffer, which S0 W~^T of chunk i - 2 has to have read
+        if (!CL) {
+            if (i >= 2) cx.wait(FB_MMA1_0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
+            const int row = w * 16 + (lane >> 1);               // zero what lies above its diagonal
+            for (int ch = (row >> 3) + 1 + (lane & 1); ch < 8; ch += 2)
+                *reinterpret_cast<uint4*>(TPP + row * 128 + ((ch ^ (row & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        team_sync();
+
+        // ---- P^ = (I + A^)^-1, block by block in place; every block of the result is also stored with its columns times
+        // e^G in T''.  8 x 8 diagonal blocks by forward substitution in fp32, then merges 8 -> 16 -> 32 -> 64 on mma.sync:
+        // X21 = -X22 (A21 X11), the intermediate product staying in registers.
+        {
+            const int g = lane >> 2, t4 = lane & 3;
+            const int b16 = 16 * w;                                   // this warp's 16 x 16 diagonal block
+            {
+                // lanes 0-7 and 8-15: the columns of the two 8 x 8 blocks; lanes 16-31 repeat them for the scaled copy
+                const int b = b16 + (lane & 8), jj = lane & 7;
+                float x[8];
+                uint4 rows[7];
+#pragma unroll
+                for (int r = 1; r < 8; ++r) rows[r - 1] = *reinterpret_cast<const uint4*>(TP + sw_off(b + r, b));
+                const float f = lane < 16 ? 1.f : col_eG[b + jj];
+                uint8_t* dst = lane < 16 ? TP : TPP;
+                __syncwarp();                                       // every row is in registers before any is overwritten
+#pragma unroll
+                for (int r = 0; r < 8; ++r) x[r] = (r == jj) ? 1.f : 0.f;
+#pragma unroll
+                for (int r = 1; r < 8; ++r) {
+                    const uint32_t wds[4] = {rows[r - 1].x, rows[r - 1].y, rows[r - 1].z, rows[r - 1].w};
+                    float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll
+                    for (int s2 = 0; s2 < r; ++s2) {
+                        const float a = (s2 & 1) ? bf_hi(wds[s2 >> 1]) : bf_lo(wds[s2 >> 1]);
+                        if (s2 & 1) acc1 = fmaf(a, x[s2], acc1); else acc0 = fmaf(a, x[s2], acc0);
+                    }
+                    x[r] = (r > jj) ? -(acc0 + acc1) : x[r];
+                }
+                // this thread's column of the diagonal block, zeros above the diagonal included
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+                    *reinterpret_cast<__nv_bfloat16*>(dst + sw_off(b + r, b + jj)) = __float2bfloat16_rn(x[r] * f);
+            }
+            __syncwarp();
+            // stores -d (two adjacent columns of row r) to T' and, scaled, to T''
+            auto put = [&](float d0, float d1, int r, int c) {
+                const uint32_t off = sw_off(r, c);
+                *reinterpret_cast<uint32_t*>(TP + off) = pack_bf16x2(-d0, -d1);
+                const float2 e = *reinterpret_cast<const float2*>(&col_eG[c]);
+                *reinterpret_cast<uint32_t*>(TPP + off) = pack_bf16x2(-d0 * e.x, -d1 * e.y);
+            };
+            {
+                uint32_t a[2], bx[2];
+                const int rr = lane & 7, i = (lane >> 3) & 1;
+                ldm_x2(a, xs + sw_off(b16 + 8 + rr, b16 + 8 * i));            // A21, X22
+                ldm_x2_trans(bx, xs + sw_off(b16 + rr, b16));                // X11
+                float m[4] = {0.f, 0.f, 0.f, 0.f}, d[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_8x8(m, a[0], bx[0]);
+                mma_8x8(d, a[1], transpose_8x8(pack_bf16x2(m[0], m[1])));
+                put(d[0], d[1], b16 + 8 + g, b16 + 2 * t4);
+            }
+            team_sync();
+            {
+                // 32-row halves; two warps per half, 8 columns each
+                const int lo = 32 * (w >> 1), hi = lo + 16, c = lo + 8 * (w & 1);
+                uint32_t a[4], a2[4], bx[2];
+                ldm_x4(a, tile_addr_sw(xs, hi, lo, lane));                   // A21
+                ldm_x4(a2, tile_addr_sw(xs, hi, hi, lane));                  // X22
+                ldm_x2_trans(bx, xs + sw_off(lo + (lane & 15), c));          // X11, this warp's columns
+                float m[4] = {0.f, 0.f, 0.f, 0.f}, d[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_bf16(m, a, bx[0], bx[1]);
+                mma_bf16(d, a2, transpose_8x8(pack_bf16x2(m[0], m[1])), transpose_8x8(pack_bf16x2(m[2], m[3])));
+                team_sync();                                                 // both warps of the half have read A21
+                put(d[0], d[1], hi + g, c + 2 * t4);
+                put(d[2], d[3], hi + g + 8, c + 2 * t4);
+            }
+            team_sync();
+            {
+                // rows 32-63, columns 0-31: 8 columns per warp
+                const int c = 8 * w;
+                uint32_t a[2][2][4], bx[4], x22[3][4];
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int kt = 0; kt < 2; ++kt) ldm_x4(a[mt][kt], tile_addr_sw(xs, 32 + 16 * mt, 16 * kt, lane));
+                ldm_x4_trans(bx, xs + sw_off(lane, c));
+                ldm_x4(x22[0], tile_addr_sw(xs, 32, 32, lane));
+                ldm_x4(x22[1], tile_addr_sw(xs, 48, 32, lane));
+                ldm_x4(x22[2], tile_addr_sw(xs, 48, 48, lane));
+                float m[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+                mma_bf16(m[0], a[0][0], bx[0], bx[1]);
+                mma_bf16(m[1], a[1][0], bx[0], bx[1]);
+                mma_bf16(m[0], a[0][1], bx[2], bx[3]);
+                mma_bf16(m[1], a[1][1], bx[2], bx[3]);
+                const uint32_t q0 = transpose_8x8(pack_bf16x2(m[0][0], m[0][1])), q1 = transpose_8x8(pack_bf16x2(m[0][2], m[0][3]));
+                const uint32_t q2 = transpose_8x8(pack_bf16x2(m[1][0], m[1][1])), q3 = transpose_8x8(pack_bf16x2(m[1][2], m[1][3]));
+                mma_bf16(d[0], x22[0], q0, q1);
+                mma_bf16(d[1], x22[1], q0, q1);
+                mma_bf16(d[1], x22[2], q2, q3);
+                team_sync();                                                 // every warp has read A21
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    put(d[mt][0], d[mt][1], 32 + 16 * mt + g, c + 2 * t4);
+                    put(d[mt][2], d[mt][3], 40 + 16 * mt + g, c + 2 * t4);
+                }
+            }
+        }
+        fence_proxy_async_smem();                               // T', T'' are read by MMAs and by the copy
+        team_sync();
+
+        // ---- W~^T = K^T T''^T, then as bf16 rows [dk][t] into the operand buffer
+        if (w == 0) {
+            tc_fence_after();
+            if (elect_one()) {
+                const uint64_t d_kt = smem_desc_sw128(kq, 16384, 1024);      // K^T, M-major
+                const uint64_t d_tpp = smem_desc_sw128(cx.sb + o_tpp, 16, 1024);
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    mma_ss(tm_wacc, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * 32), ID_WU, ks > 0);
+                mma_commit(cx.bar((CL ? PB_W0 : FB_W0) + (int)team));
+            }
+            __syncwarp();
+        }
+        cx.wait((CL ? PB_W0 : FB_W0) + (int)team, par);
+        tc_fence_after();
+        {
+            const int drow = w * 32 + lane;
+            uint8_t* wrow = cx.sm + o_w + drow * 128;
+#pragma unroll 1
+            for (int hf = 0; hf < 4; ++hf) {
+                uint32_t acc[16];
+                tmem_ld16(tm_wacc + lane_win + 16 * hf, acc);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c8 = 0; c8 < 2; ++c8) {
+                    uint4 u;
+                    u.x = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 0]), __uint_as_float(acc[c8 * 8 + 1]));
+                    u.y = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 2]), __uint_as_float(acc[c8 * 8 + 3]));
+                    u.z = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 4]), __uint_as_float(acc[c8 * 8 + 5]));
+                    u.w = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 6]), __uint_as_float(acc[c8 * 8 + 7]));
+                    *reinterpret_cast<uint4*>(wrow + (((2 * hf + c8) ^ (drow & 7)) << 4)) = u;
+                }
+            }
+            tc_fence_before();
+            fence_proxy_async_smem();
+        }
+        warp_arrive(cx.bar((CL ? PB_OPS0 : FB_OPS0) + (int)team), lane);         // the operands are complete
+        team_sync();                                            // (and the accumulators may take the next tiles)
     }
+}
+
+// ================================================================================================
+// Chain CTA
+// ================================================================================================
+// warp 0: K, Q and V tiles of the chunks to come
+__device__ void chain_producer(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v)
+{
+    ChunkCursor ck, cv;                                       // next chunk of K/Q, of V
+    ck.init(prm);
+    cv = ck;
+    const bool leader = elect_one();
+    uint32_t ik = 0, iv = 0;
+    auto load_kq = [&]() {
+        if (leader) {
+            const uint32_t bar = cx.bar(CB_KQ_FULL0 + (int)(ik & 1u)), dst = cx.sb + C_KQ + (ik & 1u) * 32768;
+            mbar_arrive_expect_tx(bar, 32768u);
+            load_tile(dst, tm_k, ck.hq, ck.row0(), bar);
+            load_tile(dst + 16384, tm_q, ck.hq, ck.row0(), bar);
+        }
+        __syncwarp();
+        ck.advance(); ++ik;
+    };
+    auto load_v = [&]() {
+        if (leader) {
+            const uint32_t bar = cx.bar(CB_OPS_FULL0 + (int)(iv % NSLOT));       // (with the operands of the chunk)
+            mbar_arrive_expect_tx(bar, 16384u);
+            load_tile(cx.sb + C_V, tm_v, cv.h, cv.row0(), bar);
+        }
+        __syncwarp();
+        cv.advance(); ++iv;
+    };
+#pragma unroll 1
+    while (cv.valid && !cx.stop()) {
+        // V of chunk i: its buffer is free once U^T of chunk i - 1 has been formed;  K/Q of chunk i: once chunk i - 2 is done
+        if (iv >= 1) cx.wait(CB_U, (iv - 1) & 1u);
+        load_v();
+        if (ik >= 2) cx.wait(CB_DONE0 + (int)((ik - 2) & 3u), ((ik - 2) >> 2) & 1u);
+        load_kq();
+    }
+}
+
+// warp 3: operands out of the ring, three chunks ahead; gives every ring slot that has been read back to its prep CTA
+template <bool RAW>
+__device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
+{
+    const uint32_t R = prm->csize - 1;
+    const uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
+    ChunkCursor cc;
+    cc.init(prm);
+    const bool leader = elect_one();
+#pragma unroll 1
+    for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
+        const uint32_t slot = j % NSLOT;
+        if (j >= NSLOT) {
+            cx.wait(CB_DONE0 + (int)((j - NSLOT) & 3u), ((j - NSLOT) >> 2) & 1u);      // (its operands have landed long ago)
+            const uint32_t f = j - NSLOT;
+            if (leader) mbar_arrive_remote(map_to_rank(cx.bar(PB_CREDIT0 + (int)((f / R) % (prm->ring / R))), 1u + f % R));
+        }
+        cx.wait_cluster(CB_RING0 + (int)(j % prm->ring), (j / prm->ring) & 1u);
+        if (leader) {
+            const uint32_t bar = cx.bar(CB_OPS_FULL0 + (int)slot);
+            const uint8_t* src = ring + (size_t)(j % prm->ring) * kRingSlotBytes;
+            fence_proxy_async_global();
+            mbar_arrive_expect_tx(bar, OPS_BYTES + (RAW ? NORM_BYTES : 0u));
+            bulk_load(cx.sb + C_OPS + slot * OPS_BYTES, src, OPS_BYTES, bar);
+            if (RAW) bulk_load(smem_u32(cx.misc->c.norms[slot]), src + OPS_BYTES, NORM_BYTES, bar);
+        }
+        __syncwarp();
+    }
+}
+
+// warp 1: MMAs.  The serial path of a chain is S0 W~^T -> Delta epilogue -> state update -> state conversion -> next chunk; the
+// other products fill the time in which the epilogues convert: S0 Q^T under the Delta epilogue, Delta^T P^T and the next
+// chunk's U^T under the state conversion.  The state is updated, converted and used in two halves of its columns, so that the
+// second half's MMAs run under the first half's conversion.
+template <bool CL>
+__device__ void chain_mma(const Ctx& cx, const TcParams* prm)
+{
+    ChunkCursor cc;
+    cc.init(prm);
+    const bool has_init = prm->p.init_state != nullptr;
+    constexpr int WH = 4, WA = 8;                           // epilogue warps per half of the state, and in all
+    constexpr uint32_t HALF = CL ? 8192 : 16384;            // from half to half of a K or Q tile
+    const bool leader = elect_one();
+    const uint32_t acc1 = cx.tmem + TM_ACC1;
+    // Shared-memory descriptors: one per operand, of which only the start address (16-byte units) moves from chunk to chunk.  The
+    // warp is on the serial path with everything that it does, so addresses are stepped, not recomputed.
+    const uint64_t d_sw = smem_desc_sw128(0u, 16, 1024), d_mn = smem_desc_sw128(0u, 8192, 1024);
+    const uint32_t sb16 = cx.sb >> 4;
+    uint32_t o_slot = 0, o_kq = 0, o_p = 0, par = 0;          // operand slot (chain CTA), K/Q slot, P buffer (fused CTA);  j & 1
+    // U^T = V^T T'^T of chunk j, whose operand slot is `os` (the Delta operands of chunk j-1 in this accumulator were read by MMAs
+    // issued before)
+    auto form_u = [&](uint32_t j, uint32_t os) {
+        if (CL) {
+            cx.wait(CB_OPS_FULL0 + (int)os, (j / NSLOT) & 1u);
+        } else {
+            cx.wait(FB_OPS0 + (int)(j & 1u), (j >> 1) & 1u);
+            cx.wait(FB_V_FULL, j & 1u);
+        }
+        tc_fence_after();
+        if (leader) {
+            const uint64_t d_v = d_mn + (sb16 + ((CL ? C_V : F_V) >> 4));              // V^T, M-major
+            const uint64_t d_tp = d_sw + (sb16 + (CL ? (C_OPS + OPS_TP) / 16 + os * (OPS_BYTES / 16) : F_TP / 16 + (j & 1u) * 512));
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+                mma_ss(acc1, desc_add(d_v, ks * 2048), desc_add(d_tp, ks * 32), ID_WU, ks > 0);
+            mma_commit(cx.bar(CL ? (int)CB_U : FB_U0 + (int)(j & 1u)));
+        }
+        __syncwarp();
+    };
+    if (CL && cc.valid) form_u(0, 0u);
+#pragma unroll 1
+    for (uint32_t j = 0; cc.valid; ++j) {
+        const bool has_state = !cc.first() || has_init;     // a zero start state is skipped, not multiplied
+        const uint32_t kq16 = sb16 + (CL ? C_KQ / 16 + par * 2048 : F_KQ / 16 + o_kq * 2048);
+        const uint64_t d_wt = d_sw + (sb16 + (CL ? (C_OPS + OPS_W) / 16 + o_slot * (OPS_BYTES / 16) : F_W / 16 + par * 1024));      // W^T rows [dk][t], N-major operand
+        const uint64_t d_p = d_sw + (sb16 + (CL ? (C_OPS + OPS_P) / 16 + o_slot * (OPS_BYTES / 16) : F_P / 16 + o_p * 512));
+        const uint64_t d_q = d_sw + (kq16 + (CL ? 1024u : 512u));            // Q rows, K-major
+        const uint64_t d_kn = d_sw + kq16;                                   // half of the K tile as N-major operand
+        const uint32_t acc2 = cx.tmem + tm_acc2<CL>(par), acc3 = cx.tmem + tm_acc3<CL>(par);
+        if (!CL) form_u(j, 0u);
+        // start state of this chunk: the previous chunk's state converted, or, at a chain start, the previous chain's
+        // state read out and this chain's start state (if any) written
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+            hand_over_sync<WH>(HB_SBF0 + hf);
+            tc_fence_after();
+            if (leader) {
+                if (has_state) {
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks)
+                        mma_ts(acc1, cx.tmem + TM_SBF + hf * 32 + ks * 8, desc_add(d_wt, hf * 8192 + ks * 2048), ID_SW, 1u);
+                }
+                if (hf == 1) mma_commit(cx.bar(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)par));                        // Delta~^T is complete
+            }
+            __syncwarp();
+        }
+        if (CL) {
+            cx.wait(CB_KQ_FULL0 + (int)par, (j >> 1) & 1u);
+            if (j >= 2) cx.wait(CB_ACC_FREE0 + (int)par, ((j >> 1) - 1u) & 1u);
+        } else if (j >= 1) {
+            cx.wait(FB_ACC_FREE, (j - 1) & 1u);
+        }
+        tc_fence_after();
+        if (has_state && leader) {
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+                mma_ts(acc2, cx.tmem + TM_SBF + ks * 8, desc_add(d_q, (ks >> 2) * HALF + (ks & 3) * 32), ID_SQ, ks > 0);
+        }
+        __syncwarp();
+        cc.advance();
+        hand_over_sync<WA>(HB_DP);
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    mma_ts(cx.tmem + TM_S32 + hf * 64, acc1 + TM_DPBF + ks * 16, desc_add(d_kn, hf * HALF + ks * 2048), ID_DK, (has_state || ks > 0) ? 1u : 0u);
+                mma_commit(cx.bar((CL ? CB_STATE0 : FB_STATE0) + hf));             // (covers S0 Q^T as well: the bf16 state may be overwritten)
+            }
+        }
+        __syncwarp();
+        hand_over_sync<WA>(HB_D);
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+                mma_ts(acc3, acc1 + TM_DBF + ks * 16, desc_add(d_p, ks * 32), ID_DP, ks > 0);
+            mma_commit(cx.bar(CL ? CB_OUT0 + (int)par : (int)FB_OUT));
+            mma_commit(cx.bar((CL ? CB_DONE0 : FB_DONE0) + (int)(j & 3u)));       // every tile and operand of this chunk has been read
+        }
+        __syncwarp();
+        par ^= 1u;
+        if (CL) {
+            o_slot = o_slot == NSLOT - 1 ? 0u : o_slot + 1;
+            if (cc.valid) form_u(j + 1, o_slot);
+        } else {
+            o_kq = (o_kq + 1) & 3u;
+            o_p = o_p == 2u ? 0u : o_p + 1;
+        }
+    }
+}
+
+// warp 2: per-chunk factors, up to three chunks ahead
+template <bool RAW>
+__device__ void chain_decay(const Ctx& cx, const TcParams* prm, int lane)
+{
+    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int, float GC, float eGC, float cprev, float c, bool rescale) {
+        const float cinv = rescale ? 1.f : __frcp_rn(c);
+        float r0 = b0 * (ex2_approx(GC - G0) * cinv), r1 = b1 * (ex2_approx(GC - G1) * cinv);
+        if (j >= 4) cx.wait(CB_DECAY_FREE0 + (int)(j & 3u), ((j >> 2) - 1u) & 1u);     // last read by the outputs of chunk j - 4
+        ChainDecay& dc = cx.misc->c.decay[j & 3u];
+        if (RAW) {
+            cx.wait(CB_OPS_FULL0 + (int)(j % NSLOT), (j / NSLOT) & 1u);
+            const float* nm = cx.misc->c.norms[j % NSLOT];
+            r0 *= nm[lane]; r1 *= nm[lane + 32];
+            dc.rq[lane] = nm[64 + lane]; dc.rq[lane + 32] = nm[96 + lane];
+        }
+        dc.eG[lane] = ex2_approx(G0) * cprev; dc.eG[lane + 32] = ex2_approx(G1) * cprev;
+        dc.bRest[lane] = r0; dc.bRest[lane + 32] = r1;
+        if (lane == 0) { dc.wb = cprev * eGC; dc.cfin = c; dc.rescale = rescale ? 1 : 0; }
+        warp_arrive(cx.bar(CB_DECAY_READY0 + (int)(j & 3u)), lane);
+    });
 }
 
 // Start state of a chain from init_state [dk][dv] fp32 (kept out of line: most calls start from zero).  The first chunk
-// starts from a rescaled state (see Decay): the fp32 copy is multiplied by wb of step j.
-__device__ __noinline__ void init_chain(const Ctx& cx, const float* __restrict__ st_in, uint32_t j, uint32_t tl, int hf, int dv)
+// starts from a rescaled state (see ChainDecay): the fp32 copy is multiplied by wb of step j.
+template <bool CL>
+__device__ __noinline__ void init_chain(const Ctx cx, const float* __restrict__ st_in, uint32_t j, uint32_t tl, int cs, int dv)
 {
-    cx.wait(B_DECAY_READY0 + (j & 3u), (j >> 2) & 1u);
-    const float wb = cx.misc->decay[j & 3u].wb;
+    cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);
+    const float wb = chain_rec<CL>(cx.misc, j & 3u).wb;
     tc_fence_after();
 #pragma unroll 1
     for (int g = 0; g < 4; ++g) {
-        const int c0 = 64 * hf + 16 * g;
+        const int c0 = 64 * cs + 16 * g;
         uint32_t acc[16], pk[8];
 #pragma unroll
         for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(st_in[(c0 + i) * 128 + dv]);
@@ -952,14 +1049,14 @@ __device__ __noinline__ void init_chain(const Ctx& cx, const float* __restrict__
     tc_fence_before();
 }
 
-// ================================================================================================
-// warps 12-19: chain group (Delta epilogue, state conversion, outputs, final state)
-// ================================================================================================
-__device__ void role_chain(const Ctx& cx, const TcParams& prm, int wtid)
+// Delta epilogue, state conversion, start and final states.  Two warps per TMEM lane window: cs is the column half (32 tokens of
+// Delta, 64 columns of the state).
+template <bool CL>
+__device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int lane)          // warp: 0 .. 7
 {
-    const Problem& p = prm.p;
-    const int lane = wtid & 31, cw = wtid >> 5;
-    const int w4 = cw & 3, hf = cw >> 2;                  // TMEM lane window, column half
+    const Problem& p = prm->p;
+    const int w4 = warp & 3, cs = warp >> 2;
+    constexpr int WH = 4, WA = 8;                         // (see chain_mma)
     const int dv = w4 * 32 + lane;                        // value-dimension index = TMEM lane
     const uint32_t tl = cx.tmem + ((uint32_t)(w4 * 32) << 16);
     Misc* misc = cx.misc;
@@ -969,186 +1066,263 @@ __device__ void role_chain(const Ctx& cx, const TcParams& prm, int wtid)
     uint32_t j = 0;
 #pragma unroll 1
     for (int r = 0;; ++r) {
-        const uint32_t item = ChunkCursor::item_of(r);
+        const uint32_t item = ChunkCursor::item_of(prm, r);
         if (item >= num_items) break;
-        const int4 ci = ChunkCursor::lookup(&p, prm.s.order, item);
+        const int4 ci = ChunkCursor::lookup(prm, item);
         const int n = ci.w, h = ci.z & 0xffff;
-        const int row_begin = ci.x, row_end = ci.y;
-        const int nchunks = (row_end - row_begin + 63) >> 6;
+        const int nchunks = (ci.y - ci.x + 63) >> 6;
         const size_t st_off = ((size_t)n * p.Hv + h) * 128 * 128;
         float* st_out = p.out_state ? p.out_state + st_off : nullptr;
         if (nchunks == 0) {                                   // empty request: the final state is the start state
             if (st_out)
                 for (int a = 0; a < 64; ++a)
-                    st_out[(64 * hf + a) * 128 + dv] = has_init ? p.init_state[st_off + (64 * hf + a) * 128 + dv] : 0.f;
+                    st_out[(64 * cs + a) * 128 + dv] = has_init ? p.init_state[st_off + (64 * cs + a) * 128 + dv] : 0.f;
             continue;
         }
         // ---- chain start: the previous chain's final state has been read out (below); a start state, if given, goes
         // into tensor memory as the first chunk's bf16 operand and, multiplied by the chunk's decay, as the fp32 state
-        if (has_init) init_chain(cx, p.init_state + st_off, j, tl, hf, dv);
-        warp_arrive(cx.bar(B_SBF_READY), lane);               // the start state of step j is in place
+        if (has_init) init_chain<CL>(cx, p.init_state + st_off, j, tl, cs, dv);
+        hand_over_arrive<WH>(HB_SBF0 + cs);                  // the start state of step j is in place
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c, ++j) {
-            const int row0 = row_begin + c * 64;
-            const int nvalid = min(64, row_end - row0);
             const bool last = c == nchunks - 1;
-            const Decay& dc = misc->decay[j & 3u];
+            const auto& dc = chain_rec<CL>(misc, j & 3u);
 
             // ---- Delta epilogue: bf16 Delta^T and decayed Delta'^T as TMEM A operands ----------------------
-            cx.wait(B_DECAY_READY0 + (j & 3u), (j >> 2) & 1u);   // decay factors of this chunk are published
-            cx.wait(B_MMA1_DONE, j & 1u);
+            cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);   // factors of this chunk are published
+            const float cfin = dc.cfin;
+            const uint32_t acc1 = tl + TM_ACC1 + 32 * cs;
+            cx.wait(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)(j & 1u), CL ? j & 1u : (j >> 1) & 1u);
             tc_fence_after();
-#pragma unroll 1
-            for (int g = 0; g < 2; ++g) {
-                const int c0 = 32 * hf + 16 * g;
-                uint32_t acc[16], d1[8], d2[8];
-                tmem_ld16(tl + TM_ACC1 + c0, acc);
+            // The accumulator holds Delta~^T = Delta^T diag(beta)^-1: times beta e^(G_C - G) / c it is the A operand of the
+            // state update, which the chain waits for; as it stands it is that of the output product (P has beta on its columns).
+            {
+                uint32_t acc[2][16], d[8];
+                tmem_ld16(acc1, acc[0]);
+                tmem_ld16(acc1 + 16, acc[1]);
                 tmem_ld_wait();
 #pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    // the accumulator holds Delta~^T = Delta^T diag(beta)^-1 (see the Gram post-processing): it is the A
-                    // operand of the output product as it stands (P has beta on its columns), and with the factors
-                    // beta e^(G_C - G) / c that of the state update
-                    const float4 er = *reinterpret_cast<const float4*>(&dc.bRest[c0 + 4 * i4]);
-                    const float a0 = __uint_as_float(acc[4 * i4]), a1 = __uint_as_float(acc[4 * i4 + 1]);
-                    const float a2 = __uint_as_float(acc[4 * i4 + 2]), a3 = __uint_as_float(acc[4 * i4 + 3]);
-                    d1[2 * i4] = pack_bf16x2(a0, a1);
-                    d1[2 * i4 + 1] = pack_bf16x2(a2, a3);
-                    d2[2 * i4] = pack_bf16x2(a0 * er.x, a1 * er.y);
-                    d2[2 * i4 + 1] = pack_bf16x2(a2 * er.z, a3 * er.w);
+                for (int g = 0; g < 2; ++g) {
+#pragma unroll
+                    for (int i4 = 0; i4 < 4; ++i4) {
+                        const float4 er = *reinterpret_cast<const float4*>(&dc.bRest[32 * cs + 16 * g + 4 * i4]);
+                        float a0 = __uint_as_float(acc[g][4 * i4]), a1 = __uint_as_float(acc[g][4 * i4 + 1]);
+                        float a2 = __uint_as_float(acc[g][4 * i4 + 2]), a3 = __uint_as_float(acc[g][4 * i4 + 3]);
+                        mul_f32x2(a0, a1, er.x, er.y);
+                        mul_f32x2(a2, a3, er.z, er.w);
+                        d[2 * i4] = pack_bf16x2(a0, a1);
+                        d[2 * i4 + 1] = pack_bf16x2(a2, a3);
+                    }
+                    tmem_st8(acc1 + TM_DPBF + 16 * g, d);
                 }
-                tmem_st8(tl + TM_DBF + c0, d1);
-                tmem_st8(tl + TM_DPBF + c0, d2);
+                tmem_st_wait();
+                tc_fence_before();
+                hand_over_arrive<WA>(HB_DP);
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) d[i] = pack_bf16x2(__uint_as_float(acc[g][2 * i]), __uint_as_float(acc[g][2 * i + 1]));
+                    tmem_st8(acc1 + TM_DBF + 16 * g, d);
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                hand_over_arrive<WA>(HB_D);
             }
-            tmem_st_wait();
-            tc_fence_before();
-            const float cfin = dc.cfin;          // read before the arrivals below let the pipeline move on to the slot's reuse
-            warp_arrive(cx.bar(B_D_READY), lane);
 
             // ---- state: bf16 copy for the next chunk's MMAs, or the final state ------------------------------
             // if the next chunk starts from a rescaled state, the stored state is multiplied by wb on the way
             float wb = 1.f;
             bool rescale = false;
             if (!last) {
-                cx.wait(B_DECAY_READY0 + ((j + 1) & 3u), ((j + 1) >> 2) & 1u);
-                wb = misc->decay[(j + 1) & 3u].wb;
-                rescale = misc->decay[(j + 1) & 3u].rescale != 0;
+                cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)((j + 1) & 3u), ((j + 1) >> 2) & 1u);
+                wb = chain_rec<CL>(misc, (j + 1) & 3u).wb;
+                rescale = chain_rec<CL>(misc, (j + 1) & 3u).rescale != 0;
             }
-            cx.wait(B_STATE_DONE, j & 1u);
-            if (!last) cx.wait(B_SQ_DONE, j & 1u);              // the bf16 state of this chunk has been read for the last time
+            cx.wait((CL ? CB_STATE0 : FB_STATE0) + cs, j & 1u);
             tc_fence_after();
-#pragma unroll 1
-            for (int g = 0; g < 4; ++g) {
-                const int c0 = 64 * hf + 16 * g;
-                uint32_t acc[16];
-                tmem_ld16(tl + TM_S32 + c0, acc);
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const int c0 = 64 * cs + 32 * g;
+                uint32_t acc[32];
+                tmem_ld32(tl + TM_S32 + c0, acc);
                 tmem_ld_wait();
                 if (!last) {
-                    uint32_t pk[8];
+                    uint32_t pk[16];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(__uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1]));
-                    tmem_st8(tl + TM_SBF + (c0 >> 1), pk);
+                    for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(__uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1]));
+                    tmem_st16(tl + TM_SBF + (c0 >> 1), pk);
                     if (rescale) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * wb);
-                        tmem_st16(tl + TM_S32 + c0, acc);
+                        for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * wb);
+                        tmem_st32(tl + TM_S32 + c0, acc);
                     }
                 } else if (st_out && !misc->abort) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) st_out[(c0 + i) * 128 + dv] = __uint_as_float(acc[i]) * cfin;
+                    for (int i = 0; i < 32; ++i) st_out[(c0 + i) * 128 + dv] = __uint_as_float(acc[i]) * cfin;
                 }
             }
             tmem_st_wait();
             tc_fence_before();
-            if (!last) warp_arrive(cx.bar(B_SBF_READY), lane);    // (a chain's first chunk is announced at the chain start)
+            if (!last) hand_over_arrive<WH>(HB_SBF0 + cs);    // (a chain's first chunk is announced at the chain start)
         }
     }
 }
 
-// ================================================================================================
-// warps 24-27: output group (one warp per TMEM lane window).  O^T = diag(e^G) (S0 Q^T) + Delta^T P^T of chunk j,
-// read from the two accumulators as soon as the chunk's last MMAs have completed: first everything is read, combined
-// and rounded into registers, which releases the accumulators for the next chunk early; the stores follow.
-// ================================================================================================
-template <bool RAW>
-__device__ void role_out(const Ctx& cx, const TcParams& prm, int warp, int lane)
+// Outputs, one warp per 16 (fused CTA: 32) TMEM lanes.  O^T = diag(e^G) (S0 Q^T) + Delta^T P^T of chunk j from its pair of
+// accumulators.  The accumulators are read as 16 x 8 fragments, which stmatrix transposes on
+// the way into a [token][value] tile; one TMA store per 64 values takes the tile out.  (Stores straight from the registers
+// cost an address and a 2-byte store per value pair: 1,200 instead of 500 instructions per chunk.)
+template <bool RAW, bool CL>
+__device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_o, int warp, int lane)
 {
-    const Problem& p = prm.p;
-    const int w4 = warp & 3;
-    const int dv = w4 * 32 + lane;
-    const uint32_t tl = cx.tmem + ((uint32_t)(w4 * 32) << 16);
-    __nv_bfloat16* __restrict__ og = reinterpret_cast<__nv_bfloat16*>(p.out_o);
+    const Problem& p = prm->p;
+    constexpr int NW = CL ? 8 : 4;
+    const int w4 = warp & 3, t4 = lane & 3;                   // warp: 0 .. NW - 1
+    const bool leader = warp == 0;
+    // the tile's two halves: a buffer of its own, or the chunk's Q tile, which its products have read (fused CTA)
+    constexpr uint32_t HALF = CL ? 8192 : 16384;
+    auto group_sync = []() { asm volatile("bar.sync 5, %0;" ::"n"(NW * 32) : "memory"); };
+    // stmatrix row addresses: matrices 0, 1 are value rows b .. b + 7, b + 8 .. b + 15 of tokens 8 c .., 2, 3 the same of tokens
+    // 8 c + 8 ..; the tile has 128-byte rows of 64 values, two halves, 16-byte chunks XORed with (token & 7)
+    const int st_tok = ((lane >> 4) << 3) + (lane & 7), v8 = w4 * 4 + (CL ? (warp >> 2) * 2 : 0) + ((lane >> 3) & 1);     // v8: 8-value block of the lane's row
+    const uint32_t st_base = cx.sb + (uint32_t)(v8 >> 3) * HALF;
     ChunkCursor cc;
-    cc.init(&p, prm.s.order);
+    cc.init(prm);
 #pragma unroll 1
     for (uint32_t j = 0; cc.valid; ++j, cc.advance()) {
         const int row0 = cc.row0(), nvalid = cc.nvalid();
         const bool first = cc.first() && p.init_state == nullptr;      // zero start state: S0 Q^T was not computed
-        const Decay& dc = cx.misc->decay[j & 3u];
-        cx.wait(B_DECAY_READY0 + (j & 3u), (j >> 2) & 1u);
-        if (RAW) cx.wait(B_RQ_READY0 + (j & 3u), (j >> 2) & 1u);
-        cx.wait(B_MMA3_DONE, j & 1u);
+        const auto& dc = chain_rec<CL>(cx.misc, j & 3u);
+        const uint32_t o_t = CL ? C_O + (j & 1u) * 16384 : F_KQ + (j & 3u) * 32768 + 8192;
+        uint8_t* const ot = cx.sm + o_t;
+        cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);
+        cx.wait(CL ? CB_OUT0 + (int)(j & 1u) : (int)FB_OUT, CL ? (j >> 1) & 1u : j & 1u);
         tc_fence_after();
-        // For a fixed token the 128 lanes hold 128 consecutive bf16 of out_o: each warp store writes 64 contiguous bytes
-        // (two full sectors), so the outputs go straight from registers to global memory, 16 tokens at a time.
-        uint16_t* optr = reinterpret_cast<uint16_t*>(og) + ((size_t)row0 * p.Hv + cc.h) * 128 + dv;
-        const uint32_t ostride = (uint32_t)p.Hv * 128u;
-        const bool full = nvalid == 64;
+        const uint32_t ta = cx.tmem + ((uint32_t)(w4 * 32 + (CL ? (warp >> 2) * 16 : 0)) << 16), ta3 = ta + tm_acc3<CL>(j), ta2 = ta + tm_acc2<CL>(j);
 #pragma unroll 1
-        for (int g = 0; g < 4; ++g) {
-            const int c0 = 16 * g;
+        for (int g = 0; g < 16 / NW; ++g) {                            // 16 values x 32 tokens
+            const int c0 = 32 * (g & 1);
+            const uint32_t o = ((uint32_t)(g >> 1) << 20) + c0;
             uint32_t a3[16], a2[16];
-            tmem_ld16(tl + TM_ACC3 + c0, a3);
-            if (!first) tmem_ld16(tl + TM_ACC2 + c0, a2);
+            tmem_ld_frag32(ta3 + o, a3);
+            if (!first) tmem_ld_frag32(ta2 + o, a2);
             tmem_ld_wait();
-            if (g == 3) {
-                // both accumulators have been read: the chain may overwrite them while the last block is stored
+            if (g == 16 / NW - 1) {
+                // both accumulators have been read: the chain may overwrite them
                 tc_fence_before();
-                warp_arrive(cx.bar(B_ACC23_FREE), lane);
+                warp_arrive(cx.bar(CL ? CB_ACC_FREE0 + (int)(j & 1u) : (int)FB_ACC_FREE), lane);
             }
             uint32_t pk[8];
 #pragma unroll
-            for (int i4 = 0; i4 < 4; ++i4) {
-                const float4 eg = *reinterpret_cast<const float4*>(&dc.eG[c0 + 4 * i4]);
-                float o0 = __uint_as_float(a3[4 * i4]), o1 = __uint_as_float(a3[4 * i4 + 1]);
-                float o2 = __uint_as_float(a3[4 * i4 + 2]), o3 = __uint_as_float(a3[4 * i4 + 3]);
+            for (int b = 0; b < 4; ++b) {                              // 8 tokens
+                float o0 = __uint_as_float(a3[4 * b]), o1 = __uint_as_float(a3[4 * b + 1]);
+                float o2 = __uint_as_float(a3[4 * b + 2]), o3 = __uint_as_float(a3[4 * b + 3]);
                 if (!first) {
-                    o0 = fmaf(eg.x, __uint_as_float(a2[4 * i4]), o0); o1 = fmaf(eg.y, __uint_as_float(a2[4 * i4 + 1]), o1);
-                    o2 = fmaf(eg.z, __uint_as_float(a2[4 * i4 + 2]), o2); o3 = fmaf(eg.w, __uint_as_float(a2[4 * i4 + 3]), o3);
+                    const float2 eg = *reinterpret_cast<const float2*>(&dc.eG[c0 + 8 * b + 2 * t4]);
+                    fma_f32x2(o0, o1, eg.x, eg.y, __uint_as_float(a2[4 * b]), __uint_as_float(a2[4 * b + 1]));
+                    fma_f32x2(o2, o3, eg.x, eg.y, __uint_as_float(a2[4 * b + 2]), __uint_as_float(a2[4 * b + 3]));
                 }
                 if (RAW) {
                     // fused input stage: the rows are scaled by 1 / norm of their query rows
-                    const float4 rv = *reinterpret_cast<const float4*>(&dc.rq[c0 + 4 * i4]);
-                    o0 *= rv.x; o1 *= rv.y; o2 *= rv.z; o3 *= rv.w;
+                    const float2 rv = *reinterpret_cast<const float2*>(&query_norms(dc)[c0 + 8 * b + 2 * t4]);
+                    mul_f32x2(o0, o1, rv.x, rv.y);
+                    mul_f32x2(o2, o3, rv.x, rv.y);
                 }
-                pk[2 * i4] = pack_bf16x2(o0, o1);
-                pk[2 * i4 + 1] = pack_bf16x2(o2, o3);
+                pk[2 * b] = pack_bf16x2(o0, o1);
+                pk[2 * b + 1] = pack_bf16x2(o2, o3);
             }
-            if (og) {
-                // a full chunk (all but a request's last) stores without per-token predicates
-                if (full) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        optr[(uint32_t)(2 * i) * ostride] = (uint16_t)(pk[i] & 0xffffu);
-                        optr[(uint32_t)(2 * i + 1) * ostride] = (uint16_t)(pk[i] >> 16);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        if (c0 + 2 * i < nvalid) optr[(uint32_t)(2 * i) * ostride] = (uint16_t)(pk[i] & 0xffffu);
-                        if (c0 + 2 * i + 1 < nvalid) optr[(uint32_t)(2 * i + 1) * ostride] = (uint16_t)(pk[i] >> 16);
-                    }
-                }
+            for (int q = 0; q < 2; ++q) {
+                const int tok = c0 + 16 * q + st_tok;
+                stm_x4_trans(st_base + o_t + (uint32_t)(tok * 128 + ((((v8 & 7) + 2 * (g >> 1)) ^ (tok & 7)) << 4)), pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
             }
-            optr += 16u * ostride;
         }
-        warp_arrive(cx.bar(B_DECAY_FREE0 + (j & 3u)), lane);    // last read of this chunk's decay factors
+        warp_arrive(cx.bar((CL ? CB_DECAY_FREE0 : FB_DECAY_FREE0) + (int)(j & 3u)), lane);    // last read of this chunk's factors
+        fence_proxy_async_smem();
+        if (CL && leader && lane == 0) bulk_wait_read();           // the tile of the chunk before has left: the next may take its buffer
+        group_sync();
+        if (p.out_o) {
+            if (nvalid == 64) {
+                if (leader && lane == 0) {
+                    tma_store_3d(tm_o, 0, row0, 2 * cc.h, cx.sb + o_t);
+                    if (!CL) tma_store_3d(tm_o, 0, row0, 2 * cc.h + 1, cx.sb + o_t + HALF);      // (halves apart: boxes of one half)
+                    bulk_commit();
+                    if (!CL) bulk_wait_read();
+                }
+            } else {
+                // a request's last, partial chunk: row by row, 8 bytes per lane
+                uint8_t* og = reinterpret_cast<uint8_t*>(p.out_o) + ((size_t)row0 * p.Hv + cc.h) * 256 + lane * 8;
+                for (int tok = warp; tok < nvalid; tok += NW) {
+                    const uint2 x = *reinterpret_cast<const uint2*>(ot + (lane >> 4) * HALF + tok * 128 + ((((lane >> 1) & 7) ^ (tok & 7)) << 4) + (lane & 1) * 8);
+                    *reinterpret_cast<uint2*>(og + (size_t)tok * p.Hv * 256) = x;
+                }
+                if (!CL) group_sync();
+            }
+        }
+        if (!CL && leader && lane == 0) mbar_arrive(cx.bar(FB_KQ_FREE0 + (int)(j & 3u)));    // the tiles may be overwritten
     }
+    if (leader && lane == 0) bulk_wait();
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-gdn_tc_kernel(const TcParams prm, const __grid_constant__ CUtensorMap tm_q,
-              const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v)
+// ================================================================================================
+// Fused CTA: the roles that differ from those of the split
+// ================================================================================================
+// warp 0: K/Q tiles, up to four chunks ahead
+__device__ void fused_producer_kq(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
+{
+    ChunkCursor cc;
+    cc.init(prm);
+#pragma unroll 1
+    for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
+        if (j >= 4) cx.wait(FB_KQ_FREE0 + (int)(j & 3u), ((j >> 2) - 1u) & 1u);
+        if ((int32_t)j != prm->skip_kq_load) {           // testing aid: the skipped tile never arrives
+            if (elect_one()) load_kq_tiles(cx.sb + F_KQ + (j & 3u) * 32768, tm_q, tm_k, cc.hq, cc.row0(), cx.bar(FB_KQ_FULL0 + (int)(j & 3u)));
+            __syncwarp();
+        }
+    }
+}
+// warp 3: V tiles; the single buffer is free once U^T of the chunk before has been formed
+__device__ void fused_producer_v(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_v)
+{
+    ChunkCursor cc;
+    cc.init(prm);
+#pragma unroll 1
+    for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
+        if (j >= 1) cx.wait(FB_U0 + (int)((j - 1) & 1u), ((j - 1) >> 1) & 1u);
+        if (elect_one()) {
+            const uint32_t bar = cx.bar(FB_V_FULL);
+            mbar_arrive_expect_tx(bar, 16384u);
+            load_tile(cx.sb + F_V, tm_v, cc.h, cc.row0(), bar);
+        }
+        __syncwarp();
+    }
+}
+// warp 2: the factors of both parts, up to three chunks ahead
+template <bool RAW>
+__device__ void fused_decay(const Ctx& cx, const TcParams* prm, int lane)
+{
+    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float GC, float eGC, float cprev, float c, bool rescale) {
+        const float G31 = __shfl_sync(0xffffffffu, G0, 31);
+        const float cinv = rescale ? 1.f : __frcp_rn(c);
+        const float e0 = ex2_approx(G0) * cprev, e1 = ex2_approx(G1) * cprev;
+        if (j >= 4) cx.wait(FB_DECAY_FREE0 + (int)(j & 3u), ((j >> 2) - 1u) & 1u);     // last read by the outputs of chunk j - 4
+        FusedDecay& dc = cx.misc->f.decay[j & 3u];
+        dc.G2[lane] = lane < nvalid ? G0 : -1.0e30f; dc.G2[lane + 32] = lane + 32 < nvalid ? G1 : -1.0e30f;      // (see prep_decay)
+        dc.beta[lane] = b0; dc.beta[lane + 32] = b1;
+        dc.eG[lane] = e0; dc.eG[lane + 32] = e1;
+        if (RAW) { dc.eGk[lane] = e0; dc.eGk[lane + 32] = e1; }
+        dc.bRest[lane] = b0 * (ex2_approx(GC - G0) * cinv); dc.bRest[lane + 32] = b1 * (ex2_approx(GC - G1) * cinv);
+        dc.colfb[lane] = ex2_approx(G31 - G0) * b0;
+        if (lane == 0) { dc.wb = cprev * eGC; dc.G2mid = G31; dc.cfin = c; dc.rescale = rescale ? 1 : 0; }
+        warp_arrive(cx.bar(FB_DECAY_READY0 + (int)(j & 3u)), lane);
+    });
+}
+
+template <bool RAW, bool CL>
+__global__ void __launch_bounds__(kThreads<CL>, 1)
+gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+              const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_qt,
+              const __grid_constant__ CUtensorMap tm_kt)      // q, k: boxes of one half;  v, qt, kt: of both;  o: of one (fused) or both
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -1156,73 +1330,73 @@ gdn_tc_kernel(const TcParams prm, const __grid_constant__ CUtensorMap tm_q,
     cx.sb = (raw + 1023u) & ~1023u;
     cx.sm = smem_raw + (cx.sb - raw);
     cx.misc = reinterpret_cast<Misc*>(cx.sm + SM_MISC);
+    const uint32_t rank = CL ? blockIdx.x % prm.csize : 0u;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // Start-up.  Everybody zeroes its share of the operand tiles T' (3), T'' and P (3), contiguous, which are only ever
-    // written on and below their 16 x 16 diagonal blocks.  The producer then sets up the barriers of its own slots and
-    // goes straight to its first tile copies; it only announces itself at the start-up barrier (named barrier 2) and
-    // joins the others again (named barrier 5) before its main loop, which needs their barriers.  Warp 3 allocates
-    // tensor memory, threads 36.. set up one barrier each.
-    for (uint32_t i = tid; i < 7u * 8192u / 16u; i += kThreads)
-        *reinterpret_cast<uint4*>(cx.sm + SM_TP + i * 16u) = make_uint4(0u, 0u, 0u, 0u);
-    fence_proxy_async_smem();
-    Producer prod;
-    if (warp == 0) {
-        if (lane == 0) {
-            prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
-            for (int i = B_FULL_KQ0; i <= B_FULL_V; ++i) mbar_init(cx.bar(i), 1u);
-            fence_mbar_init();
-            fence_proxy_async_smem();
+    if (!CL) {
+        // T' and P are only ever written on and below their 16 x 16 diagonal blocks: zero above them
+        for (uint32_t i = tid; i < 5u * 8192u / 16u; i += kThreads<CL>)
+            *reinterpret_cast<uint4*>(cx.sm + F_TP + i * 16u) = make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async_smem();
+    } else if (rank != 0) {
+        // T', P and T'' of every team are only ever written on and below their 16 x 16 diagonal blocks: zero above them
+        for (uint32_t i = tid; i < NT * 24576u / 16u; i += kThreads<CL>) {
+            const uint32_t team = i / 1536u, o = (i % 1536u) * 16u;
+            *reinterpret_cast<uint4*>(cx.sm + team * P_TEAM + P_OPS + OPS_TP + o) = make_uint4(0u, 0u, 0u, 0u);
         }
-        __syncwarp();
-        asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");
-        prod.begin(cx, prm, &tm_q, &tm_k);
-        asm volatile("bar.sync 5, %0;" ::"n"(kThreads) : "memory");
-    } else {
-        if (warp == 3) {
-            tmem_alloc(cx.sb + SM_MISC + (uint32_t)offsetof(Misc, tmem_base), 512);
-            tmem_relinquish();
-        } else if (tid - 32 > B_FULL_V && tid - 32 < NUM_BARS) {
-            // Arrivals per phase: one per warp of the arriving group (G1 and chain: 8 warps, output group: 4, a solve
-            // team: 2), one for barriers that a single thread or an MMA commit completes; in the fused input stage a
-            // K/Q slot is released by the chain's last MMAs and by the Gram warp's reading of Q
-            const int i = tid - 32;
-            const bool wg_bar = i == B_GRAM_READ || i == B_D_READY || i == B_SBF_READY ||
-                                i == B_WACC_READ || i == B_PRE_DONE0 || i == B_PRE_DONE1 ||
-                                i == B_A_READY0 || i == B_A_READY1 || i == B_A_READY2;
-            const bool out_bar = i == B_ACC23_FREE || (i >= B_DECAY_FREE0 && i <= B_DECAY_FREE3);
-            const bool g2_bar = i == B_TP_READY0 || i == B_TP_READY1 || i == B_TP_READY2;
-            const bool kq_free2 = prm.p.input_raw && i >= B_KQ_FREE0 && i <= B_KQ_FREE2;
-            mbar_init(cx.bar(i), wg_bar ? 8u : out_bar ? 4u : (g2_bar || kq_free2) ? 2u : 1u);
-            fence_mbar_init();
-            if (i == NUM_BARS - 1) {
-                cx.misc->abort = 0u;
-                cx.misc->timeout_ns = prm.wait_timeout_ns;
-            }
-        }
-        tc_fence_before();
-        asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-        asm volatile("bar.arrive 5, %0;" ::"n"(kThreads) : "memory");
-        tc_fence_after();
+        fence_proxy_async_smem();
     }
+    if (warp == 0) {
+        if (lane == 0) { prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); if (rank == 0) prefetch_tmap(&tm_v); }
+    } else if (warp == 3) {
+        tmem_alloc(cx.sb + SM_MISC + (uint32_t)offsetof(Misc, tmem_base), 512);
+        tmem_relinquish();
+    } else if (tid >= 128 && tid < 128 + 40) {
+        // Arrivals per phase: one per warp of the arriving group, one where a single thread or an MMA commit completes it
+        const int i = tid - 128;
+        uint32_t count = 1;
+        if (!CL) {
+            if (i == FB_OPS0 || i == FB_OPS0 + 1) count = 4;
+            if (i == FB_ACC_FREE || i >= FB_DECAY_FREE0) count = 4;
+        } else if (rank == 0) {
+            if (i >= CB_OPS_FULL0 && i < CB_OPS_FULL0 + (int)NSLOT) count = 2;              // V tile and operands
+            if (i == CB_ACC_FREE0 || i == CB_ACC_FREE1 || (i >= CB_DECAY_FREE0 && i < CB_DECAY_FREE0 + 4)) count = 8;
+        } else if (i >= PB_OPS0 && i < PB_OPS0 + (int)NT) {
+            count = 4;
+        }
+        mbar_init(cx.bar(i), count);
+        fence_mbar_init();
+        if (i == 0) {
+            cx.misc->abort = 0u;
+            cx.misc->timeout_ns = prm.wait_timeout_ns;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (CL) cluster_sync_all();               // every CTA's barriers exist before another CTA arrives on them
+    tc_fence_after();
     cx.tmem = cx.misc->tmem_base;
 
-    // the fused input stage is a property of the launch: the roles it touches exist in two versions, and a launch only
-    // ever executes one of them (its instructions never compete for the instruction cache with the other's)
-    const bool fused = prm.p.input_raw != 0;
-    if (warp < 4) {
-        if (warp == 0) prod.run(cx, prm, &tm_q, &tm_k, &tm_v);
-        else if (warp == 1) role_mma_chain(cx, prm);
-        else if (warp == 2) { if (fused) role_mma_gram<true>(cx, prm); else role_mma_gram<false>(cx, prm); }
-        else { if (fused) role_decay<true>(cx, prm); else role_decay<false>(cx, prm); }
-    } else if (warp >= 24) {
-        if (fused) role_out<true>(cx, prm, warp, lane); else role_out<false>(cx, prm, warp, lane);
-    } else if (warp < 12) {
-        if (fused) role_g1<true>(cx, prm, tid - 128); else role_g1<false>(cx, prm, tid - 128);
-    } else if (warp < 20) {
-        role_chain(cx, prm, tid - 384);
+    if (!CL) {
+        if (warp == 0) fused_producer_kq(cx, &prm, &tm_q, &tm_k);
+        else if (warp == 1) chain_mma<false>(cx, &prm);
+        else if (warp == 2) fused_decay<RAW>(cx, &prm, lane);
+        else if (warp == 3) fused_producer_v(cx, &prm, &tm_v);
+        else if (warp < 12) prep_team<RAW, false>(cx, &prm, 0u, (uint32_t)(warp - 4) >> 2, warp & 3, lane);
+        else if (warp < 20) chain_epilogue<false>(cx, &prm, warp - 12, lane);
+        else chain_out<RAW, false>(cx, &prm, &tm_o, warp - 20, lane);
+    } else if (rank == 0) {
+        if (warp == 0) chain_producer(cx, &prm, &tm_qt, &tm_kt, &tm_v);
+        else if (warp == 1) chain_mma<true>(cx, &prm);
+        else if (warp == 2) chain_decay<RAW>(cx, &prm, lane);
+        else if (warp == 3) chain_receiver<RAW>(cx, &prm);
+        else if (warp < 12) chain_epilogue<true>(cx, &prm, warp - 4, lane);
+        else chain_out<RAW, true>(cx, &prm, &tm_o, warp - 12, lane);
     } else {
-        role_g2(cx, prm, (tid - 640) & 63, (warp - 20) >> 1);
+        if (warp == 0) prep_producer(cx, &prm, rank, &tm_q, &tm_k);
+        else if (warp == 2) prep_decay<RAW>(cx, &prm, rank, lane);
+        else if (warp >= 4 && warp < 4 + 4 * (int)NT) prep_team<RAW, true>(cx, &prm, rank, (uint32_t)(warp - 4) >> 2, warp & 3, lane);
+        else if (warp >= 16 && warp < 16 + (int)NT) prep_sender<RAW>(cx, &prm, rank, (uint32_t)warp - 16u);
     }
 
     tc_fence_before();
@@ -1234,6 +1408,7 @@ gdn_tc_kernel(const TcParams prm, const __grid_constant__ CUtensorMap tm_q,
         __syncthreads();
     }
     if (warp == 3) tmem_dealloc(cx.tmem, 512);
+    if (CL) cluster_sync_all();               // no CTA leaves while another may still signal it
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1253,19 +1428,85 @@ EncodeTiledFn get_encode()
     return fn;
 }
 
-// [rows][cols] bf16 row-major viewed as a 2-D tensor; boxes of 64 columns (128 bytes) x 64 rows,
-// 128-byte swizzle; rows past the end read as zero.
-bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols)
+// [rows][heads][128] bf16 row-major viewed as [half head][row][64]; boxes of 64 rows and 1 or 2 halves, 128-byte swizzle; rows
+// past the end read as zero.
+bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t heads, uint32_t halves)
 {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {64, 64};
-    cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+    cuuint64_t dims[3] = {64, rows, 2 * heads};
+    cuuint64_t strides[2] = {heads * 256, 128};
+    cuuint32_t box[3] = {64, 64, halves};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+struct Maps { CUtensorMap q, k, v, o, qt, kt; };
+
+// CTAs (csize 1) or clusters of a size that fit on a device at the same time; the kernels' attributes are set on the first
+// call per device.
+template <bool RAW, bool CL>
+cudaError_t capacity(int dev, uint32_t csize, int* out)
+{
+    static int cap[64] = {};
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (cap[dev] == 0) {
+        cudaError_t e = cudaFuncSetAttribute(gdn_tc_kernel<RAW, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        int n = 0;
+        if (CL) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+            cfg.gridDim = csize; cfg.blockDim = kThreads<CL>; cfg.dynamicSmemBytes = SMEM_BYTES; cfg.attrs = at; cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&n, gdn_tc_kernel<RAW, CL>, &cfg);
+        } else {
+            e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        }
+        if (e != cudaSuccess) return e;
+        cap[dev] = n > 0 ? n : 1;
+    }
+    *out = cap[dev];
+    return cudaSuccess;
+}
+template <bool RAW, bool CL>
+cudaError_t launch_as(TcParams& prm, uint32_t csize, long long groups, Maps& m, cudaStream_t stream)
+{
+    prm.csize = csize;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = (unsigned)groups * csize;
+    cfg.blockDim = kThreads<CL>; cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = CL ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, gdn_tc_kernel<RAW, CL>, (const TcParams)prm, m.q, m.k, m.v, m.o, m.qt, m.kt);
+}
+template <bool RAW>
+cudaError_t launch(TcParams& prm, Maps& m, cudaStream_t stream)
+{
+    int dev = 0, cap = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const long long items = (long long)prm.p.num_seqs * prm.p.Hv;
+    static_assert(kRingSlots % (NT * (kClusterCtas - 1)) == 0, "see TcParams::ring");
+    prm.ring = kRingSlots;
+    if (prm.s.ring && items <= kRingClusters) {
+        e = capacity<RAW, true>(dev, kClusterCtas, &cap);
+        if (e != cudaSuccess) return e;
+        if (items <= cap) {
+            const Problem& p = prm.p;
+            if (!make_map(&m.qt, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) || !make_map(&m.kt, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) ||
+                !make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2))
+                return cudaErrorUnknown;
+            return launch_as<RAW, true>(prm, kClusterCtas, items, m, stream);
+        }
+    }
+    e = capacity<RAW, false>(dev, 1, &cap);
+    if (e != cudaSuccess) return e;
+    return launch_as<RAW, false>(prm, 1, items < cap ? items : cap, m, stream);
 }
 
 unsigned long long g_wait_timeout_ns = 2000000000ull;
@@ -1288,30 +1529,17 @@ bool tcgen05_supported(const Problem& p)
 cudaError_t launch_tcgen05(const Problem& p, const Sched& s, cudaStream_t stream, int* launches)
 {
     if (!tcgen05_supported(p)) return cudaErrorNotSupported;
-    CUtensorMap tq, tk, tv;
-    if (!make_map(&tq, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq * 128) ||
-        !make_map(&tk, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq * 128) ||
-        !make_map(&tv, p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv * 128))
+    Maps m;
+    if (!make_map(&m.q, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 1) || !make_map(&m.k, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 1) ||
+        !make_map(&m.v, p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2) ||
+        !make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 1))
         return cudaErrorUnknown;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    static bool attr_set[64] = {};
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(gdn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    long long grid = (long long)p.num_seqs * p.Hv;
-    if (grid > sms) grid = sms;
+    m.qt = m.q; m.kt = m.k;
     TcParams prm;
     prm.p = p; prm.s = s;
     prm.wait_timeout_ns = g_wait_timeout_ns; prm.skip_kq_load = g_skip_kq_load;
     g_skip_kq_load = -1;                                        // one-shot: consumed by this launch
-    gdn_tc_kernel<<<(unsigned)grid, kThreads, SMEM_BYTES, stream>>>(prm, tq, tk, tv);
-    e = cudaGetLastError();
+    const cudaError_t e = p.input_raw ? launch<true>(prm, m, stream) : launch<false>(prm, m, stream);
     if (e == cudaSuccess && launches) *launches += 1;
     return e;
 }
