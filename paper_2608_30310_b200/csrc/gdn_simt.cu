@@ -1,207 +1,536 @@
-// fp32 path of the GDN forward: token-recurrent evaluation of Eq. 1 with plain FFMA.
+// fp32 path of the GDN forward: Eq. 1 in blocks of eight tokens with plain FFMA.
 //
-// One CTA walks one chain (request n, v-head h) at a time.  The dv x dk state S lives in
-// registers: thread (j, part) owns 32 entries of row j of S.  Per token, with the state before
-// the token S' and a = alpha_t, b = beta_t:
-//     r = S' k,  p = S' q                      (row dot products, reduced over the row's threads)
-//     delta = b (v - a r)
-//     S = a S' + delta k^T                      (== S' a (I - b k k^T) + b v k^T, Eq. 1)
-//     o = S q = a p + delta (k . q)
-// This path serves fp32 io (tolerance 1e-4 rules out tf32/bf16 tensor cores) and every shape
-// the tensor-core path does not cover.
+// Per block with start state S (dv x dk), G_t = product of alpha over the block up to token t, R(t, i) = G_t / G_i (formed as the
+// product of the alphas between, so that alpha = 0 is exact):
+//     r_t = S k_t,  p_t = S q_t                                                       (state-dependent dot products)
+//     y_t = beta_t (v_t - G_t r_t),  M[t][i] = beta_t R(t,i) (k_i . k_t) for i < t,  N[t][i] = R(t,i) (k_i . q_t) for i <= t
+//     delta = (I + M)^-1 y,  o_t = G_t p_t + (N (I + M)^-1 y)_t                        (8 x 8 matrices, formed ahead)
+//     S = G_8 S + sum_i R(8,i) delta_i k_i^T
+// which is 3 dk dv FMAs per token and head; the rows of S are independent of each other.
+//
+// A CTA owns a slice of 2 RPT NW rows of one chain (request, v-head): NW warps of 2 RPT rows each.  Sixteen lanes share RPT
+// rows, DK / 16 columns per lane, all in registers.  The dot products of a token are reduced over the sixteen lanes by a
+// reduce-scatter that leaves each lane one of the 2 RPT values (a row's r or p) for all eight tokens, so that the 8 x 8 products run
+// inside a lane; eight tokens share the latency (one token at a time, each waited for a shuffle reduction: 400 ns a token).  NH helper warps
+// run ahead by a stage of 8 NH tokens: they load k, q, g and beta, apply the input stage if asked, and form the 8 x 8
+// coefficients.
+//
+// What bounds it: with RPT = 8 the FMA pipe (240 of its cycles per token and 16 rows, 192 of them the 3 dk dv) and, nearly as
+// much, the shared-memory loads: a 16-byte load occupies the SM's load path for four cycles whatever it broadcasts, so a loaded
+// k or q value has to serve many rows (8 lanes to RPT = 4 rows: 340 cycles a token, bound by the loads; RPT = 1: four times as many).
+//
+// This path serves fp32 io (tolerance 1e-4 rules out tf32/bf16 tensor cores) and every shape the tensor-core path does not cover.
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace gdn {
+namespace {
 
-template <typename T> __device__ __forceinline__ float to_f32(T x);
-template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
+using ptx::fma_f32x2;
+using ptx::mul_f32x2;
+
 template <typename T> __device__ __forceinline__ T from_f32(float x);
 template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
-constexpr int kTokBlock = 16;   // tokens staged in shared memory per step
+constexpr int kBlk = 8;            // tokens per block
+constexpr int kBufs = 3;           // stages in flight
 
-template <int DK, int DV, typename T>
-__global__ void __launch_bounds__(DV * (DK / 32))
-gdn_simt_kernel(const Problem p, const Sched s)
+// coefficients of one block (see the head of the file)
+struct __align__(16) Coef {
+    float A[2][kBlk][kBlk];               // [0][i][t]  (I + M)^-1 - I;  [1][i][t]  N (I + M)^-1  (zero for i > t)
+    float c1[2][kBlk], c2[2][kBlk];       // [0] delta's lanes: beta, -beta G;  [1] the outputs' lanes: 0, G
+    float rest[kBlk];                     // R(8, i)
+    float gend; float pad[3];             // G_8
+};
+
+template <int DK, int RPT, int NW, int NH>
+struct Smem {
+    static constexpr int LD = DK + 4;     // row stride: 16-byte aligned, and eight rows at one column fall into different banks
+    float k[kBufs][NH * kBlk][LD], q[kBufs][NH * kBlk][LD];
+    Coef coef[kBufs][NH];
+    __align__(16) float al[NH][2 * kBlk];                // helpers: alpha and beta of the block at hand
+    __align__(16) float mn[NH][2][kBlk][kBlk];           // helpers: [0][i][t] -M, [1][i][t] N
+    __align__(16) float dr[NW][kBlk][2 * RPT];           // R(8, i) delta_i by token
+    __align__(16) float v[NW][kBlk][2 * RPT];            // v of the block
+};
+
+// N consecutive values of v as fp32, in one load that stays where it is written (the compiler would sink a prefetch to its first
+// use, a block later); zeros where !ok
+template <int N> __device__ __forceinline__ void load_early(float (&x)[N], const float* p, bool ok)
 {
-    constexpr int TPR = DK / 32;           // threads per state row
-    constexpr int NT = DV * TPR;
-    constexpr int R = 32;                   // state entries per thread
-    __shared__ __align__(16) float ks[kTokBlock][DK];
-    __shared__ __align__(16) float qs[kTokBlock][DK];
-    __shared__ float vs[kTokBlock][DV];
-    __shared__ float os[kTokBlock][DV];
-    __shared__ float as[kTokBlock], bs[kTokBlock], kqs[kTokBlock];
-    __shared__ uint32_t item_s;
+    uint32_t u[4] = {0u, 0u, 0u, 0u};
+    if constexpr (N == 4)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];\n\t}" : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]) : "l"(p), "r"((uint32_t)ok));
+    else if constexpr (N == 2)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p ld.global.nc.v2.b32 {%0, %1}, [%2];\n\t}" : "+r"(u[0]), "+r"(u[1]) : "l"(p), "r"((uint32_t)ok));
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}" : "+r"(u[0]) : "l"(p), "r"((uint32_t)ok));
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = __uint_as_float(u[i]);
+}
+template <int N> __device__ __forceinline__ void load_early(uint32_t (&u)[(N + 1) / 2], const __nv_bfloat16* p, bool ok)
+{
+#pragma unroll
+    for (int i = 0; i < (N + 1) / 2; ++i) u[i] = 0u;
+    if constexpr (N == 4)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p ld.global.nc.v2.b32 {%0, %1}, [%2];\n\t}" : "+r"(u[0]), "+r"(u[1]) : "l"(p), "r"((uint32_t)ok));
+    else if constexpr (N == 2)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}" : "+r"(u[0]) : "l"(p), "r"((uint32_t)ok));
+    else
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.b16 h, 0;\n\t@p ld.global.nc.b16 h, [%1];\n\tmov.b32 %0, {h, 0};\n\t}" : "=r"(u[0]) : "l"(p), "r"((uint32_t)ok));
+}
+// v of the next block in registers: N values per lane of one token
+template <typename T, int N> struct VNext;
+template <int N> struct VNext<float, N> {
+    float x[N];
+    __device__ __forceinline__ void load(const float* p, bool ok) { load_early<N>(x, p, ok); }
+    __device__ __forceinline__ float get(int i) const { return x[i]; }
+};
+template <int N> struct VNext<__nv_bfloat16, N> {
+    uint32_t u[(N + 1) / 2];
+    __device__ __forceinline__ void load(const __nv_bfloat16* p, bool ok) { load_early<N>(u, p, ok); }
+    __device__ __forceinline__ float get(int i) const { return __uint_as_float((i & 1) ? (u[i / 2] & 0xffff0000u) : (u[i / 2] << 16)); }
+};
 
-    const int tid = threadIdx.x;
-    const int j = tid / TPR;               // state row (dv index)
-    const int part = tid % TPR;            // which interleaved slice of dk
-    const int lane = tid & 31, warp = tid >> 5;
-    const int G = p.Hv / p.Hq;
-    const uint32_t num_items = (uint32_t)p.num_seqs * (uint32_t)p.Hv;
-    const T* __restrict__ qg = (const T*)p.q;
+// x += a * (b0, b1), kept in the order written
+__device__ __forceinline__ void fma_f32x2_here(float2& x, float2 a, float b0, float b1)
+{
+    asm volatile("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%0, %1};\n\tmov.b64 q, {%2, %3};\n\tmov.b64 r, {%4, %5};\n\t"
+        "fma.rn.f32x2 p, q, r, p;\n\tmov.b64 {%0, %1}, p;\n\t}"
+        : "+f"(x.x), "+f"(x.y) : "f"(a.x), "f"(a.y), "f"(b0), "f"(b1));
+}
+
+template <int ID> __device__ __forceinline__ void bar_sync(int buf, int n) { asm volatile("bar.sync %0, %1;" ::"r"(ID + buf), "r"(n) : "memory"); }
+template <int ID> __device__ __forceinline__ void bar_arrive(int buf, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(ID + buf), "r"(n) : "memory"); }
+constexpr int BAR_FULL = 1, BAR_EMPTY = 1 + kBufs;
+
+// Item -> (request, v-head, row slice), longest requests first.  The items are dealt to the SMs in snake order (block b runs on
+// SM b modulo their number as long as the GPU is empty): the longest share their SM with the shortest.
+struct Item { int n, h, hq, slice, row_begin, row_end; };
+template <int SLICES>
+__device__ __forceinline__ bool item_at(const Problem& p, const Sched& s, int sms, uint32_t round, Item& it)
+{
+    const uint32_t pos = blockIdx.x % sms, r = blockIdx.x / sms + round * ((gridDim.x + sms - 1) / sms);
+    const uint32_t item = r * sms + ((r & 1u) ? sms - 1 - pos : pos);
+    if (item >= (uint32_t)p.num_seqs * p.Hv * SLICES) return false;
+    it.slice = (int)(item % SLICES);
+    const uint32_t c = item / SLICES;
+    it.h = (int)(c % p.Hv);
+    it.n = s.order[c / p.Hv];
+    it.hq = it.h / (p.Hv / p.Hq);
+    it.row_begin = p.cu[it.n]; it.row_end = p.cu[it.n + 1];
+    return true;
+}
+
+// the next item of the block with round >= round, which it updates; false when there is none
+template <int SLICES>
+__device__ __forceinline__ bool more(const Problem& p, const Sched& s, int sms, uint32_t& round, Item& it)
+{
+    const uint32_t per = (gridDim.x + sms - 1) / sms, items = (uint32_t)p.num_seqs * p.Hv * SLICES;
+    for (; (blockIdx.x / sms + round * per) * sms < items; ++round)
+        if (item_at<SLICES>(p, s, sms, round, it)) return true;
+    return false;
+}
+
+// four values of a 16-byte piece (fp32) or eight (bf16), as fp32
+template <typename T> struct Piece { static constexpr int N = 16 / sizeof(T); uint4 u; };
+__device__ __forceinline__ void widen(const Piece<float>& x, float (&f)[4])
+{
+    f[0] = __uint_as_float(x.u.x); f[1] = __uint_as_float(x.u.y); f[2] = __uint_as_float(x.u.z); f[3] = __uint_as_float(x.u.w);
+}
+__device__ __forceinline__ void widen(const Piece<__nv_bfloat16>& x, float (&f)[8])
+{
+    const uint32_t w[4] = {x.u.x, x.u.y, x.u.z, x.u.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(w[i] << 16); f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+}
+
+// ---- helper warp: block `hw` of every stage ---------------------------------------------------------------
+template <int DK, int SLICES, typename T, int RPT, int NW, int NH>
+__device__ void helper(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& sm, int sms, int hw, int lane)
+{
+    constexpr int NTHR = (NW + NH) * 32;
+    constexpr int PV = Piece<T>::N, PPR = DK / PV;        // values per 16-byte piece, pieces (lanes) per row
+    constexpr int RPL = 32 / PPR, NL = kBlk / RPL;        // rows per warp-wide load, loads per block
+    const int prow = lane / PPR, pcol = (lane % PPR) * PV;
     const T* __restrict__ kg = (const T*)p.k;
+    const T* __restrict__ qg = (const T*)p.q;
+    Piece<T> rk[NL], rq[NL];
+    float gb = 0.f;                                       // lanes 0-7: g, lanes 8-15: beta
+    auto load = [&](const Item& it, int row0) {
+#pragma unroll
+        for (int i = 0; i < NL; ++i) {
+            const int row = row0 + i * RPL + prow;
+            rk[i].u = make_uint4(0u, 0u, 0u, 0u); rq[i].u = make_uint4(0u, 0u, 0u, 0u);
+            if (row < it.row_end) {
+                const size_t off = ((size_t)row * p.Hq + it.hq) * DK + pcol;
+                rk[i].u = *reinterpret_cast<const uint4*>(kg + off);
+                rq[i].u = *reinterpret_cast<const uint4*>(qg + off);
+            }
+        }
+        const int row = row0 + (lane & 7);
+        gb = 0.f;
+        if (lane < 16 && row < it.row_end) gb = (lane < 8 ? p.g : p.beta)[(size_t)row * p.Hv + it.h];
+    };
+
+    uint32_t stage = 0;
+    Item it;
+    for (uint32_t round = 0; more<SLICES>(p, s, sms, round, it); ++round) {
+        int row0 = it.row_begin + hw * kBlk;
+        if (it.row_begin < it.row_end) load(it, row0);
+#pragma unroll 1
+        for (int base = it.row_begin; base < it.row_end; base += NH * kBlk, row0 += NH * kBlk, ++stage) {
+            const int buf = (int)(stage % kBufs);
+            if (stage >= kBufs) bar_sync<BAR_EMPTY>(buf, NTHR);
+            float (*ks)[Smem<DK, RPT, NW, NH>::LD] = &sm.k[buf][hw * kBlk];
+            float (*qs)[Smem<DK, RPT, NW, NH>::LD] = &sm.q[buf][hw * kBlk];
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                float fk[PV], fq[PV];
+                widen(rk[i], fk); widen(rq[i], fq);
+                if (p.input_raw) {
+                    // fused input stage: rows L2-normalised, x / sqrt(sum x^2 + eps)
+                    float sk = 0.f, sq = 0.f;
+#pragma unroll
+                    for (int e = 0; e < PV; ++e) { sk = fmaf(fk[e], fk[e], sk); sq = fmaf(fq[e], fq[e], sq); }
+#pragma unroll
+                    for (int o = PPR / 2; o > 0; o >>= 1) { sk += __shfl_xor_sync(0xffffffffu, sk, o); sq += __shfl_xor_sync(0xffffffffu, sq, o); }
+                    const float nk = rsqrtf(sk + kNormEps), nq = rsqrtf(sq + kNormEps);
+#pragma unroll
+                    for (int e = 0; e < PV; ++e) { fk[e] *= nk; fq[e] *= nq; }
+                }
+#pragma unroll
+                for (int e = 0; e < PV; e += 4) {
+                    *reinterpret_cast<float4*>(&ks[i * RPL + prow][pcol + e]) = make_float4(fk[e], fk[e + 1], fk[e + 2], fk[e + 3]);
+                    *reinterpret_cast<float4*>(&qs[i * RPL + prow][pcol + e]) = make_float4(fq[e], fq[e + 1], fq[e + 2], fq[e + 3]);
+                }
+            }
+            {
+                // rows past the end: alpha = 1, beta = 0 (k, q are zero)
+                const bool ok = row0 + (lane & 7) < it.row_end;
+                float x;
+                if (p.input_raw) x = ok ? 1.f / (1.f + expf(-gb)) : (lane < 8 ? 1.f : 0.f);      // sigmoid of both pre-activations
+                else x = lane < 8 ? (ok ? expf(gb) : 1.f) : gb;
+                if (lane < 16) sm.al[hw][lane] = x;
+            }
+            __syncwarp();
+            if (base + NH * kBlk < it.row_end) load(it, row0 + NH * kBlk);
+            // Lanes 8 m .. 8 m + 7: the products of k_t and q_t, t = 2 m and 2 m + 1, with all eight k_i, an eighth of the columns
+            // per lane; a reduce-scatter leaves each lane four of them: kind (k or q), t, i = 4 b0 .. + 3.
+            const int sl = lane & 7, m = lane >> 3;
+            float acc[2][2][kBlk];
+#pragma unroll
+            for (int x = 0; x < 4 * kBlk; ++x) (&acc[0][0][0])[x] = 0.f;
+#pragma unroll 1
+            for (int c = 4 * sl; c < DK; c += 32) {
+                float4 y[2][2];
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    y[0][b] = *reinterpret_cast<const float4*>(&ks[2 * m + b][c]);
+                    y[1][b] = *reinterpret_cast<const float4*>(&qs[2 * m + b][c]);
+                }
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i) {
+                    const float4 x = *reinterpret_cast<const float4*>(&ks[i][c]);
+#pragma unroll
+                    for (int kind = 0; kind < 2; ++kind)
+#pragma unroll
+                        for (int b = 0; b < 2; ++b) {
+                            float& z = acc[kind][b][i];
+                            z = fmaf(x.x, y[kind][b].x, z); z = fmaf(x.y, y[kind][b].y, z);
+                            z = fmaf(x.z, y[kind][b].z, z); z = fmaf(x.w, y[kind][b].w, z);
+                        }
+                }
+            }
+            const bool b2 = (sl & 4) != 0, b1 = (sl & 2) != 0, b0 = (sl & 1) != 0;
+            float s2[2][kBlk], s1[kBlk], dot[4];
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i)
+                    s2[b][i] = (b2 ? acc[1][b][i] : acc[0][b][i]) + __shfl_xor_sync(0xffffffffu, b2 ? acc[0][b][i] : acc[1][b][i], 4);
+#pragma unroll
+            for (int i = 0; i < kBlk; ++i) s1[i] = (b1 ? s2[1][i] : s2[0][i]) + __shfl_xor_sync(0xffffffffu, b1 ? s2[0][i] : s2[1][i], 2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) dot[i] = (b0 ? s1[4 + i] : s1[i]) + __shfl_xor_sync(0xffffffffu, b0 ? s1[i] : s1[4 + i], 1);
+            const int kind = sl >> 2, t = 2 * m + ((sl >> 1) & 1), i0 = 4 * (sl & 1);
+            float r[4] = {1.f, 1.f, 1.f, 1.f}, e[4] = {1.f, 1.f, 1.f, 1.f}, gt = 1.f, ge = 1.f;     // R(t, i), R(8, i), G_t, G_8
+#pragma unroll
+            for (int x = 0; x < kBlk; ++x) {
+                const float ax = sm.al[hw][x];
+                if (x <= t) gt *= ax;
+                ge *= ax;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (x > i0 + i) { e[i] *= ax; if (x <= t) r[i] *= ax; }
+            }
+            const float bt = sm.al[hw][kBlk + t];
+            Coef& cf = sm.coef[buf][hw];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int ii = i0 + i;
+                sm.mn[hw][kind][ii][t] = kind ? (ii <= t ? r[i] * dot[i] : 0.f) : (ii < t ? -bt * (r[i] * dot[i]) : 0.f);
+                if (kind == 0 && t == 0) cf.rest[ii] = e[i];
+            }
+            if (i0 == 0) { cf.c1[kind][t] = kind ? 0.f : bt; cf.c2[kind][t] = kind ? gt : -bt * gt; }
+            if (lane == 0) cf.gend = ge;
+            __syncwarp();
+            {
+                // lanes j, j + 8, ..: column j of the inverse, by forward substitution, and two rows of N times it
+                const int j = lane & 7, t0 = lane >> 3;
+                float x[kBlk];
+#pragma unroll
+                for (int t2 = 0; t2 < kBlk; ++t2) x[t2] = t2 == j ? 1.f : 0.f;
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i)
+#pragma unroll
+                    for (int t2 = i + 1; t2 < kBlk; ++t2) x[t2] = fmaf(sm.mn[hw][0][i][t2], x[i], x[t2]);
+                float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i) { o0 = fmaf(sm.mn[hw][1][i][t0], x[i], o0); o1 = fmaf(sm.mn[hw][1][i][t0 + 4], x[i], o1); }
+                cf.A[1][j][t0] = o0; cf.A[1][j][t0 + 4] = o1;
+                if (t0 == 0) {
+#pragma unroll
+                    for (int t2 = 0; t2 < kBlk; ++t2) cf.A[0][j][t2] = t2 == j ? 0.f : x[t2];
+                }
+            }
+            bar_arrive<BAR_FULL>(buf, NTHR);
+        }
+    }
+    for (uint32_t n = stage < kBufs ? 0u : stage - kBufs; n < stage; ++n) bar_sync<BAR_EMPTY>((int)(n % kBufs), NTHR);      // (leave no barrier half arrived)
+}
+
+// ---- compute warp ---------------------------------------------------------------------------------------------
+template <int DK, int DV, typename T, int RPT, int NW, int NH>
+__device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& sm, int sms, int warp, int lane)
+{
+    constexpr int NTHR = (NW + NH) * 32, R = 2 * RPT * NW, SLICES = DV / R, NC = DK / 64;      // NC: 16-byte pieces per lane and row
+    constexpr int TB = 16 / RPT;                          // tokens whose dot products are formed together
+    const int l = lane & 15, rg = lane >> 4;
+    // What the reduce-scatter leaves in this lane: outputs' p (1) or delta's r (0), and which of the RPT rows.  The lane keeps its
+    // rows in the order row, row ^ 1, .. and its dot products in the order own type, other type, so that every step of the
+    // reduction sends and keeps fixed registers (no selects).
+    const int type = l >> 3, row = (l & 7) / (8 / RPT);
+    const bool store_o = type == 1 && (l & (8 / RPT - 1)) == 0;
+    const int wrow = rg * RPT + row;                      // row within the warp
     const T* __restrict__ vg = (const T*)p.v;
     T* __restrict__ og = (T*)p.out_o;
 
-    for (;;) {
-        if (tid == 0) item_s = atomicAdd(&s.header->next_item, 1u);
-        __syncthreads();
-        const uint32_t item = item_s;
-        __syncthreads();
-        if (item >= num_items) break;
-        const int n = s.order[item / p.Hv];
-        const int h = item % p.Hv;
-        const int hq = h / G;
-        const int64_t row_begin = p.cu[n], row_end = p.cu[n + 1];
-        const size_t state_off = ((size_t)n * p.Hv + h) * DK * DV;
-
-        float S[R];
-        if (p.init_state) {
+    uint32_t stage = 0;
+    Item it;
+    for (uint32_t round = 0; more<SLICES>(p, s, sms, round, it); ++round) {
+        const int j0 = it.slice * R + warp * 2 * RPT;     // first row (value index) of the warp
+        const size_t st_off = ((size_t)it.n * p.Hv + it.h) * DK * DV + j0 + rg * RPT;
+        float2 S[RPT][2 * NC];                            // [row ^ r], piece c: columns 64 c + 4 l .. + 3
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int d = part * 4 + (r >> 2) * 4 * TPR + (r & 3);
-                S[r] = p.init_state[state_off + (size_t)d * DV + j];
-            }
-        } else {
+        for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int r = 0; r < R; ++r) S[r] = 0.f;
-        }
-
-        for (int64_t row0 = row_begin; row0 < row_end; row0 += kTokBlock) {
-            const int nvalid = (int)min((int64_t)kTokBlock, row_end - row0);
-            // stage q, k, v, decay and beta of this token block
-            for (int idx = tid; idx < kTokBlock * DK; idx += NT) {
-                const int t = idx / DK, d = idx % DK;
-                float kv = 0.f, qv = 0.f;
-                if (t < nvalid) {
-                    const size_t off = ((size_t)(row0 + t) * p.Hq + hq) * DK + d;
-                    kv = to_f32<T>(kg[off]);
-                    qv = to_f32<T>(qg[off]);
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const float x = p.init_state ? p.init_state[st_off + (size_t)(64 * c + 4 * l + e) * DV + (row ^ r)] : 0.f;
+                    if (e & 1) S[r][2 * c + (e >> 1)].y = x; else S[r][2 * c + (e >> 1)].x = x;
                 }
-                ks[t][d] = kv;
-                qs[t][d] = qv;
-            }
-            for (int idx = tid; idx < kTokBlock * DV; idx += NT) {
-                const int t = idx / DV, d = idx % DV;
-                vs[t][d] = (t < nvalid) ? to_f32<T>(vg[((size_t)(row0 + t) * p.Hv + h) * DV + d]) : 0.f;
-            }
-            if (tid < kTokBlock) {
-                const bool ok = tid < nvalid;
-                const float gin = ok ? p.g[(size_t)(row0 + tid) * p.Hv + h] : 0.f;
-                const float bin = ok ? p.beta[(size_t)(row0 + tid) * p.Hv + h] : 0.f;
-                if (p.input_raw) {
-                    // fused input stage: alpha = sigmoid(gate), beta = sigmoid(pre-activation)
-                    as[tid] = ok ? 1.f / (1.f + expf(-gin)) : 1.f;
-                    bs[tid] = ok ? 1.f / (1.f + expf(-bin)) : 0.f;
-                } else {
-                    as[tid] = ok ? expf(gin) : 1.f;
-                    bs[tid] = bin;
-                }
-            }
-            __syncthreads();
-            if (p.input_raw) {
-                // fused input stage: q and k rows L2-normalised, x / sqrt(sum x^2 + eps)
-                for (int t = warp; t < kTokBlock; t += NT / 32) {
-                    float sk = 0.f, sq = 0.f;
-                    for (int d = lane; d < DK; d += 32) { sk = fmaf(ks[t][d], ks[t][d], sk); sq = fmaf(qs[t][d], qs[t][d], sq); }
+        const size_t vstride = (size_t)p.Hv * DV;
+        const size_t vo = ((size_t)it.row_begin * p.Hv + it.h) * DV + j0 + wrow;
+        T* op = og ? og + vo : nullptr;
+        // this lane's part of the next block's v: VPL rows of token lane / 4
+        constexpr int VPL = RPT / 2;
+        const int vtok = lane >> 2, vrow = VPL * (lane & 3);
+        const T* vp = vg + ((size_t)(it.row_begin + vtok) * p.Hv + it.h) * DV + j0 + vrow;
+        VNext<T, VPL> vn;
+        int left = it.row_end - it.row_begin;             // tokens from the current block on
+        vn.load(vp, vtok < left);
+#pragma unroll 1
+        for (; left > 0; ++stage) {
+            const int buf = (int)(stage % kBufs);
+            bar_sync<BAR_FULL>(buf, NTHR);
+#pragma unroll 1
+            for (int sb = 0; sb < NH && left > 0; ++sb, left -= kBlk) {
+                const float (*ks)[Smem<DK, RPT, NW, NH>::LD] = &sm.k[buf][sb * kBlk];
+                const float (*qs)[Smem<DK, RPT, NW, NH>::LD] = &sm.q[buf][sb * kBlk];
+                const Coef& cf = sm.coef[buf][sb];
 #pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        sk += __shfl_xor_sync(0xffffffffu, sk, off);
-                        sq += __shfl_xor_sync(0xffffffffu, sq, off);
+                for (int i = 0; i < VPL; ++i) sm.v[warp][vtok][vrow + i] = vn.get(i);
+                vp += kBlk * vstride;
+                vn.load(vp, vtok < left - kBlk);
+                __syncwarp();
+                float y[kBlk];
+                float Areg[RPT == 2 ? kBlk * kBlk : 1], rreg[RPT == 2 ? kBlk : 1];
+                if constexpr (RPT == 2) {
+                    // few warps: the coefficients are fetched ahead, so that their latency passes under the dot products
+#pragma unroll
+                    for (int i = 0; i < kBlk; ++i) {
+#pragma unroll
+                        for (int t = i; t < kBlk; ++t) Areg[i * kBlk + t] = cf.A[type][i][t];
+                        rreg[i] = cf.rest[i];
                     }
-                    const float rk = rsqrtf(sk + kNormEps), rq = rsqrtf(sq + kNormEps);
-                    for (int d = lane; d < DK; d += 32) { ks[t][d] *= rk; qs[t][d] *= rq; }
-                }
-                __syncthreads();
-            }
-            for (int t = warp; t < kTokBlock; t += NT / 32) {
-                float acc = 0.f;
-                for (int d = lane; d < DK; d += 32) acc = fmaf(ks[t][d], qs[t][d], acc);
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (lane == 0) kqs[t] = acc;
-            }
-            __syncthreads();
-
-            for (int tt = 0; tt < nvalid; ++tt) {
-                const float a = as[tt], b = bs[tt];
-                float r = 0.f, pq = 0.f;
+                    for (int i = 0; i < kBlk; ++i) asm volatile("" ::"f"(Areg[i * kBlk + i]), "f"(Areg[i * kBlk + kBlk - 1]), "f"(rreg[i]));
+                }
+                const float* const A = RPT == 2 ? Areg : &cf.A[type][0][0];
+                const float* const rest = RPT == 2 ? rreg : cf.rest;
+                // r_t, p_t of TB tokens at a time: products of all, then the reductions side by side
+                const float (*own)[Smem<DK, RPT, NW, NH>::LD] = type ? qs : ks, (*oth)[Smem<DK, RPT, NW, NH>::LD] = type ? ks : qs;
 #pragma unroll
-                for (int i = 0; i < R / 4; ++i) {
-                    const float4 k4 = *reinterpret_cast<const float4*>(&ks[tt][part * 4 + i * 4 * TPR]);
-                    const float4 q4 = *reinterpret_cast<const float4*>(&qs[tt][part * 4 + i * 4 * TPR]);
-                    r = fmaf(S[4 * i + 0], k4.x, r); pq = fmaf(S[4 * i + 0], q4.x, pq);
-                    r = fmaf(S[4 * i + 1], k4.y, r); pq = fmaf(S[4 * i + 1], q4.y, pq);
-                    r = fmaf(S[4 * i + 2], k4.z, r); pq = fmaf(S[4 * i + 2], q4.z, pq);
-                    r = fmaf(S[4 * i + 3], k4.w, r); pq = fmaf(S[4 * i + 3], q4.w, pq);
-                }
+                for (int t0 = 0; t0 < kBlk; t0 += TB) {
+                    float2 a[TB][2][RPT];                 // [token][own type, other type][row]
 #pragma unroll
-                for (int off = 1; off < TPR; off <<= 1) {
-                    r += __shfl_xor_sync(0xffffffffu, r, off);
-                    pq += __shfl_xor_sync(0xffffffffu, pq, off);
-                }
-                const float delta = b * (vs[tt][j] - a * r);
+                    for (int x = 0; x < TB; ++x)
 #pragma unroll
-                for (int i = 0; i < R / 4; ++i) {
-                    const float4 k4 = *reinterpret_cast<const float4*>(&ks[tt][part * 4 + i * 4 * TPR]);
-                    S[4 * i + 0] = fmaf(a, S[4 * i + 0], delta * k4.x);
-                    S[4 * i + 1] = fmaf(a, S[4 * i + 1], delta * k4.y);
-                    S[4 * i + 2] = fmaf(a, S[4 * i + 2], delta * k4.z);
-                    S[4 * i + 3] = fmaf(a, S[4 * i + 3], delta * k4.w);
+                        for (int r = 0; r < RPT; ++r) { a[x][0][r] = make_float2(0.f, 0.f); a[x][1][r] = make_float2(0.f, 0.f); }
+#pragma unroll
+                    for (int c = 0; c < NC; ++c)
+#pragma unroll
+                        for (int x = 0; x < TB; ++x) {
+                            const float4 u = *reinterpret_cast<const float4*>(&own[t0 + x][64 * c + 4 * l]);
+                            const float4 w = *reinterpret_cast<const float4*>(&oth[t0 + x][64 * c + 4 * l]);
+                            // (one multiplicand stays the same from instruction to instruction: with three new 64-bit operands each, the
+                            // register file would feed the pipe every third cycle only)
+#pragma unroll
+                            for (int r = 0; r < RPT; ++r) fma_f32x2_here(a[x][0][r], S[r][2 * c], u.x, u.y);
+#pragma unroll
+                            for (int r = 0; r < RPT; ++r) fma_f32x2_here(a[x][1][r], S[r][2 * c], w.x, w.y);
+#pragma unroll
+                            for (int r = 0; r < RPT; ++r) fma_f32x2_here(a[x][0][r], S[r][2 * c + 1], u.z, u.w);
+#pragma unroll
+                            for (int r = 0; r < RPT; ++r) fma_f32x2_here(a[x][1][r], S[r][2 * c + 1], w.z, w.w);
+                        }
+                    float z[TB][RPT];
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                        for (int x = 0; x < TB; ++x)
+                            z[x][r] = (a[x][0][r].x + a[x][0][r].y) + __shfl_xor_sync(0xffffffffu, a[x][1][r].x + a[x][1][r].y, 8);
+#pragma unroll
+                    for (int h = RPT / 2; h > 0; h >>= 1)
+#pragma unroll
+                        for (int r = 0; r < h; ++r)
+#pragma unroll
+                            for (int x = 0; x < TB; ++x) z[x][r] += __shfl_xor_sync(0xffffffffu, z[x][r + h], h * (8 / RPT));
+#pragma unroll
+                    for (int o = 4 / RPT; o > 0; o >>= 1)
+#pragma unroll
+                        for (int x = 0; x < TB; ++x) z[x][0] += __shfl_xor_sync(0xffffffffu, z[x][0], o);
+#pragma unroll
+                    for (int x = 0; x < TB; ++x)
+                        y[t0 + x] = fmaf(cf.c2[type][t0 + x], z[x][0], cf.c1[type][t0 + x] * sm.v[warp][t0 + x][wrow]);
                 }
-                if (part == 0) os[tt][j] = fmaf(a, pq, delta * kqs[tt]);
-            }
-            __syncthreads();
-            if (og) {
-                for (int idx = tid; idx < nvalid * DV; idx += NT) {
-                    const int t = idx / DV, d = idx % DV;
-                    og[((size_t)(row0 + t) * p.Hv + h) * DV + d] = from_f32<T>(os[t][d]);
+                // delta in the lanes of type 0, the outputs in those of type 1: both from the eight y of the row
+                float e[kBlk];
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i) e[i] = __shfl_sync(0xffffffffu, y[i], lane & ~8);
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i)
+#pragma unroll
+                    for (int t = i; t < kBlk; ++t) y[t] = fmaf(A[i * kBlk + t], e[i], y[t]);
+                if (l % (8 / RPT) == 0 && type == 0) {
+#pragma unroll
+                    for (int i = 0; i < kBlk; ++i) sm.dr[warp][i][wrow] = y[i] * rest[i];
                 }
+                __syncwarp();
+                if (og) {
+                    if (store_o) {
+#pragma unroll
+                        for (int t = 0; t < kBlk; ++t)
+                            if (t < left) op[t * vstride] = from_f32<T>(y[t]);
+                    }
+                    op += kBlk * vstride;
+                }
+                // S = G_8 S + sum_i R(8, i) delta_i k_i^T
+                const float ge = cf.gend;
+#pragma unroll
+                for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                    for (int c = 0; c < 2 * NC; ++c) mul_f32x2(S[r][c].x, S[r][c].y, ge, ge);
+#pragma unroll 4
+                for (int i = 0; i < kBlk; ++i) {
+                    float dv[RPT];
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r) dv[r] = sm.dr[warp][i][rg * RPT + (row ^ r)];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const float4 k4 = *reinterpret_cast<const float4*>(&ks[i][64 * c + 4 * l]);
+#pragma unroll
+                        for (int r = 0; r < RPT; ++r) fma_f32x2_here(S[r][2 * c], make_float2(dv[r], dv[r]), k4.x, k4.y);
+#pragma unroll
+                        for (int r = 0; r < RPT; ++r) fma_f32x2_here(S[r][2 * c + 1], make_float2(dv[r], dv[r]), k4.z, k4.w);
+                    }
+                }
+                __syncwarp();                             // the scratch may be overwritten
             }
-            __syncthreads();
+            bar_arrive<BAR_EMPTY>(buf, NTHR);
         }
-
         if (p.out_state) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int d = part * 4 + (r >> 2) * 4 * TPR + (r & 3);
-                p.out_state[state_off + (size_t)d * DV + j] = S[r];
-            }
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r)
+                        p.out_state[st_off + (size_t)(64 * c + 4 * l + e) * DV + (row ^ r)] = (e & 1) ? S[r][2 * c + (e >> 1)].y : S[r][2 * c + (e >> 1)].x;
         }
     }
 }
 
-template <int DK, int DV, typename T>
-static cudaError_t launch_one(const Problem& p, const Sched& s, cudaStream_t stream)
+template <int DK, int DV, typename T, int RPT, int NW, int NH>
+__global__ void __launch_bounds__((NW + NH) * 32, 2)
+gdn_simt_kernel(const Problem p, const Sched s, const int sms)
 {
-    constexpr int NT = DV * (DK / 32);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gdn_simt_kernel<DK, DV, T>, NT, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    const long long items = (long long)p.num_seqs * p.Hv;
-    long long grid = (long long)sms * per_sm;
-    if (grid > items) grid = items;
-    if (grid < 1) grid = 1;
-    gdn_simt_kernel<DK, DV, T><<<(unsigned)grid, NT, 0, stream>>>(p, s);
+    extern __shared__ __align__(16) uint8_t raw[];
+    Smem<DK, RPT, NW, NH>& sm = *reinterpret_cast<Smem<DK, RPT, NW, NH>*>(raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < NW) compute<DK, DV, T, RPT, NW, NH>(p, s, sm, sms, warp, lane);
+    else helper<DK, DV / (2 * RPT * NW), T, RPT, NW, NH>(p, s, sm, sms, warp - NW, lane);
+}
+
+template <int DK, int DV, typename T, int RPT, int NW, int NH>
+cudaError_t launch_one(const Problem& p, const Sched& s, int dev, int sms, cudaStream_t stream)
+{
+    constexpr int NTHR = (NW + NH) * 32, SMEM = (int)sizeof(Smem<DK, RPT, NW, NH>);
+    static int per_sm[64] = {};                          // resident CTAs per SM; found on the first call per device
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (per_sm[dev] == 0) {
+        cudaError_t e = cudaFuncSetAttribute(gdn_simt_kernel<DK, DV, T, RPT, NW, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        int n = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gdn_simt_kernel<DK, DV, T, RPT, NW, NH>, NTHR, SMEM);
+        if (e != cudaSuccess) return e;
+        per_sm[dev] = n > 0 ? n : 1;
+    }
+    const long long items = (long long)p.num_seqs * p.Hv * (DV / (2 * RPT * NW));
+    long long per = (items + sms - 1) / sms;
+    if (per > per_sm[dev]) per = per_sm[dev];
+    const long long grid = items < sms ? (items > 0 ? items : 1) : per * sms;
+    gdn_simt_kernel<DK, DV, T, RPT, NW, NH><<<(unsigned)grid, NTHR, SMEM, stream>>>(p, s, sms);
     return cudaGetLastError();
 }
+
+template <int DK, int DV, typename T>
+cudaError_t launch_shape(const Problem& p, const Sched& s, cudaStream_t stream)
+{
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // Rows per warp: 16 have the lowest cost per row, 8 and 4 the lowest time per token.  The finer splits pay while they find idle
+    // SMs: 4 rows (16 per CTA) up to one CTA per SM, 8 (32 per CTA) up to one and a half.  us for 1,000 tokens at d = 128:
+    // 1,024 rows 138 / 193 / 282 (4 / 8 / 16 rows a warp), 4,096 rows 358 / 195 / 279, 8,192 rows 714 / 305 / 281.
+    const long long rows = (long long)p.num_seqs * p.Hv * DV;
+    if (rows > 48ll * sms) return launch_one<DK, DV, T, 8, 4, 2>(p, s, dev, sms, stream);
+    if (rows > 16ll * sms) return launch_one<DK, DV, T, 4, 4, 2>(p, s, dev, sms, stream);
+    return launch_one<DK, DV, T, 2, 2, 4>(p, s, dev, sms, stream);
+}
+
+}  // namespace
 
 cudaError_t launch_simt(const Problem& p, const Sched& s, int io_dtype, cudaStream_t stream, int* launches)
 {
     cudaError_t e = cudaErrorNotSupported;
 #define GDN_SIMT_CASE(DKV, DVV)                                                           \
     if (p.dk == DKV && p.dv == DVV)                                                       \
-        e = (io_dtype == GDN_BF16) ? launch_one<DKV, DVV, __nv_bfloat16>(p, s, stream)    \
-                                   : launch_one<DKV, DVV, float>(p, s, stream);
+        e = (io_dtype == GDN_BF16) ? launch_shape<DKV, DVV, __nv_bfloat16>(p, s, stream)  \
+                                   : launch_shape<DKV, DVV, float>(p, s, stream);
     GDN_SIMT_CASE(64, 64)
     GDN_SIMT_CASE(64, 128)
     GDN_SIMT_CASE(128, 64)
