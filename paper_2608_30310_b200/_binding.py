@@ -1,4 +1,4 @@
-"""ctypes binding of libgdn_tail_replay.so: argument marshalling only."""
+"""Binding of libgdn_tail_replay.so: argument marshalling only (csrc/native.cpp, with ctypes as the general path)."""
 from __future__ import annotations
 
 import ctypes
@@ -8,6 +8,7 @@ from typing import Optional
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "libgdn_tail_replay.so")
 _lib = None
+_native = None
 
 GDN_OK = 0
 GDN_F32, GDN_BF16 = 0, 1
@@ -69,8 +70,19 @@ def load_library():
     lib.gdn_last_launch_count.argtypes = []
     lib.gdn_test_hooks.restype = None
     lib.gdn_test_hooks.argtypes = [ctypes.c_uint64, ctypes.c_int32]
+    _bind_native(lib)
     _lib = lib
     return lib
+
+
+def _bind_native(lib):
+    """The extension that checks and marshals a call's tensors; it takes the library's entry points by address."""
+    global _native
+    import torch  # noqa: F401  (its libraries first)
+    from . import _native as ext
+    ext.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in
+               ("gdn_tail_replay", "gdn_full_prefill", "gdn_tail_replay_static_scratch", "gdn_decode_step", "gdn_workspace_size")))
+    _native = ext
 
 
 def status_string(status: int) -> str:
@@ -170,6 +182,27 @@ def _forward(fn_name, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, *
     return rc
 
 
+_ENTRIES = ("gdn_tail_replay", "gdn_full_prefill", "gdn_tail_replay_static_scratch")
+
+
+def _call(which, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, *, total_tokens=None, init_state=None, workspace=None,
+          status_word=None, kernel=GDN_KERNEL_AUTO, stream=None, check=True, raw_inputs=False) -> int:
+    """One forward call: marshalled natively where the arguments are in order, else by _forward (errors, workspace growth)."""
+    if _native is None:
+        load_library()
+    rc = None
+    if total_tokens is None:
+        rc = _native.forward(which, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, init_state, workspace, status_word,
+                             kernel, stream, raw_inputs)
+    if rc is None:
+        return _forward(_ENTRIES[which], q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, total_tokens=total_tokens,
+                        init_state=init_state, workspace=workspace, status_word=status_word, kernel=kernel, stream=stream,
+                        check=check, raw_inputs=raw_inputs)
+    if rc != GDN_OK and check:
+        raise GdnError(rc, _ENTRIES[which])
+    return rc
+
+
 def gdn_tail_replay(q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw) -> int:
     """Tail replay (paper Eq. 2) on torch tensors; see include/gdn_tail_replay.h for layouts.
 
@@ -178,7 +211,7 @@ def gdn_tail_replay(q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **k
     (or given) stream.  Keyword arguments: init_state, workspace, status_word, kernel, stream,
     check, raw_inputs (q, k, g, beta are raw projection outputs: the fused input stage of the header).
     """
-    return _forward("gdn_tail_replay", q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
+    return _call(0, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
 
 
 def gdn_tail_replay_static_scratch(q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw) -> int:
@@ -187,12 +220,12 @@ def gdn_tail_replay_static_scratch(q, k, v, g, beta, cu_tail_lens, chunk, out_o,
     no workspace and creates no tensor).  Device tensors only, at most 4096 requests per call, and calls
     must not overlap on the GPU because they all share that one array.  Make the first call on a device
     outside any stream capture: it looks up the array's address once."""
-    return _forward("gdn_tail_replay_static_scratch", q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
+    return _call(2, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
 
 
 def gdn_full_prefill(q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw) -> int:
     """Full prefill (paper Eq. 1 over whole prefixes); same arguments as ``gdn_tail_replay``."""
-    return _forward("gdn_full_prefill", q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
+    return _call(1, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, **kw)
 
 
 def gdn_decode_step(q, k, v, g, beta, state_in, out_o, state_out, *, stream=None, check: bool = True) -> int:
@@ -200,6 +233,13 @@ def gdn_decode_step(q, k, v, g, beta, state_in, out_o, state_out, *, stream=None
 
     q, k [N, Hq, dk], v [N, Hv, dv], g, beta [N, Hv], state_in / state_out [N, Hv, dk, dv] fp32 (may be the
     same tensor), out_o [N, Hv, dv] or None.  Device tensors only."""
+    if _native is None:
+        load_library()
+    rc = _native.decode(q, k, v, g, beta, state_in, out_o, state_out, stream)
+    if rc is not None:
+        if rc != GDN_OK and check:
+            raise GdnError(rc, "gdn_decode_step")
+        return rc
     import torch
     lib = load_library()
     N, Hq, dk = q.shape

@@ -16,16 +16,39 @@ NVCC_FLAGS = [
 ]
 
 
+NATIVE = os.path.join(PKG, "_native.so")
+NATIVE_SRC = os.path.join(CSRC, "native.cpp")
+
+
+def build_native(force: bool = False) -> str:
+    """Compile the binding's argument path (a CPython extension on torch's C++ tensors; host code only)."""
+    deps = [NATIVE_SRC, os.path.join(ROOT, "include", "gdn_tail_replay.h")]
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
+        return NATIVE
+    import sysconfig
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    inc = [x for d in include_paths("cuda") + [sysconfig.get_paths()["include"]] for x in ("-isystem", d)]
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+                           *inc, NATIVE_SRC, "-o", tmp, "-L" + lib, "-Wl,-rpath," + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "gdn_tail_replay.h"), __file__]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "native.cpp"] + [os.path.join(ROOT, "include", "gdn_tail_replay.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into libgdn_tail_replay.so (objects under build/)."""
+    """Compile every .cu under csrc/ into libgdn_tail_replay.so (objects under build/), and the binding's extension."""
+    build_native(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
