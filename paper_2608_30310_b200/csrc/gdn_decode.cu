@@ -47,6 +47,8 @@ gdn_decode_kernel(const DecodeArgs a)
     const float* Hin = a.state_in + (size_t)chain * DK * DV;      // may be the same memory as Hout: every thread
     float* Hout = a.state_out + (size_t)chain * DK * DV;          // writes only the entries it has read itself
 
+    allow_successor();
+    wait_for_predecessor();
     // the state first: these loads are the kernel
     float4 Hr[RPT];
 #pragma unroll
@@ -104,9 +106,8 @@ template <int DK, int DV>
 static cudaError_t launch_dtype(const DecodeArgs& a, int io_dtype, cudaStream_t stream)
 {
     const unsigned grid = (unsigned)a.num_seqs * (unsigned)a.Hv;
-    if (io_dtype == GDN_BF16) gdn_decode_kernel<DK, DV, __nv_bfloat16><<<grid, 256, 0, stream>>>(a);
-    else gdn_decode_kernel<DK, DV, float><<<grid, 256, 0, stream>>>(a);
-    return cudaGetLastError();
+    if (io_dtype == GDN_BF16) return launch_kernel(gdn_decode_kernel<DK, DV, __nv_bfloat16>, grid, 256, 0, stream, 1, a);
+    return launch_kernel(gdn_decode_kernel<DK, DV, float>, grid, 256, 0, stream, 1, a);
 }
 
 cudaError_t launch_decode(const void* q, const void* k, const void* v, const float* g, const float* beta,

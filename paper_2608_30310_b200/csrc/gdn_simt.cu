@@ -481,8 +481,10 @@ gdn_simt_kernel(const Problem p, const Sched s, const int sms)
     extern __shared__ __align__(16) uint8_t raw[];
     Smem<DK, RPT, NW, NH>& sm = *reinterpret_cast<Smem<DK, RPT, NW, NH>*>(raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_for_predecessor();
     if (warp < NW) compute<DK, DV, T, RPT, NW, NH>(p, s, sm, sms, warp, lane);
     else helper<DK, DV / (2 * RPT * NW), T, RPT, NW, NH>(p, s, sm, sms, warp - NW, lane);
+    allow_successor();       // at the end: a successor's blocks placed among this kernel's would land on the SMs in another order
 }
 
 template <int DK, int DV, typename T, int RPT, int NW, int NH>
@@ -502,8 +504,7 @@ cudaError_t launch_one(const Problem& p, const Sched& s, int dev, int sms, cudaS
     long long per = (items + sms - 1) / sms;
     if (per > per_sm[dev]) per = per_sm[dev];
     const long long grid = items < sms ? (items > 0 ? items : 1) : per * sms;
-    gdn_simt_kernel<DK, DV, T, RPT, NW, NH><<<(unsigned)grid, NTHR, SMEM, stream>>>(p, s, sms);
-    return cudaGetLastError();
+    return launch_kernel(gdn_simt_kernel<DK, DV, T, RPT, NW, NH>, (unsigned)grid, NTHR, SMEM, stream, 1, p, s, sms);
 }
 
 template <int DK, int DV, typename T>

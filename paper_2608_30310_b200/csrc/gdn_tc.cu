@@ -1331,6 +1331,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     cx.sm = smem_raw + (cx.sb - raw);
     cx.misc = reinterpret_cast<Misc*>(cx.sm + SM_MISC);
     const uint32_t rank = CL ? blockIdx.x % prm.csize : 0u;
+    if (CL) allow_successor();                // (many chains: at the end, see below)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (!CL) {
@@ -1373,6 +1374,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     }
     tc_fence_before();
     __syncthreads();
+    wait_for_predecessor();
     if (CL) cluster_sync_all();               // every CTA's barriers exist before another CTA arrives on them
     tc_fence_after();
     cx.tmem = cx.misc->tmem_base;
@@ -1399,6 +1401,8 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
         else if (warp >= 16 && warp < 16 + (int)NT) prep_sender<RAW>(cx, &prm, rank, (uint32_t)warp - 16u);
     }
 
+    // A successor's CTAs take the SMs of chains that end early; with many chains that costs more than its start-up gains.
+    if (!CL) allow_successor();
     tc_fence_before();
     __syncthreads();
     if (cx.misc->abort) {
@@ -1476,13 +1480,7 @@ template <bool RAW, bool CL>
 cudaError_t launch_as(TcParams& prm, uint32_t csize, long long groups, Maps& m, cudaStream_t stream)
 {
     prm.csize = csize;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = (unsigned)groups * csize;
-    cfg.blockDim = kThreads<CL>; cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = CL ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, gdn_tc_kernel<RAW, CL>, (const TcParams)prm, m.q, m.k, m.v, m.o, m.qt, m.kt);
+    return launch_kernel(gdn_tc_kernel<RAW, CL>, (unsigned)groups * csize, kThreads<CL>, SMEM_BYTES, stream, csize, prm, m.q, m.k, m.v, m.o, m.qt, m.kt);
 }
 template <bool RAW>
 cudaError_t launch(TcParams& prm, Maps& m, cudaStream_t stream)
