@@ -84,11 +84,11 @@ enum ChainBar {
 enum FusedBar {
     FB_KQ_FULL0 = 0, FB_KQ_FREE0 = 4, FB_V_FULL = 8, FB_U0, FB_GRAM0 = FB_U0 + 2, FB_W0 = FB_GRAM0 + 2, FB_OPS0 = FB_W0 + 2, FB_MMA1_0 = FB_OPS0 + 2,
     FB_STATE0 = FB_MMA1_0 + 2, FB_OUT = FB_STATE0 + 2, FB_DONE0, FB_ACC_FREE = FB_DONE0 + 4, FB_DECAY_READY0, FB_DECAY_FREE0 = FB_DECAY_READY0 + 4,
-    FB_NUM = FB_DECAY_FREE0 + 4
+    FB_TACC_FREE0 = FB_DECAY_FREE0 + 4, FB_NUM = FB_TACC_FREE0 + 2
 };
 enum PrepBar {
     PB_KQ_FULL0 = 0, PB_GRAM0 = 3, PB_W0 = 6, PB_OPS0 = 9, PB_SENT0 = 12, PB_DECAY_READY0 = 15, PB_DECAY_FREE0 = 19, PB_CREDIT0 = 23,
-    PB_NUM = PB_CREDIT0 + NT
+    PB_TACC_FREE0 = PB_CREDIT0 + NT, PB_NUM = PB_TACC_FREE0 + NT
 };
 
 // Per-chunk factors.  The fp32 state lives in tensor memory divided by a running factor c (the product of the chunk decays
@@ -114,7 +114,9 @@ struct PrepMisc { PrepDecay decay[4]; };
 // Fused CTA: both in one record.  eGk: eG times the key norms (fused input stage)
 struct __align__(16) FusedDecay { float G2[64], beta[64], eG[64], colfb[32], norms[128]; float G2mid, wb, cfin; int rescale; float bRest[64], eGk[64]; };
 struct FusedMisc { FusedDecay decay[4]; };
+constexpr int kChainTable = 64;
 struct Misc {
+    int4 chains[kChainTable];          // the CTA's (cluster's) first work items, see chain_entry
     unsigned long long bars[40];
     uint32_t tmem_base;
     volatile uint32_t abort;
@@ -150,10 +152,12 @@ template <bool CL> __device__ __forceinline__ uint32_t tm_acc2(uint32_t j) { ret
 template <bool CL> __device__ __forceinline__ uint32_t tm_acc3(uint32_t j) { return CL ? TM_ACC3 + (j & 1u) * 64 : TM_F_ACC3; }
 
 constexpr uint32_t ID_GRAM = idesc_bf16(128, 64, 0, 0, 0);    // [K;Q] (K-major) x K (K-major)
-constexpr uint32_t ID_WU = idesc_bf16(128, 64, 1, 0, 0);      // K^T or V^T (M-major) x T (K-major)
+constexpr uint32_t id_wu(int N) { return idesc_bf16(128, N, 1, 0, 0); }      // K^T or V^T (M-major) x T (K-major)
 constexpr uint32_t ID_SW = idesc_bf16(128, 64, 0, 1, 1);      // -S0 (TMEM) x W^T (N-major)
 constexpr uint32_t ID_SQ = idesc_bf16(128, 64, 0, 0, 0);      // S0 (TMEM) x Q (K-major)
-constexpr uint32_t ID_DP = idesc_bf16(128, 64, 0, 0, 0);      // Delta^T (TMEM) x P (K-major)
+constexpr uint32_t id_dp(int N) { return idesc_bf16(128, N, 0, 0, 0); }      // Delta^T (TMEM) x P (K-major)
+// T', T'' and P are lower triangular: the product's step over columns s .. s + 15 takes rows t >= s only (N = 64 - s), so that
+// nothing above the 16 x 16 diagonal blocks is read.
 constexpr uint32_t ID_DK = idesc_bf16(128, 64, 0, 1, 0);      // Delta'^T (TMEM) x half of K (N-major)
 
 struct TcParams {
@@ -166,56 +170,41 @@ struct TcParams {
                                   // to one team, so that no wait looks more than one phase ahead
 };
 
-// Walks the chunk sequence of one cluster: chains dealt in snake order over the longest-first list,
-// chunks of 64 rows inside each chain.  Every role keeps its own cursor(s).
+// Work item of round r of this cluster: chains dealt in snake order over the longest-first list.  x = first row, y = end row,
+// z = v-head | q/k head << 16, w = request, or -1 when the items are exhausted.
+__device__ __noinline__ int4 load_chain_entry(const TcParams* prm, int r)
+{
+    const Problem& p = prm->p;
+    const uint32_t G = gridDim.x / prm->csize, b = blockIdx.x / prm->csize;
+    const uint32_t item = (uint32_t)r * G + ((r & 1) ? (G - 1 - b) : b);
+    if (item >= (uint32_t)p.num_seqs * (uint32_t)p.Hv) return make_int4(0, 0, 0, -1);
+    const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);   // no order list: requests as given
+    const int h = item % p.Hv;
+    return make_int4(p.cu[n], p.cu[n + 1], h | ((h / (p.Hv / p.Hq)) << 16), n);
+}
+// The same from shared memory, where the first kChainTable of them are put at the start of the kernel, side by side: divisions and
+// three dependent loads from global memory, some 1,500 cycles that every role would otherwise spend at every chain.
+__device__ __noinline__ int4 chain_entry(const TcParams* prm, const Misc* misc, int r)
+{
+    return r < kChainTable ? misc->chains[r] : load_chain_entry(prm, r);
+}
+// Walks the chunk sequence of one cluster: its chains, chunks of 64 rows inside each chain.  Every role keeps its own cursor(s).
 struct ChunkCursor {
     const TcParams* prm;
+    const Misc* misc;
     int r, h, hq, row_begin, row_end, nchunks, c;
     bool valid;
 
-    __device__ void init(const TcParams* pp)
+    __device__ void init(const TcParams* pp, const Misc* m)
     {
-        prm = pp; r = -1;
+        prm = pp; misc = m; r = -1;
         next_chain();
-    }
-    __device__ static uint32_t item_of(const TcParams* prm, int round)
-    {
-        const uint32_t G = gridDim.x / prm->csize, b = blockIdx.x / prm->csize;
-        return (uint32_t)round * G + ((round & 1) ? (G - 1 - b) : b);
-    }
-    // The next work item of this cluster after round r that has at least one chunk, kept out of line (integer divisions,
-    // dependent global loads and a loop over empty requests, needed once per chain by every role; everything goes and
-    // comes back in registers): x = first row, y = end row, z = v-head | q/k head << 16, w = its round, or -1 when
-    // the cluster's items are exhausted.
-    __device__ __noinline__ static int4 find_chain(const TcParams* prm, int r)
-    {
-        const Problem& p = prm->p;
-        const uint32_t num_items = (uint32_t)p.num_seqs * (uint32_t)p.Hv;
-        for (;;) {
-            ++r;
-            const uint32_t item = item_of(prm, r);
-            if (item >= num_items) return make_int4(0, 0, 0, -1);
-            const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);   // no order list: requests as given
-            const int h = item % p.Hv;
-            const int hq = h / (p.Hv / p.Hq);
-            const int a = p.cu[n], b = p.cu[n + 1];
-            if (b - a > 0) return make_int4(a, b, h | (hq << 16), r);
-        }
-    }
-    // Row range and heads of one work item: x = first row, y = end row, z = v-head | q/k head << 16, w = request index.
-    __device__ __noinline__ static int4 lookup(const TcParams* prm, uint32_t item)
-    {
-        const Problem& p = prm->p;
-        const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);
-        const int h = item % p.Hv;
-        const int hq = h / (p.Hv / p.Hq);
-        return make_int4(p.cu[n], p.cu[n + 1], h | (hq << 16), n);
     }
     // moves to the next chain that has at least one chunk
     __device__ void next_chain()
     {
-        const int4 ci = find_chain(prm, r);
-        r = ci.w;
+        int4 ci;
+        do { ci = chain_entry(prm, misc, ++r); } while (ci.w >= 0 && ci.y <= ci.x);
         valid = ci.w >= 0;
         row_begin = ci.x; row_end = ci.y; h = ci.z & 0xffff; hq = ci.z >> 16;
         nchunks = (row_end - row_begin + 63) >> 6;
@@ -246,8 +235,9 @@ struct Ctx {
     // Bounded wait.  On expiry it raises the CTA-wide abort flag; from then on no wait blocks any more, so
     // every role still runs through its (data-independent) loop structure, keeps meeting its named
     // barriers and reaches the end of the kernel; the results are garbage and the host sees the status word.
-    // (A ready barrier costs a few cycles; a try_wait that has to wait suspends the warp in hardware, without polling, and
-    // returns about 90 cycles after the last arrival.)
+    // A ready barrier costs a few cycles, a try_wait that has to wait returns about 90 cycles after the last arrival.  It does not
+    // sleep all that time: waiting warps poll, and half of the instructions of a fused CTA were polls.  There, one warp of a
+    // group waits for the group, and the others at a named barrier, which does sleep.
     __device__ __forceinline__ void wait(int i, uint32_t parity) const
     {
         const uint32_t b = bar(i);
@@ -257,7 +247,8 @@ struct Ctx {
     __device__ __noinline__ static void wait_slow(uint32_t b, uint32_t parity, Misc* misc)
     {
         uint64_t t0 = 0;
-        while (!mbar_try_wait(b, parity)) {
+        for (uint32_t n = 0; !mbar_try_wait(b, parity); ++n) {
+            if ((n & 15u) != 0u) continue;
             if (misc->abort) return;
             const uint64_t t = globaltimer_ns();
             if (t0 == 0) t0 = t;
@@ -412,10 +403,10 @@ __device__ __forceinline__ TokenLoad load_tokens(const Problem& p, const ChunkCu
 // G_C, c_prev, c, rescale)
 // The loads run three chunks ahead (strided 4-byte loads from DRAM take up to 2,000 cycles, a chunk takes 1,500).
 template <bool RAW, typename F>
-__device__ __forceinline__ void walk_decays(const TcParams* prm, int lane, F publish)
+__device__ __forceinline__ void walk_decays(const Ctx& cx, const TcParams* prm, int lane, F publish)
 {
     ChunkCursor cc, cl;                                       // current chunk, next chunk to load
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     cl = cc;
     float c = 1.f;
     TokenLoad t0 = {}, t1 = {}, t2 = {};
@@ -450,7 +441,7 @@ __device__ void prep_producer(const Ctx& cx, const TcParams* prm, uint32_t rank,
 {
     const int R = (int)prm->csize - 1;
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     cc.advance((int)rank - 1);
 #pragma unroll 1
     for (uint32_t i = 0; cc.valid && !cx.stop(); ++i, cc.advance(R)) {
@@ -469,7 +460,7 @@ __device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, u
 {
     const uint32_t R = prm->csize - 1, own = prm->ring / R;            // ring slots of this CTA (kRingSlots / 3 or kRingSlotsPair)
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     cc.advance((int)(rank - 1 + team * R));
     uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
 #pragma unroll 1
@@ -497,7 +488,7 @@ __device__ void prep_decay(const Ctx& cx, const TcParams* prm, uint32_t rank, in
 {
     const uint32_t R = prm->csize - 1;
     uint32_t i = 0;
-    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float, float, float cprev, float, bool) {
+    walk_decays<RAW>(cx, prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float, float, float cprev, float, bool) {
         if (j % R != rank - 1) return;
         if (i >= 4) cx.wait(PB_DECAY_FREE0 + (int)(i & 3u), ((i >> 2) - 1u) & 1u);
         PrepDecay& dc = cx.misc->p.decay[i & 3u];
@@ -512,6 +503,36 @@ __device__ void prep_decay(const Ctx& cx, const TcParams* prm, uint32_t rank, in
         warp_arrive(cx.bar(PB_DECAY_READY0 + (int)(i & 3u)), lane);
         ++i;
     });
+}
+
+// One warp issues the Gram products of all teams, as soon as a chunk's tiles are there and the team's accumulator is free: issuing
+// takes a warp some 500 cycles, which a team's own warp would add to the way of its chunk.
+template <bool CL>
+__device__ void gram_issuer(const Ctx& cx, const TcParams* prm, uint32_t rank)
+{
+    const uint32_t R = CL ? prm->csize - 1 : 1u, NTEAM = CL ? NT : 2u;
+    ChunkCursor cc;
+    cc.init(prm, cx.misc);
+    if (CL) cc.advance((int)rank - 1);
+    const bool leader = elect_one();
+#pragma unroll 1
+    for (uint32_t i = 0; cc.valid; ++i, cc.advance((int)R)) {
+        const uint32_t team = i % NTEAM, use = i / NTEAM, o = CL ? team * P_TEAM : F_KQ + (i & 3u) * 32768;
+        const uint32_t tm = cx.tmem + (CL ? team * TM_TEAM + TM_GRAM : TM_F_TEAM + team * 64);
+        cx.wait(CL ? PB_KQ_FULL0 + (int)team : FB_KQ_FULL0 + (int)(i & 3u), CL ? use & 1u : (i >> 2) & 1u);
+        if (use >= 1) cx.wait((CL ? PB_TACC_FREE0 : FB_TACC_FREE0) + (int)team, (use - 1) & 1u);
+        tc_fence_after();
+        if (leader) {
+            const uint64_t d_kq = smem_desc_sw128(cx.sb + o, 16, 1024);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                const uint64_t d = desc_add(d_kq, (ks >> 2) * 16384 + (ks & 3) * 32);
+                mma_ss(tm, d, d, ID_GRAM, ks > 0);
+            }
+            mma_commit(cx.bar((CL ? PB_GRAM0 : FB_GRAM0) + (int)team));
+        }
+        __syncwarp();
+    }
 }
 
 // One team of four warps (w = 0..3, TMEM lane window w): chunk after chunk from the K/Q tiles to the operands W~^T, T', P.
@@ -535,40 +556,28 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
     const bool lower_rows = (w & 1) != 0;                     // rows 32-63
 
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     cc.advance((CL ? (int)rank - 1 : 0) + R * (int)team);
 #pragma unroll 1
-    for (uint32_t k = 0; cc.valid; ++k, cc.advance(R * (int)NTEAM)) {
+    for (uint32_t k = 0; cc.valid; ++k) {
         const uint32_t par = k & 1u, i = k * NTEAM + team;        // position in the CTA's chunk sequence
         const uint32_t o_kq = CL ? team * P_TEAM : F_KQ + (i & 3u) * 32768, kq = cx.sb + o_kq;
         const uint32_t o_p = CL ? team * P_TEAM + P_OPS + OPS_P : F_P + (i % 3u) * 8192;
         const int b_kq = CL ? PB_KQ_FULL0 + (int)team : FB_KQ_FULL0 + (int)(i & 3u);
         const uint32_t kq_par = CL ? par : (i >> 2) & 1u;
         auto& dc = prep_rec<CL>(cx.misc, i & 3u);
-        if (w == 0) {
-            // ---- Gram = [K;Q] K^T
-            cx.wait(b_kq, kq_par);
-            tc_fence_after();
-            if (elect_one()) {
-                const uint64_t d_kq = smem_desc_sw128(kq, 16, 1024);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t d = desc_add(d_kq, (ks >> 2) * 16384 + (ks & 3) * 32);
-                    mma_ss(tm_gram, d, d, ID_GRAM, ks > 0);
-                }
-                mma_commit(cx.bar((CL ? PB_GRAM0 : FB_GRAM0) + (int)team));
-            }
-            __syncwarp();
-        }
         if (CL) {
             if (k >= 1) cx.wait(PB_SENT0 + (int)team, (k - 1) & 1u);        // the operands of the team's last chunk are in the ring
         } else {
             // T' and P were last read by U^T of chunk i - 2 and the outputs of chunk i - 3
-            if (i >= 2) cx.wait(FB_U0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
-            if (i >= 3) cx.wait(FB_DONE0 + (int)((i - 3) & 3u), ((i - 3) >> 2) & 1u);
+            if (w == 0 && i >= 2) cx.wait(FB_U0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
+            if (w == 0 && i >= 3) cx.wait(FB_DONE0 + (int)((i - 3) & 3u), ((i - 3) >> 2) & 1u);
         }
-        cx.wait((CL ? PB_DECAY_READY0 : FB_DECAY_READY0) + (int)(i & 3u), (i >> 2) & 1u);
-        cx.wait((CL ? PB_GRAM0 : FB_GRAM0) + (int)team, par);
+        if (CL || w == 0) {
+            cx.wait((CL ? PB_DECAY_READY0 : FB_DECAY_READY0) + (int)(i & 3u), (i >> 2) & 1u);
+            cx.wait((CL ? PB_GRAM0 : FB_GRAM0) + (int)team, par);
+        }
+        if (!CL) team_sync();
         tc_fence_after();
         float G2t = dc.G2[t];
         float* col_eG = dc.eG;                                  // column factors of T''
@@ -622,7 +631,7 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
             uint8_t* prow = (isA ? TP : cx.sm + o_p) + t * 128;
             const float rowf = lower_rows ? ex2_approx(G2t - dc.G2mid) : 0.f;
 #pragma unroll 1
-            for (int cb = 0; cb < (lower_rows ? 4 : 2); ++cb) {       // (blocks above the diagonal: zero since the start)
+            for (int cb = 0; cb < (lower_rows ? 4 : 2); ++cb) {       // (blocks above the diagonal are not read)
                 const int c0 = 16 * cb;
                 uint32_t acc[16];
                 tmem_ld16(tm_gram + lane_win + c0, acc);
@@ -669,12 +678,7 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
             tc_fence_before();
         }
         // T'' of a fused CTA takes the first half of the W~^T buffer, which S0 W~^T of chunk i - 2 has to have read
-        if (!CL) {
-            if (i >= 2) cx.wait(FB_MMA1_0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
-            const int row = w * 16 + (lane >> 1);               // zero what lies above its diagonal
-            for (int ch = (row >> 3) + 1 + (lane & 1); ch < 8; ch += 2)
-                *reinterpret_cast<uint4*>(TPP + row * 128 + ((ch ^ (row & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-        }
+        if (!CL && w == 0 && i >= 2) cx.wait(FB_MMA1_0 + (int)(i & 1u), ((i >> 1) - 1u) & 1u);
         team_sync();
 
         // ---- P^ = (I + A^)^-1, block by block in place; every block of the result is also stored with its columns times
@@ -711,6 +715,8 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
                 for (int r = 0; r < 8; ++r)
                     *reinterpret_cast<__nv_bfloat16*>(dst + sw_off(b + r, b + jj)) = __float2bfloat16_rn(x[r] * f);
             }
+            // (the quarter of the 16 x 16 block above the diagonal; the post-processing has written it in T')
+            if (lane < 8) *reinterpret_cast<uint4*>(TPP + sw_off(b16 + lane, b16 + 8)) = make_uint4(0u, 0u, 0u, 0u);
             __syncwarp();
             // stores -d (two adjacent columns of row r) to T' and, scaled, to T''
             auto put = [&](float d0, float d1, int r, int c) {
@@ -786,36 +792,43 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
                 const uint64_t d_tpp = smem_desc_sw128(cx.sb + o_tpp, 16, 1024);
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_ss(tm_wacc, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * 32), ID_WU, ks > 0);
+                    mma_ss(tm_wacc + 16 * ks, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * (2048 + 32)), id_wu(64 - 16 * ks), ks > 0);
                 mma_commit(cx.bar((CL ? PB_W0 : FB_W0) + (int)team));
             }
             __syncwarp();
         }
-        cx.wait((CL ? PB_W0 : FB_W0) + (int)team, par);
+        cc.advance(R * (int)NTEAM);
+        if (CL || w == 0) cx.wait((CL ? PB_W0 : FB_W0) + (int)team, par);
+        if (!CL) team_sync();
         tc_fence_after();
         {
             const int drow = w * 32 + lane;
             uint8_t* wrow = cx.sm + o_w + drow * 128;
 #pragma unroll 1
-            for (int hf = 0; hf < 4; ++hf) {
-                uint32_t acc[16];
-                tmem_ld16(tm_wacc + lane_win + 16 * hf, acc);
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t acc[32];
+                tmem_ld32(tm_wacc + lane_win + 32 * hf, acc);
                 tmem_ld_wait();
+                if (hf == 1) {
+                    // the team's accumulator has been read: it may take the next Gram tile
+                    tc_fence_before();
+                    warp_arrive(cx.bar((CL ? PB_TACC_FREE0 : FB_TACC_FREE0) + (int)team), lane);
+                }
 #pragma unroll
-                for (int c8 = 0; c8 < 2; ++c8) {
+                for (int c8 = 0; c8 < 4; ++c8) {
                     uint4 u;
                     u.x = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 0]), __uint_as_float(acc[c8 * 8 + 1]));
                     u.y = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 2]), __uint_as_float(acc[c8 * 8 + 3]));
                     u.z = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 4]), __uint_as_float(acc[c8 * 8 + 5]));
                     u.w = pack_bf16x2(__uint_as_float(acc[c8 * 8 + 6]), __uint_as_float(acc[c8 * 8 + 7]));
-                    *reinterpret_cast<uint4*>(wrow + (((2 * hf + c8) ^ (drow & 7)) << 4)) = u;
+                    *reinterpret_cast<uint4*>(wrow + (((4 * hf + c8) ^ (drow & 7)) << 4)) = u;
                 }
             }
             tc_fence_before();
             fence_proxy_async_smem();
         }
         warp_arrive(cx.bar((CL ? PB_OPS0 : FB_OPS0) + (int)team), lane);         // the operands are complete
-        team_sync();                                            // (and the accumulators may take the next tiles)
+        team_sync();                                            // (T'' and the factors may be overwritten)
     }
 }
 
@@ -826,7 +839,7 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
 __device__ void chain_producer(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v)
 {
     ChunkCursor ck, cv;                                       // next chunk of K/Q, of V
-    ck.init(prm);
+    ck.init(prm, cx.misc);
     cv = ck;
     const bool leader = elect_one();
     uint32_t ik = 0, iv = 0;
@@ -866,7 +879,7 @@ __device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
     const uint32_t R = prm->csize - 1;
     const uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     const bool leader = elect_one();
 #pragma unroll 1
     for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
@@ -897,7 +910,7 @@ template <bool CL>
 __device__ void chain_mma(const Ctx& cx, const TcParams* prm)
 {
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
     const bool has_init = prm->p.init_state != nullptr;
     constexpr int WH = 4, WA = 8;                           // epilogue warps per half of the state, and in all
     constexpr uint32_t HALF = CL ? 8192 : 16384;            // from half to half of a K or Q tile
@@ -923,7 +936,7 @@ __device__ void chain_mma(const Ctx& cx, const TcParams* prm)
             const uint64_t d_tp = d_sw + (sb16 + (CL ? (C_OPS + OPS_TP) / 16 + os * (OPS_BYTES / 16) : F_TP / 16 + (j & 1u) * 512));
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma_ss(acc1, desc_add(d_v, ks * 2048), desc_add(d_tp, ks * 32), ID_WU, ks > 0);
+                mma_ss(acc1 + 16 * ks, desc_add(d_v, ks * 2048), desc_add(d_tp, ks * (2048 + 32)), id_wu(64 - 16 * ks), ks > 0);
             mma_commit(cx.bar(CL ? (int)CB_U : FB_U0 + (int)(j & 1u)));
         }
         __syncwarp();
@@ -986,7 +999,7 @@ __device__ void chain_mma(const Ctx& cx, const TcParams* prm)
         if (leader) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma_ts(acc3, acc1 + TM_DBF + ks * 16, desc_add(d_p, ks * 32), ID_DP, ks > 0);
+                mma_ts(acc3 + 16 * ks, acc1 + TM_DBF + ks * 16, desc_add(d_p, ks * (2048 + 32)), id_dp(64 - 16 * ks), ks > 0);
             mma_commit(cx.bar(CL ? CB_OUT0 + (int)par : (int)FB_OUT));
             mma_commit(cx.bar((CL ? CB_DONE0 : FB_DONE0) + (int)(j & 3u)));       // every tile and operand of this chunk has been read
         }
@@ -1006,7 +1019,7 @@ __device__ void chain_mma(const Ctx& cx, const TcParams* prm)
 template <bool RAW>
 __device__ void chain_decay(const Ctx& cx, const TcParams* prm, int lane)
 {
-    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int, float GC, float eGC, float cprev, float c, bool rescale) {
+    walk_decays<RAW>(cx, prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int, float GC, float eGC, float cprev, float c, bool rescale) {
         const float cinv = rescale ? 1.f : __frcp_rn(c);
         float r0 = b0 * (ex2_approx(GC - G0) * cinv), r1 = b1 * (ex2_approx(GC - G1) * cinv);
         if (j >= 4) cx.wait(CB_DECAY_FREE0 + (int)(j & 3u), ((j >> 2) - 1u) & 1u);     // last read by the outputs of chunk j - 4
@@ -1049,6 +1062,32 @@ __device__ __noinline__ void init_chain(const Ctx cx, const float* __restrict__ 
     tc_fence_before();
 }
 
+// What the state epilogue does now and then, out of its way (hot code competes for the instruction cache): the stored state times wb,
+// and the final state, columns a .. a + 63 of the lane's value index.
+__device__ __noinline__ void rescale_state(uint32_t ta, float wb)
+{
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+        uint32_t acc[16];
+        tmem_ld16(ta + 16 * g, acc);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * wb);
+        tmem_st16(ta + 16 * g, acc);
+    }
+}
+__device__ __noinline__ void store_state(uint32_t ta, float* out, float c)
+{
+#pragma unroll 1
+    for (int g = 0; g < 2; ++g) {
+        uint32_t acc[32];
+        tmem_ld32(ta + 32 * g, acc);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) out[(32 * g + i) * 128] = __uint_as_float(acc[i]) * c;
+    }
+}
+
 // Delta epilogue, state conversion, start and final states.  Two warps per TMEM lane window: cs is the column half (32 tokens of
 // Delta, 64 columns of the state).
 template <bool CL>
@@ -1057,18 +1096,17 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
     const Problem& p = prm->p;
     const int w4 = warp & 3, cs = warp >> 2;
     constexpr int WH = 4, WA = 8;                         // (see chain_mma)
+    auto half_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(6 + cs) : "memory"); };
     const int dv = w4 * 32 + lane;                        // value-dimension index = TMEM lane
     const uint32_t tl = cx.tmem + ((uint32_t)(w4 * 32) << 16);
     Misc* misc = cx.misc;
-    const uint32_t num_items = (uint32_t)p.num_seqs * (uint32_t)p.Hv;
     const bool has_init = p.init_state != nullptr;
 
     uint32_t j = 0;
 #pragma unroll 1
     for (int r = 0;; ++r) {
-        const uint32_t item = ChunkCursor::item_of(prm, r);
-        if (item >= num_items) break;
-        const int4 ci = ChunkCursor::lookup(prm, item);
+        const int4 ci = chain_entry(prm, misc, r);
+        if (ci.w < 0) break;
         const int n = ci.w, h = ci.z & 0xffff;
         const int nchunks = (ci.y - ci.x + 63) >> 6;
         const size_t st_off = ((size_t)n * p.Hv + h) * 128 * 128;
@@ -1089,10 +1127,13 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
             const auto& dc = chain_rec<CL>(misc, j & 3u);
 
             // ---- Delta epilogue: bf16 Delta^T and decayed Delta'^T as TMEM A operands ----------------------
-            cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);   // factors of this chunk are published
-            const float cfin = dc.cfin;
             const uint32_t acc1 = tl + TM_ACC1 + 32 * cs;
-            cx.wait(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)(j & 1u), CL ? j & 1u : (j >> 1) & 1u);
+            if (CL || w4 == 0) {
+                cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);   // factors of this chunk are published
+                cx.wait(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)(j & 1u), CL ? j & 1u : (j >> 1) & 1u);
+            }
+            if (!CL) half_sync();
+            const float cfin = dc.cfin;
             tc_fence_after();
             // The accumulator holds Delta~^T = Delta^T diag(beta)^-1: times beta e^(G_C - G) / c it is the A operand of the
             // state update, which the chain waits for; as it stands it is that of the output product (P has beta on its columns).
@@ -1131,35 +1172,31 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
 
             // ---- state: bf16 copy for the next chunk's MMAs, or the final state ------------------------------
             // if the next chunk starts from a rescaled state, the stored state is multiplied by wb on the way
+            if (CL || w4 == 0) {
+                if (!last) cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)((j + 1) & 3u), ((j + 1) >> 2) & 1u);
+                cx.wait((CL ? CB_STATE0 : FB_STATE0) + cs, j & 1u);
+            }
+            if (!CL) half_sync();
             float wb = 1.f;
             bool rescale = false;
             if (!last) {
-                cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)((j + 1) & 3u), ((j + 1) >> 2) & 1u);
                 wb = chain_rec<CL>(misc, (j + 1) & 3u).wb;
                 rescale = chain_rec<CL>(misc, (j + 1) & 3u).rescale != 0;
             }
-            cx.wait((CL ? CB_STATE0 : FB_STATE0) + cs, j & 1u);
             tc_fence_after();
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                const int c0 = 64 * cs + 32 * g;
-                uint32_t acc[32];
-                tmem_ld32(tl + TM_S32 + c0, acc);
-                tmem_ld_wait();
-                if (!last) {
-                    uint32_t pk[16];
+            if (!last) {
+#pragma unroll (CL ? 2 : 1)
+                for (int g = 0; g < 2; ++g) {
+                    uint32_t acc[32], pk[16];
+                    tmem_ld32(tl + TM_S32 + 64 * cs + 32 * g, acc);
+                    tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(__uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1]));
-                    tmem_st16(tl + TM_SBF + (c0 >> 1), pk);
-                    if (rescale) {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * wb);
-                        tmem_st32(tl + TM_S32 + c0, acc);
-                    }
-                } else if (st_out && !misc->abort) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) st_out[(c0 + i) * 128 + dv] = __uint_as_float(acc[i]) * cfin;
+                    tmem_st16(tl + TM_SBF + 32 * cs + 16 * g, pk);
                 }
+                if (rescale) rescale_state(tl + TM_S32 + 64 * cs, wb);
+            } else if (st_out && !misc->abort) {
+                store_state(tl + TM_S32 + 64 * cs, st_out + 64 * cs * 128 + dv, cfin);
             }
             tmem_st_wait();
             tc_fence_before();
@@ -1187,7 +1224,7 @@ __device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap*
     const int st_tok = ((lane >> 4) << 3) + (lane & 7), v8 = w4 * 4 + (CL ? (warp >> 2) * 2 : 0) + ((lane >> 3) & 1);     // v8: 8-value block of the lane's row
     const uint32_t st_base = cx.sb + (uint32_t)(v8 >> 3) * HALF;
     ChunkCursor cc;
-    cc.init(prm);
+    cc.init(prm, cx.misc);
 #pragma unroll 1
     for (uint32_t j = 0; cc.valid; ++j, cc.advance()) {
         const int row0 = cc.row0(), nvalid = cc.nvalid();
@@ -1195,8 +1232,11 @@ __device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap*
         const auto& dc = chain_rec<CL>(cx.misc, j & 3u);
         const uint32_t o_t = CL ? C_O + (j & 1u) * 16384 : F_KQ + (j & 3u) * 32768 + 8192;
         uint8_t* const ot = cx.sm + o_t;
-        cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);
-        cx.wait(CL ? CB_OUT0 + (int)(j & 1u) : (int)FB_OUT, CL ? (j >> 1) & 1u : j & 1u);
+        if (CL || leader) {
+            cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);
+            cx.wait(CL ? CB_OUT0 + (int)(j & 1u) : (int)FB_OUT, CL ? (j >> 1) & 1u : j & 1u);
+        }
+        if (!CL) group_sync();
         tc_fence_after();
         const uint32_t ta = cx.tmem + ((uint32_t)(w4 * 32 + (CL ? (warp >> 2) * 16 : 0)) << 16), ta3 = ta + tm_acc3<CL>(j), ta2 = ta + tm_acc2<CL>(j);
 #pragma unroll 1
@@ -1267,41 +1307,41 @@ __device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap*
 // ================================================================================================
 // Fused CTA: the roles that differ from those of the split
 // ================================================================================================
-// warp 0: K/Q tiles, up to four chunks ahead
-__device__ void fused_producer_kq(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
+// warp 0: K/Q tiles, up to four chunks ahead, and V tiles; the single V buffer is free once U^T of the chunk before has been formed
+__device__ void fused_producer(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v)
 {
-    ChunkCursor cc;
-    cc.init(prm);
+    ChunkCursor ck, cv;
+    ck.init(prm, cx.misc);
+    cv = ck;
+    const bool leader = elect_one();
+    uint32_t ik = 0;
+    auto load_kq = [&]() {
+        if ((int32_t)ik != prm->skip_kq_load && leader)           // testing aid: the skipped tile never arrives
+            load_kq_tiles(cx.sb + F_KQ + (ik & 3u) * 32768, tm_q, tm_k, ck.hq, ck.row0(), cx.bar(FB_KQ_FULL0 + (int)(ik & 3u)));
+        __syncwarp();
+        ck.advance(); ++ik;
+    };
+    while (ik < 4 && ck.valid) load_kq();
 #pragma unroll 1
-    for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
-        if (j >= 4) cx.wait(FB_KQ_FREE0 + (int)(j & 3u), ((j >> 2) - 1u) & 1u);
-        if ((int32_t)j != prm->skip_kq_load) {           // testing aid: the skipped tile never arrives
-            if (elect_one()) load_kq_tiles(cx.sb + F_KQ + (j & 3u) * 32768, tm_q, tm_k, cc.hq, cc.row0(), cx.bar(FB_KQ_FULL0 + (int)(j & 3u)));
-            __syncwarp();
-        }
-    }
-}
-// warp 3: V tiles; the single buffer is free once U^T of the chunk before has been formed
-__device__ void fused_producer_v(const Ctx& cx, const TcParams* prm, const CUtensorMap* tm_v)
-{
-    ChunkCursor cc;
-    cc.init(prm);
-#pragma unroll 1
-    for (uint32_t j = 0; cc.valid && !cx.stop(); ++j, cc.advance()) {
+    for (uint32_t j = 0; cv.valid && !cx.stop(); ++j, cv.advance()) {
         if (j >= 1) cx.wait(FB_U0 + (int)((j - 1) & 1u), ((j - 1) >> 1) & 1u);
-        if (elect_one()) {
+        if (leader) {
             const uint32_t bar = cx.bar(FB_V_FULL);
             mbar_arrive_expect_tx(bar, 16384u);
-            load_tile(cx.sb + F_V, tm_v, cc.h, cc.row0(), bar);
+            load_tile(cx.sb + F_V, tm_v, cv.h, cv.row0(), bar);
         }
         __syncwarp();
+        if (j >= 1 && ck.valid) {
+            cx.wait(FB_KQ_FREE0 + (int)(ik & 3u), ((ik >> 2) - 1u) & 1u);
+            load_kq();
+        }
     }
 }
 // warp 2: the factors of both parts, up to three chunks ahead
 template <bool RAW>
 __device__ void fused_decay(const Ctx& cx, const TcParams* prm, int lane)
 {
-    walk_decays<RAW>(prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float GC, float eGC, float cprev, float c, bool rescale) {
+    walk_decays<RAW>(cx, prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float GC, float eGC, float cprev, float c, bool rescale) {
         const float G31 = __shfl_sync(0xffffffffu, G0, 31);
         const float cinv = rescale ? 1.f : __frcp_rn(c);
         const float e0 = ex2_approx(G0) * cprev, e1 = ex2_approx(G1) * cprev;
@@ -1334,19 +1374,6 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     if (CL) allow_successor();                // (many chains: at the end, see below)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (!CL) {
-        // T' and P are only ever written on and below their 16 x 16 diagonal blocks: zero above them
-        for (uint32_t i = tid; i < 5u * 8192u / 16u; i += kThreads<CL>)
-            *reinterpret_cast<uint4*>(cx.sm + F_TP + i * 16u) = make_uint4(0u, 0u, 0u, 0u);
-        fence_proxy_async_smem();
-    } else if (rank != 0) {
-        // T', P and T'' of every team are only ever written on and below their 16 x 16 diagonal blocks: zero above them
-        for (uint32_t i = tid; i < NT * 24576u / 16u; i += kThreads<CL>) {
-            const uint32_t team = i / 1536u, o = (i % 1536u) * 16u;
-            *reinterpret_cast<uint4*>(cx.sm + team * P_TEAM + P_OPS + OPS_TP + o) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        fence_proxy_async_smem();
-    }
     if (warp == 0) {
         if (lane == 0) { prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); if (rank == 0) prefetch_tmap(&tm_v); }
     } else if (warp == 3) {
@@ -1362,7 +1389,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
         } else if (rank == 0) {
             if (i >= CB_OPS_FULL0 && i < CB_OPS_FULL0 + (int)NSLOT) count = 2;              // V tile and operands
             if (i == CB_ACC_FREE0 || i == CB_ACC_FREE1 || (i >= CB_DECAY_FREE0 && i < CB_DECAY_FREE0 + 4)) count = 8;
-        } else if (i >= PB_OPS0 && i < PB_OPS0 + (int)NT) {
+        } else if ((i >= PB_OPS0 && i < PB_OPS0 + (int)NT) || (i >= PB_TACC_FREE0 && i < PB_NUM)) {
             count = 4;
         }
         mbar_init(cx.bar(i), count);
@@ -1372,18 +1399,19 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
             cx.misc->timeout_ns = prm.wait_timeout_ns;
         }
     }
+    wait_for_predecessor();
+    if (tid < kChainTable) cx.misc->chains[tid] = load_chain_entry(&prm, tid);
     tc_fence_before();
     __syncthreads();
-    wait_for_predecessor();
     if (CL) cluster_sync_all();               // every CTA's barriers exist before another CTA arrives on them
     tc_fence_after();
     cx.tmem = cx.misc->tmem_base;
 
     if (!CL) {
-        if (warp == 0) fused_producer_kq(cx, &prm, &tm_q, &tm_k);
+        if (warp == 0) fused_producer(cx, &prm, &tm_q, &tm_k, &tm_v);
         else if (warp == 1) chain_mma<false>(cx, &prm);
         else if (warp == 2) fused_decay<RAW>(cx, &prm, lane);
-        else if (warp == 3) fused_producer_v(cx, &prm, &tm_v);
+        else if (warp == 3) gram_issuer<false>(cx, &prm, 0u);
         else if (warp < 12) prep_team<RAW, false>(cx, &prm, 0u, (uint32_t)(warp - 4) >> 2, warp & 3, lane);
         else if (warp < 20) chain_epilogue<false>(cx, &prm, warp - 12, lane);
         else chain_out<RAW, false>(cx, &prm, &tm_o, warp - 20, lane);
@@ -1396,6 +1424,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
         else chain_out<RAW, true>(cx, &prm, &tm_o, warp - 12, lane);
     } else {
         if (warp == 0) prep_producer(cx, &prm, rank, &tm_q, &tm_k);
+        else if (warp == 1) gram_issuer<true>(cx, &prm, rank);
         else if (warp == 2) prep_decay<RAW>(cx, &prm, rank, lane);
         else if (warp >= 4 && warp < 4 + 4 * (int)NT) prep_team<RAW, true>(cx, &prm, rank, (uint32_t)(warp - 4) >> 2, warp & 3, lane);
         else if (warp >= 16 && warp < 16 + (int)NT) prep_sender<RAW>(cx, &prm, rank, (uint32_t)warp - 16u);
