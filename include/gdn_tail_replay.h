@@ -112,8 +112,9 @@ typedef struct gdn_desc {
 } gdn_desc;
 
 /*
- * Device scratch the two forward calls need for this descriptor (scheduler work list and
- * counter; plus staging for every input and output when desc->memory == GDN_MEM_HOST).
+ * Device scratch the two forward calls need for this descriptor (scheduler work list;
+ * staging for every input and output when desc->memory == GDN_MEM_HOST; and, for calls with up to 37 chains on the tensor-core
+ * path, some 300 KB per chain through which CTAs hand each other operands).
  * Returns 0 for an invalid descriptor.  Host-only; no CUDA call.
  */
 GDN_API size_t gdn_workspace_size(const gdn_desc* desc);
@@ -174,7 +175,7 @@ GDN_API int32_t gdn_decode_step(const gdn_desc* desc, const void* q, const void*
  * and it stalls every stream of the device while it runs); and callers that only hold raw pointers handed
  * down from another runtime's allocator and have no allocator of their own to ask.
  *
- * It is gdn_tail_replay with the scheduler scratch (work counter + longest-first request order) taken from
+ * It is gdn_tail_replay with the scheduler scratch (the longest-first request order) taken from
  * an array that is compiled into the library's device image instead of from desc->workspace, which is
  * ignored together with desc->workspace_bytes.  The array is GDN_STATIC_SCRATCH_BYTES large and is held by
  * every GPU that loads the library until the process exits.  Limits and rules:
@@ -185,7 +186,7 @@ GDN_API int32_t gdn_decode_step(const gdn_desc* desc, const void* q, const void*
  *     caches it; make that first call before starting any stream capture;
  *   - the call itself allocates and frees nothing, on the host side of CUDA or on the device;
  *   - every call on a device shares the one array and the array keeps the previous call's contents; the
- *     scheduler kernel rewrites the counter and the part of the order list it uses before the forward
+ *     scheduler kernel rewrites the part of the order list it uses before the forward
  *     kernel reads them, so back-to-back calls on one stream are fine, but two calls that overlap on the
  *     GPU (different streams, or different host threads without ordering) race on it and are not allowed.
  * All other arguments, layouts, results and error codes are those of gdn_tail_replay.

@@ -154,7 +154,6 @@ int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, 
     cudaStream_t stream = (cudaStream_t)d->stream;
     char* ws = (char*)d->workspace;
     gdn::Sched sched;
-    sched.header = (gdn::SchedHeader*)ws;
     sched.order = (int32_t*)(ws + sizeof(gdn::SchedHeader));
     ws += sched_bytes(d);
     sched.ring = ring && d->workspace_bytes >= need + ring ? (uint8_t*)d->workspace + need : nullptr;

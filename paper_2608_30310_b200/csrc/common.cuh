@@ -33,15 +33,13 @@ constexpr int64_t kRingClusters = 37;
 
 // Scheduler scratch at the head of the workspace.
 struct SchedHeader {
-    uint32_t next_item;       // dynamic work counter, reset by the scheduler kernel
-    uint32_t pad[63];
+    uint32_t reserved[64];
 };
 static_assert(sizeof(SchedHeader) == 256, "header is one 256-byte line");
 
 // Work list: requests ordered longest-first (paper is silent on scheduling; ragged tails from
 // concurrent cache hits differ up to 8x in length, so long chains must start first).
 struct Sched {
-    SchedHeader* header;
     int32_t* order;           // [N] request indices, longest first; null: the requests in the order given (the
                               // tensor-core path with a single request, which then needs no scheduler kernel)
     uint8_t* ring;            // kRingSlots * kRingSlotBytes per chain, for calls of up to kRingClusters chains on the
