@@ -70,13 +70,12 @@ size_t ring_bytes(const gdn_desc* d)
     return tc && chains <= gdn::kRingClusters ? round256((size_t)chains * gdn::kRingSlots * gdn::kRingSlotBytes) : 0;
 }
 
-// Scheduler + forward kernel of one (sub-)batch on `stream`; sets the launch count of this thread.
-int32_t run_kernels(gdn::Problem& p, gdn::Sched sched, bool use_tc, int32_t kernel, int32_t io_dtype, cudaStream_t stream)
+// Forward kernel of one (sub-)batch on `stream`, with the scheduler kernel before it where the requests are many (see kSelfSort)
+// or the caller wants the order as a list; sets the launch count of this thread.
+int32_t run_kernels(gdn::Problem& p, gdn::Sched sched, bool use_tc, bool list, int32_t kernel, int32_t io_dtype, cudaStream_t stream)
 {
     g_last_launches = 0;
-    // A single request needs no ordering: the tensor-core path then runs without the scheduler kernel, which
-    // matters for the batch-1 state rebuild (one call per layer, a few microseconds each).
-    if (use_tc && p.num_seqs == 1 && p.total_tokens > 0 && gdn::tcgen05_supported(p)) {
+    if (list ? use_tc && p.num_seqs == 1 && gdn::tcgen05_supported(p) : p.num_seqs <= gdn::kSelfSort) {
         sched.order = nullptr;
     } else {
         if (gdn::launch_scheduler(p.cu, p.num_seqs, sched, stream) != cudaSuccess) return GDN_ERR_CUDA;
@@ -123,7 +122,7 @@ HostPipe* host_pipe()
 }
 
 int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, const float* g,
-                const float* beta, const int32_t* cu, int32_t chunk, void* out_o, float* out_state)
+                const float* beta, const int32_t* cu, int32_t chunk, void* out_o, float* out_state, bool list = false)
 {
     g_last_launches = 0;
     if (!desc_shape_ok(d)) return GDN_ERR_INVALID_ARG;
@@ -169,7 +168,7 @@ int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, 
     if (d->memory == GDN_MEM_DEVICE) {
         p.q = q; p.k = k; p.v = v; p.g = g; p.beta = beta; p.cu = cu;
         p.init_state = d->init_state; p.out_o = out_o; p.out_state = out_state;
-        return run_kernels(p, sched, use_tc, d->kernel, d->io_dtype, stream);
+        return run_kernels(p, sched, use_tc, list, d->kernel, d->io_dtype, stream);
     }
 
     // ---- host memory: staged through the workspace and pipelined by groups of requests over three streams: the
@@ -241,7 +240,7 @@ int32_t forward(const gdn_desc* d, const void* q, const void* k, const void* v, 
         gdn::Sched sg = sched;
         sg.order = sched.order + n0;
         const int before = g_last_launches;
-        status = run_kernels(pg, sg, use_tc, d->kernel, d->io_dtype, stream);
+        status = run_kernels(pg, sg, use_tc, list, d->kernel, d->io_dtype, stream);
         g_last_launches += before;
         if (status != GDN_OK) break;
         err = cudaEventRecord(hp->ev_k[gi], stream);
@@ -314,7 +313,8 @@ int32_t gdn_tail_replay_static_scratch(const gdn_desc* desc, const void* q, cons
     gdn_desc d = *desc;
     d.workspace = scratch;
     d.workspace_bytes = GDN_STATIC_SCRATCH_BYTES;
-    return forward(&d, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state);
+    // the order of several requests is always made in that array here: its contract
+    return forward(&d, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, true);
 }
 
 int32_t gdn_decode_step(const gdn_desc* d, const void* q, const void* k, const void* v, const float* g,

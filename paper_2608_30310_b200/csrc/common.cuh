@@ -40,8 +40,8 @@ static_assert(sizeof(SchedHeader) == 256, "header is one 256-byte line");
 // Work list: requests ordered longest-first (paper is silent on scheduling; ragged tails from
 // concurrent cache hits differ up to 8x in length, so long chains must start first).
 struct Sched {
-    int32_t* order;           // [N] request indices, longest first; null: the requests in the order given (the
-                              // tensor-core path with a single request, which then needs no scheduler kernel)
+    int32_t* order;           // [N] request indices, longest first, from the scheduler kernel; null: every CTA orders the
+                              // requests itself (up to kSelfSort of them)
     uint8_t* ring;            // kRingSlots * kRingSlotBytes per chain, for calls of up to kRingClusters chains on the
                               // tensor-core path; null: none (the call then runs without clusters)
 };
@@ -64,6 +64,38 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
 }
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Up to this many requests the kernels order the requests themselves, each CTA for itself: two lengths per lane, a rank is two
+// ballots, so the whole order costs one load of cu and a few hundred cycles, less than the scheduler kernel's turn in the
+// stream (a microsecond a call, although its launch is hidden).  Beyond two lengths per lane the calls are long and the scheduler kernel does it once.
+constexpr int kSelfSort = 64;
+// table[rank] = (first row, end row, request), longest first, ties by index.  All warps of the CTA call it, then synchronise.
+static __device__ __noinline__ void sort_requests(const int32_t* cu, int num_seqs, int4* table, int warp, int nwarps, int lane)
+{
+    int len[2], row[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int n = lane + 32 * i;
+        row[i] = n < num_seqs ? cu[n] : 0;
+        len[i] = n < num_seqs ? cu[n + 1] - row[i] : (int)0x80000000;      // (longer than no request)
+    }
+    for (int n = warp; n < num_seqs; n += nwarps) {
+        const int ln = __shfl_sync(0xffffffffu, n < 32 ? len[0] : len[1], n & 31);
+        const int rn = __shfl_sync(0xffffffffu, n < 32 ? row[0] : row[1], n & 31);
+        const int rank = __popc(__ballot_sync(0xffffffffu, len[0] > ln || (len[0] == ln && lane < n))) +
+                         __popc(__ballot_sync(0xffffffffu, len[1] > ln || (len[1] == ln && lane + 32 < n)));
+        if (lane == 0) table[rank] = make_int4(rn, rn + ln, n, 0);
+    }
+}
+// Whether the CTAs have to call sort_requests; a single request needs no order.
+__device__ __forceinline__ bool self_sorted(const Problem& p, const Sched& s) { return !s.order && p.num_seqs > 1; }
+// (first row, end row, request) of place `i` in the order
+__device__ __forceinline__ int4 request_at(const Problem& p, const Sched& s, const int4* table, uint32_t i)
+{
+    if (self_sorted(p, s)) return table[i];
+    const int n = s.order ? s.order[i] : 0;
+    return make_int4(p.cu[n], p.cu[n + 1], n, 0);
+}
 
 cudaError_t launch_scheduler(const int32_t* cu, int32_t num_seqs, const Sched& s, cudaStream_t stream);
 cudaError_t launch_simt(const Problem& p, const Sched& s, int io_dtype, cudaStream_t stream, int* launches);

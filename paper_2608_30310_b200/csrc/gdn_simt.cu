@@ -53,6 +53,7 @@ struct Smem {
     __align__(16) float mn[NH][2][kBlk][kBlk];           // helpers: [0][i][t] -M, [1][i][t] N
     __align__(16) float dr[NW][kBlk][2 * RPT];           // R(8, i) delta_i by token
     __align__(16) float v[NW][kBlk][2 * RPT];            // v of the block
+    int4 requests[kSelfSort];                            // the requests, longest first (see sort_requests)
 };
 
 // N consecutive values of v as fp32, in one load that stays where it is written (the compiler would sink a prefetch to its first
@@ -109,7 +110,7 @@ constexpr int BAR_FULL = 1, BAR_EMPTY = 1 + kBufs;
 // SM b modulo their number as long as the GPU is empty): the longest share their SM with the shortest.
 struct Item { int n, h, hq, slice, row_begin, row_end; };
 template <int SLICES>
-__device__ __forceinline__ bool item_at(const Problem& p, const Sched& s, int sms, uint32_t round, Item& it)
+__device__ __forceinline__ bool item_at(const Problem& p, const Sched& s, const int4* requests, int sms, uint32_t round, Item& it)
 {
     const uint32_t pos = blockIdx.x % sms, r = blockIdx.x / sms + round * ((gridDim.x + sms - 1) / sms);
     const uint32_t item = r * sms + ((r & 1u) ? sms - 1 - pos : pos);
@@ -117,19 +118,19 @@ __device__ __forceinline__ bool item_at(const Problem& p, const Sched& s, int sm
     it.slice = (int)(item % SLICES);
     const uint32_t c = item / SLICES;
     it.h = (int)(c % p.Hv);
-    it.n = s.order[c / p.Hv];
     it.hq = it.h / (p.Hv / p.Hq);
-    it.row_begin = p.cu[it.n]; it.row_end = p.cu[it.n + 1];
+    const int4 rq = request_at(p, s, requests, c / p.Hv);
+    it.row_begin = rq.x; it.row_end = rq.y; it.n = rq.z;
     return true;
 }
 
 // the next item of the block with round >= round, which it updates; false when there is none
 template <int SLICES>
-__device__ __forceinline__ bool more(const Problem& p, const Sched& s, int sms, uint32_t& round, Item& it)
+__device__ __forceinline__ bool more(const Problem& p, const Sched& s, const int4* requests, int sms, uint32_t& round, Item& it)
 {
     const uint32_t per = (gridDim.x + sms - 1) / sms, items = (uint32_t)p.num_seqs * p.Hv * SLICES;
     for (; (blockIdx.x / sms + round * per) * sms < items; ++round)
-        if (item_at<SLICES>(p, s, sms, round, it)) return true;
+        if (item_at<SLICES>(p, s, requests, sms, round, it)) return true;
     return false;
 }
 
@@ -176,7 +177,7 @@ __device__ void helper(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& 
 
     uint32_t stage = 0;
     Item it;
-    for (uint32_t round = 0; more<SLICES>(p, s, sms, round, it); ++round) {
+    for (uint32_t round = 0; more<SLICES>(p, s, sm.requests, sms, round, it); ++round) {
         int row0 = it.row_begin + hw * kBlk;
         if (it.row_begin < it.row_end) load(it, row0);
 #pragma unroll 1
@@ -319,7 +320,7 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
 
     uint32_t stage = 0;
     Item it;
-    for (uint32_t round = 0; more<SLICES>(p, s, sms, round, it); ++round) {
+    for (uint32_t round = 0; more<SLICES>(p, s, sm.requests, sms, round, it); ++round) {
         const int j0 = it.slice * R + warp * 2 * RPT;     // first row (value index) of the warp
         const size_t st_off = ((size_t)it.n * p.Hv + it.h) * DK * DV + j0 + rg * RPT;
         float2 S[RPT][2 * NC];                            // [row ^ r], piece c: columns 64 c + 4 l .. + 3
@@ -482,6 +483,10 @@ gdn_simt_kernel(const Problem p, const Sched s, const int sms)
     Smem<DK, RPT, NW, NH>& sm = *reinterpret_cast<Smem<DK, RPT, NW, NH>*>(raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     wait_for_predecessor();
+    if (self_sorted(p, s)) {
+        sort_requests(p.cu, p.num_seqs, sm.requests, warp, NW + NH, lane);
+        __syncthreads();
+    }
     if (warp < NW) compute<DK, DV, T, RPT, NW, NH>(p, s, sm, sms, warp, lane);
     else helper<DK, DV / (2 * RPT * NW), T, RPT, NW, NH>(p, s, sm, sms, warp - NW, lane);
     allow_successor();       // at the end: a successor's blocks placed among this kernel's would land on the SMs in another order

@@ -33,7 +33,7 @@
 // Many chains, CL = false ("fused CTA"): one CTA per SM does both parts of a chain, with two prep teams and everything in its
 // own shared memory.  Its period per chunk is longer (the parts compete for the SM's issue slots), but no SM waits.
 //
-// Chains are ordered longest-first by the scheduler kernel and dealt to clusters (CTAs) in snake order, so each role can walk
+// Chains are ordered longest-first (by the scheduler kernel where there are many requests) and dealt to clusters (CTAs) in snake order, so each role can walk
 // its cluster's chunk sequence without any broadcast.  Padding rows of a ragged last chunk get beta = 0 and a cumulative
 // decay that makes their rows of A^ and P vanish, which keeps them inert whatever (finite) values follow the request
 // in memory; their outputs are not stored.  Every mbarrier wait is bounded: on expiry the CTA records
@@ -55,7 +55,7 @@ constexpr uint32_t OPS_BYTES = 32768;         // W~^T 16 KB, T' 8 KB, P 8 KB
 constexpr uint32_t OPS_W = 0, OPS_TP = 16384, OPS_P = 24576;
 constexpr uint32_t NORM_BYTES = 512;          // fused input stage: 1 / norms of the chunk's key and query rows
 static_assert(OPS_BYTES + NORM_BYTES == kRingSlotBytes, "");
-constexpr uint32_t kClusterCtas = 4;          // of a cluster: one chain CTA, three prep CTAs
+constexpr uint32_t kClusterCtas = 4, kPrepCtas = kClusterCtas - 1;          // of a cluster: one chain CTA, three prep CTAs
 
 // ---- shared memory of a chain CTA (bytes from a 1024-aligned base) -----------------------------
 constexpr uint32_t C_OPS = 0;                              // NSLOT operand slots                             96 KB
@@ -116,6 +116,7 @@ struct __align__(16) FusedDecay { float G2[64], beta[64], eG[64], colfb[32], nor
 struct FusedMisc { FusedDecay decay[4]; };
 constexpr int kChainTable = 64;
 struct Misc {
+    int4 requests[kSelfSort];          // the requests, longest first (see sort_requests)
     int4 chains[kChainTable];          // the CTA's (cluster's) first work items, see chain_entry
     unsigned long long bars[40];
     uint32_t tmem_base;
@@ -165,28 +166,37 @@ struct TcParams {
     Sched s;
     unsigned long long wait_timeout_ns;   // bound of every device-side wait
     int32_t skip_kq_load;         // testing aid: chunk whose K/Q copy is left out (-1: none)
-    uint32_t csize;               // CTAs per cluster (1 chain CTA + R prep CTAs)
-    uint32_t ring;                // slots of a cluster's operand ring, a multiple of NT * R: a ring slot and its credits belong
-                                  // to one team, so that no wait looks more than one phase ahead
 };
+// A ring slot and its credits belong to one team, so that no wait looks more than one phase ahead.
+static_assert(kRingSlots % (NT * kPrepCtas) == 0, "");
 
-// Work item of round r of this cluster: chains dealt in snake order over the longest-first list.  x = first row, y = end row,
-// z = v-head | q/k head << 16, w = request, or -1 when the items are exhausted.
-__device__ __noinline__ int4 load_chain_entry(const TcParams* prm, int r)
+// Place of the work item of round r of this cluster, chains dealt in snake order over the longest-first list: x = place in the
+// order of requests, or -1 when the items are exhausted, y = v-head | q/k head << 16.
+template <bool CL>
+__device__ __forceinline__ int2 chain_place(const TcParams* prm, int r)
 {
     const Problem& p = prm->p;
-    const uint32_t G = gridDim.x / prm->csize, b = blockIdx.x / prm->csize;
+    constexpr uint32_t csize = CL ? kClusterCtas : 1u;
+    const uint32_t G = gridDim.x / csize, b = blockIdx.x / csize;
     const uint32_t item = (uint32_t)r * G + ((r & 1) ? (G - 1 - b) : b);
-    if (item >= (uint32_t)p.num_seqs * (uint32_t)p.Hv) return make_int4(0, 0, 0, -1);
-    const int n = prm->s.order ? prm->s.order[item / p.Hv] : (int)(item / p.Hv);   // no order list: requests as given
-    const int h = item % p.Hv;
-    return make_int4(p.cu[n], p.cu[n + 1], h | ((h / (p.Hv / p.Hq)) << 16), n);
+    if (item >= (uint32_t)p.num_seqs * (uint32_t)p.Hv) return make_int2(-1, 0);
+    const uint32_t h = item % (uint32_t)p.Hv;
+    return make_int2((int)(item / (uint32_t)p.Hv), (int)(h | (h / ((uint32_t)p.Hv / (uint32_t)p.Hq)) << 16));
 }
+// The work item: x = first row, y = end row, z = v-head | q/k head << 16, w = request, or -1 when the items are exhausted.
+__device__ __forceinline__ int4 chain_at(const TcParams* prm, const Misc* misc, int2 place)
+{
+    if (place.x < 0) return make_int4(0, 0, 0, -1);
+    const int4 rq = request_at(prm->p, prm->s, misc->requests, (uint32_t)place.x);
+    return make_int4(rq.x, rq.y, place.y, rq.z);
+}
+// (a cluster has a single work item: rounds beyond the table are the fused form's)
+__device__ __noinline__ int4 load_chain_entry(const TcParams* prm, const Misc* misc, int r) { return chain_at(prm, misc, chain_place<false>(prm, r)); }
 // The same from shared memory, where the first kChainTable of them are put at the start of the kernel, side by side: divisions and
 // three dependent loads from global memory, some 1,500 cycles that every role would otherwise spend at every chain.
 __device__ __noinline__ int4 chain_entry(const TcParams* prm, const Misc* misc, int r)
 {
-    return r < kChainTable ? misc->chains[r] : load_chain_entry(prm, r);
+    return r < kChainTable ? misc->chains[r] : load_chain_entry(prm, misc, r);
 }
 // Walks the chunk sequence of one cluster: its chains, chunks of 64 rows inside each chain.  Every role keeps its own cursor(s).
 struct ChunkCursor {
@@ -439,7 +449,7 @@ __device__ __forceinline__ void walk_decays(const Ctx& cx, const TcParams* prm, 
 // warp 0: K/Q tiles of the CTA's chunks, one buffer per team, refilled as soon as the team's W~^T product has read it
 __device__ void prep_producer(const Ctx& cx, const TcParams* prm, uint32_t rank, const CUtensorMap* tm_q, const CUtensorMap* tm_k)
 {
-    const int R = (int)prm->csize - 1;
+    constexpr uint32_t R = kPrepCtas;
     ChunkCursor cc;
     cc.init(prm, cx.misc);
     cc.advance((int)rank - 1);
@@ -458,14 +468,14 @@ __device__ void prep_producer(const Ctx& cx, const TcParams* prm, uint32_t rank,
 template <bool RAW>
 __device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, uint32_t team)
 {
-    const uint32_t R = prm->csize - 1, own = prm->ring / R;            // ring slots of this CTA (kRingSlots / 3 or kRingSlotsPair)
+    constexpr uint32_t R = kPrepCtas, own = kRingSlots / R;            // ring slots of this CTA
     ChunkCursor cc;
     cc.init(prm, cx.misc);
     cc.advance((int)(rank - 1 + team * R));
-    uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
+    uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / kClusterCtas) * kRingSlots * kRingSlotBytes;
 #pragma unroll 1
     for (uint32_t i = team; cc.valid; i += NT, cc.advance((int)(R * NT))) {
-        const uint32_t j = rank - 1 + i * R, slot = j % prm->ring;
+        const uint32_t j = rank - 1 + i * R, slot = j % kRingSlots;
         cx.wait(PB_OPS0 + (int)team, (i / NT) & 1u);
         if (i >= own) cx.wait_cluster(PB_CREDIT0 + (int)(i % own), (i / own - 1u) & 1u);
         if (elect_one()) {
@@ -486,7 +496,7 @@ __device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, u
 template <bool RAW>
 __device__ void prep_decay(const Ctx& cx, const TcParams* prm, uint32_t rank, int lane)
 {
-    const uint32_t R = prm->csize - 1;
+    constexpr uint32_t R = kPrepCtas;
     uint32_t i = 0;
     walk_decays<RAW>(cx, prm, lane, [&](uint32_t j, float G0, float G1, float b0, float b1, int nvalid, float, float, float cprev, float, bool) {
         if (j % R != rank - 1) return;
@@ -510,7 +520,7 @@ __device__ void prep_decay(const Ctx& cx, const TcParams* prm, uint32_t rank, in
 template <bool CL>
 __device__ void gram_issuer(const Ctx& cx, const TcParams* prm, uint32_t rank)
 {
-    const uint32_t R = CL ? prm->csize - 1 : 1u, NTEAM = CL ? NT : 2u;
+    constexpr uint32_t R = CL ? kPrepCtas : 1u, NTEAM = CL ? NT : 2u;
     ChunkCursor cc;
     cc.init(prm, cx.misc);
     if (CL) cc.advance((int)rank - 1);
@@ -539,8 +549,8 @@ __device__ void gram_issuer(const Ctx& cx, const TcParams* prm, uint32_t rank)
 template <bool RAW, bool CL>
 __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uint32_t team, int w, int lane)
 {
-    const int R = CL ? (int)prm->csize - 1 : 1;
-    const uint32_t NTEAM = CL ? NT : 2u;
+    constexpr uint32_t R = CL ? kPrepCtas : 1u;
+    constexpr uint32_t NTEAM = CL ? NT : 2u;
     const uint32_t o_w = CL ? team * P_TEAM + P_OPS + OPS_W : F_W + team * 16384;
     const uint32_t o_tp = CL ? team * P_TEAM + P_OPS + OPS_TP : F_TP + team * 8192;
     const uint32_t o_tpp = CL ? team * P_TEAM + P_TPP : o_w;
@@ -876,8 +886,8 @@ __device__ void chain_producer(const Ctx& cx, const TcParams* prm, const CUtenso
 template <bool RAW>
 __device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
 {
-    const uint32_t R = prm->csize - 1;
-    const uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / prm->csize) * prm->ring * kRingSlotBytes;
+    constexpr uint32_t R = kPrepCtas;
+    const uint8_t* const ring = prm->s.ring + (size_t)(blockIdx.x / kClusterCtas) * kRingSlots * kRingSlotBytes;
     ChunkCursor cc;
     cc.init(prm, cx.misc);
     const bool leader = elect_one();
@@ -887,12 +897,12 @@ __device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
         if (j >= NSLOT) {
             cx.wait(CB_DONE0 + (int)((j - NSLOT) & 3u), ((j - NSLOT) >> 2) & 1u);      // (its operands have landed long ago)
             const uint32_t f = j - NSLOT;
-            if (leader) mbar_arrive_remote(map_to_rank(cx.bar(PB_CREDIT0 + (int)((f / R) % (prm->ring / R))), 1u + f % R));
+            if (leader) mbar_arrive_remote(map_to_rank(cx.bar(PB_CREDIT0 + (int)((f / R) % (kRingSlots / R))), 1u + f % R));
         }
-        cx.wait_cluster(CB_RING0 + (int)(j % prm->ring), (j / prm->ring) & 1u);
+        cx.wait_cluster(CB_RING0 + (int)(j % kRingSlots), (j / kRingSlots) & 1u);
         if (leader) {
             const uint32_t bar = cx.bar(CB_OPS_FULL0 + (int)slot);
-            const uint8_t* src = ring + (size_t)(j % prm->ring) * kRingSlotBytes;
+            const uint8_t* src = ring + (size_t)(j % kRingSlots) * kRingSlotBytes;
             fence_proxy_async_global();
             mbar_arrive_expect_tx(bar, OPS_BYTES + (RAW ? NORM_BYTES : 0u));
             bulk_load(cx.sb + C_OPS + slot * OPS_BYTES, src, OPS_BYTES, bar);
@@ -1370,7 +1380,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     cx.sb = (raw + 1023u) & ~1023u;
     cx.sm = smem_raw + (cx.sb - raw);
     cx.misc = reinterpret_cast<Misc*>(cx.sm + SM_MISC);
-    const uint32_t rank = CL ? blockIdx.x % prm.csize : 0u;
+    const uint32_t rank = CL ? blockIdx.x % kClusterCtas : 0u;
     if (CL) allow_successor();                // (many chains: at the end, see below)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1399,12 +1409,17 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
             cx.misc->timeout_ns = prm.wait_timeout_ns;
         }
     }
-    // Every CTA's barriers exist before another CTA arrives on them. Nothing here depends on the scheduler's output, so
-    // the cluster's barrier stands before the wait for it and its latency passes under the scheduler: 36 layers of
+    // Every CTA's barriers exist before another CTA arrives on them. Nothing here depends on earlier kernels, so the
+    // cluster's barrier stands before the wait for them and its latency passes under the predecessor's tail: 36 layers of
     // 8,192 tokens (5 % replayed) 726 -> 708 us, one layer of 1,638 tokens 47.4 -> 46.9 us.
     if (CL) cluster_sync_all();
+    const int2 place = chain_place<CL>(&prm, tid);       // (divisions: before the wait)
     wait_for_predecessor();
-    if (tid < kChainTable) cx.misc->chains[tid] = load_chain_entry(&prm, tid);
+    if (self_sorted(prm.p, prm.s)) {
+        sort_requests(prm.p.cu, prm.p.num_seqs, cx.misc->requests, warp, kThreads<CL> / 32, lane);
+        __syncthreads();
+    }
+    if (tid < kChainTable) cx.misc->chains[tid] = chain_at(&prm, cx.misc, place);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1481,10 +1496,10 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t heads, u
 
 struct Maps { CUtensorMap q, k, v, o, qt, kt; };
 
-// CTAs (csize 1) or clusters of a size that fit on a device at the same time; the kernels' attributes are set on the first
+// CTAs (fused form) or clusters that fit on a device at the same time; the kernels' attributes are set on the first
 // call per device.
 template <bool RAW, bool CL>
-cudaError_t capacity(int dev, uint32_t csize, int* out)
+cudaError_t capacity(int dev, int* out)
 {
     static int cap[64] = {};
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -1496,8 +1511,8 @@ cudaError_t capacity(int dev, uint32_t csize, int* out)
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-            cfg.gridDim = csize; cfg.blockDim = kThreads<CL>; cfg.dynamicSmemBytes = SMEM_BYTES; cfg.attrs = at; cfg.numAttrs = 1;
+            at[0].val.clusterDim.x = kClusterCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+            cfg.gridDim = kClusterCtas; cfg.blockDim = kThreads<CL>; cfg.dynamicSmemBytes = SMEM_BYTES; cfg.attrs = at; cfg.numAttrs = 1;
             e = cudaOccupancyMaxActiveClusters(&n, gdn_tc_kernel<RAW, CL>, &cfg);
         } else {
             e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
@@ -1509,9 +1524,9 @@ cudaError_t capacity(int dev, uint32_t csize, int* out)
     return cudaSuccess;
 }
 template <bool RAW, bool CL>
-cudaError_t launch_as(TcParams& prm, uint32_t csize, long long groups, Maps& m, cudaStream_t stream)
+cudaError_t launch_as(const TcParams& prm, long long groups, const Maps& m, cudaStream_t stream)
 {
-    prm.csize = csize;
+    constexpr unsigned csize = CL ? kClusterCtas : 1;
     return launch_kernel(gdn_tc_kernel<RAW, CL>, (unsigned)groups * csize, kThreads<CL>, SMEM_BYTES, stream, csize, prm, m.q, m.k, m.v, m.o, m.qt, m.kt);
 }
 template <bool RAW>
@@ -1521,22 +1536,20 @@ cudaError_t launch(TcParams& prm, Maps& m, cudaStream_t stream)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const long long items = (long long)prm.p.num_seqs * prm.p.Hv;
-    static_assert(kRingSlots % (NT * (kClusterCtas - 1)) == 0, "see TcParams::ring");
-    prm.ring = kRingSlots;
     if (prm.s.ring && items <= kRingClusters) {
-        e = capacity<RAW, true>(dev, kClusterCtas, &cap);
+        e = capacity<RAW, true>(dev, &cap);
         if (e != cudaSuccess) return e;
         if (items <= cap) {
             const Problem& p = prm.p;
             if (!make_map(&m.qt, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) || !make_map(&m.kt, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) ||
                 !make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2))
                 return cudaErrorUnknown;
-            return launch_as<RAW, true>(prm, kClusterCtas, items, m, stream);
+            return launch_as<RAW, true>(prm, items, m, stream);
         }
     }
-    e = capacity<RAW, false>(dev, 1, &cap);
+    e = capacity<RAW, false>(dev, &cap);
     if (e != cudaSuccess) return e;
-    return launch_as<RAW, false>(prm, 1, items < cap ? items : cap, m, stream);
+    return launch_as<RAW, false>(prm, items < cap ? items : cap, m, stream);
 }
 
 unsigned long long g_wait_timeout_ns = 2000000000ull;
