@@ -464,6 +464,9 @@ __device__ void prep_producer(const Ctx& cx, const TcParams* prm, uint32_t rank,
     }
 }
 
+// Bytes of the operands, W~^T at their head, that the chunk has none of (see prep_team).
+__device__ __forceinline__ uint32_t skipped_w(const ChunkCursor& cc) { return cc.first() && !cc.prm->p.init_state ? OPS_TP : 0u; }
+
 // warps 16-18: finished operands into the cluster's ring, one warp per team (a store takes 1-2 us until it is complete)
 template <bool RAW>
 __device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, uint32_t team)
@@ -480,7 +483,8 @@ __device__ void prep_sender(const Ctx& cx, const TcParams* prm, uint32_t rank, u
         if (i >= own) cx.wait_cluster(PB_CREDIT0 + (int)(i % own), (i / own - 1u) & 1u);
         if (elect_one()) {
             uint8_t* dst = ring + (size_t)slot * kRingSlotBytes;
-            bulk_store(dst, cx.sb + team * P_TEAM + P_OPS, OPS_BYTES);
+            const uint32_t o = skipped_w(cc);
+            bulk_store(dst + o, cx.sb + team * P_TEAM + P_OPS + o, OPS_BYTES - o);
             if (RAW) bulk_store(dst + OPS_BYTES, smem_u32(cx.misc->p.decay[i & 3u].norms), NORM_BYTES);
             bulk_commit();
             bulk_wait();                                               // in L2, where the bulk load finds it; source buffers free
@@ -564,6 +568,7 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
     const int t = ((w & 1) << 5) + lane;                      // this thread's row of the Gram tile
     const bool isA = w < 2;                                   // windows 0, 1 hold K K^T rows, 2, 3 hold Q K^T rows
     const bool lower_rows = (w & 1) != 0;                     // rows 32-63
+    const bool has_init = prm->p.init_state != nullptr;
 
     ChunkCursor cc;
     cc.init(prm, cx.misc);
@@ -794,24 +799,34 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
         fence_proxy_async_smem();                               // T', T'' are read by MMAs and by the copy
         team_sync();
 
-        // ---- W~^T = K^T T''^T, then as bf16 rows [dk][t] into the operand buffer
+        // ---- W~^T = K^T T''^T, then as bf16 rows [dk][t] into the operand buffer.  Cluster: not of a chunk that starts from a
+        // zero state, whose way to the first output it would lengthen (product, copy into and out of the ring): one layer of 1,638
+        // tokens 43.7 -> 43.0 us, 36 layers of 410 tokens 672 -> 659 us.  In a fused CTA the code costs more than the few first
+        // chunks give (32 hits 524 -> 532 us).
+        const bool need_w = !CL || has_init || !cc.first();
         if (w == 0) {
             tc_fence_after();
             if (elect_one()) {
                 const uint64_t d_kt = smem_desc_sw128(kq, 16384, 1024);      // K^T, M-major
                 const uint64_t d_tpp = smem_desc_sw128(cx.sb + o_tpp, 16, 1024);
+                if (need_w) {
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_ss(tm_wacc + 16 * ks, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * (2048 + 32)), id_wu(64 - 16 * ks), ks > 0);
+                    for (int ks = 0; ks < 4; ++ks)
+                        mma_ss(tm_wacc + 16 * ks, desc_add(d_kt, ks * 2048), desc_add(d_tpp, ks * (2048 + 32)), id_wu(64 - 16 * ks), ks > 0);
+                }
                 mma_commit(cx.bar((CL ? PB_W0 : FB_W0) + (int)team));
             }
             __syncwarp();
         }
         cc.advance(R * (int)NTEAM);
+        if (!need_w) warp_arrive(cx.bar((CL ? PB_OPS0 : FB_OPS0) + (int)team), lane);         // the operands are complete
         if (CL || w == 0) cx.wait((CL ? PB_W0 : FB_W0) + (int)team, par);
         if (!CL) team_sync();
         tc_fence_after();
-        {
+        if (!need_w) {
+            tc_fence_before();
+            warp_arrive(cx.bar((CL ? PB_TACC_FREE0 : FB_TACC_FREE0) + (int)team), lane);
+        } else {
             const int drow = w * 32 + lane;
             uint8_t* wrow = cx.sm + o_w + drow * 128;
 #pragma unroll 1
@@ -836,8 +851,8 @@ __device__ void prep_team(const Ctx& cx, const TcParams* prm, uint32_t rank, uin
             }
             tc_fence_before();
             fence_proxy_async_smem();
+            warp_arrive(cx.bar((CL ? PB_OPS0 : FB_OPS0) + (int)team), lane);         // the operands are complete
         }
-        warp_arrive(cx.bar((CL ? PB_OPS0 : FB_OPS0) + (int)team), lane);         // the operands are complete
         team_sync();                                            // (T'' and the factors may be overwritten)
     }
 }
@@ -904,8 +919,9 @@ __device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
             const uint32_t bar = cx.bar(CB_OPS_FULL0 + (int)slot);
             const uint8_t* src = ring + (size_t)(j % kRingSlots) * kRingSlotBytes;
             fence_proxy_async_global();
-            mbar_arrive_expect_tx(bar, OPS_BYTES + (RAW ? NORM_BYTES : 0u));
-            bulk_load(cx.sb + C_OPS + slot * OPS_BYTES, src, OPS_BYTES, bar);
+            const uint32_t o = skipped_w(cc);
+            mbar_arrive_expect_tx(bar, OPS_BYTES - o + (RAW ? NORM_BYTES : 0u));
+            bulk_load(cx.sb + C_OPS + slot * OPS_BYTES + o, src + o, OPS_BYTES - o, bar);
             if (RAW) bulk_load(smem_u32(cx.misc->c.norms[slot]), src + OPS_BYTES, NORM_BYTES, bar);
         }
         __syncwarp();
