@@ -66,8 +66,9 @@ __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepco
 __device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Up to this many requests the kernels order the requests themselves, each CTA for itself: two lengths per lane, a rank is two
-// ballots, so the whole order costs one load of cu and a few hundred cycles, less than the scheduler kernel's turn in the
-// stream (a microsecond a call, although its launch is hidden).  Beyond two lengths per lane the calls are long and the scheduler kernel does it once.
+// ballots, so the whole order costs one load of cu and a few hundred cycles, less than the scheduler kernel's turn in the stream
+// (a microsecond a call, although its launch is hidden).  Beyond two lengths per lane the calls are long and the scheduler kernel
+// does it once.
 constexpr int kSelfSort = 64;
 // table[rank] = (first row, end row, request), longest first, ties by index.  All warps of the CTA call it, then synchronise.
 static __device__ __noinline__ void sort_requests(const int32_t* cu, int num_seqs, int4* table, int warp, int nwarps, int lane)
