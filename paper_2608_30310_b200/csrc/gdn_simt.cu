@@ -49,7 +49,8 @@ struct Smem {
     static constexpr int LD = DK + 4;     // row stride: 16-byte aligned, and eight rows at one column fall into different banks
     float k[kBufs][NH * kBlk][LD], q[kBufs][NH * kBlk][LD];
     Coef coef[kBufs][NH];
-    __align__(16) float al[NH][2 * kBlk];                // helpers: alpha and beta of the block at hand
+    __align__(16) double al[NH][kBlk];                   // helpers: alpha and beta of the block at hand
+    float be[NH][kBlk];
     __align__(16) float mn[NH][2][kBlk][kBlk];           // helpers: [0][i][t] -M, [1][i][t] N
     __align__(16) float dr[NW][kBlk][2 * RPT];           // R(8, i) delta_i by token
     __align__(16) float v[NW][kBlk][2 * RPT];            // v of the block
@@ -208,12 +209,14 @@ __device__ void helper(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& 
                 }
             }
             {
-                // rows past the end: alpha = 1, beta = 0 (k, q are zero)
+                // Rows past the end: alpha = 1, beta = 0 (k, q are zero).  alpha and its products are formed in fp64 and rounded once
+                // where they are used: eight factors rounded to fp32, and their products again, would weigh on the state more than
+                // a token-by-token evaluation does, and for equal decays with the same sign in every block (relative error of
+                // the state, 256 tokens of g = -0.01: 2.7e-7 token by token, 8.8e-7 with fp32 products, 2.0e-7 so).
                 const bool ok = row0 + (lane & 7) < it.row_end;
-                float x;
-                if (p.input_raw) x = ok ? 1.f / (1.f + expf(-gb)) : (lane < 8 ? 1.f : 0.f);      // sigmoid of both pre-activations
-                else x = lane < 8 ? (ok ? expf(gb) : 1.f) : gb;
-                if (lane < 16) sm.al[hw][lane] = x;
+                const double y = p.input_raw ? 1.0 / (1.0 + exp(-(double)gb)) : exp((double)gb);      // sigmoid of both pre-activations
+                if (lane < 8) sm.al[hw][lane] = ok ? y : 1.0;
+                else if (lane < 16) sm.be[hw][lane & 7] = p.input_raw ? (ok ? (float)y : 0.f) : gb;
             }
             __syncwarp();
             if (base + NH * kBlk < it.row_end) load(it, row0 + NH * kBlk);
@@ -256,26 +259,21 @@ __device__ void helper(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& 
 #pragma unroll
             for (int i = 0; i < 4; ++i) dot[i] = (b0 ? s1[4 + i] : s1[i]) + __shfl_xor_sync(0xffffffffu, b0 ? s1[i] : s1[4 + i], 1);
             const int kind = sl >> 2, t = 2 * m + ((sl >> 1) & 1), i0 = 4 * (sl & 1);
-            float r[4] = {1.f, 1.f, 1.f, 1.f}, e[4] = {1.f, 1.f, 1.f, 1.f}, gt = 1.f, ge = 1.f;     // R(t, i), R(8, i), G_t, G_8
+            double suf[kBlk];                             // R(t, i): the alphas of the tokens i + 1 .. t (of the last t: to the block's end)
+            suf[kBlk - 1] = 1.;
 #pragma unroll
-            for (int x = 0; x < kBlk; ++x) {
-                const float ax = sm.al[hw][x];
-                if (x <= t) gt *= ax;
-                ge *= ax;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (x > i0 + i) { e[i] *= ax; if (x <= t) r[i] *= ax; }
-            }
-            const float bt = sm.al[hw][kBlk + t];
+            for (int x = kBlk - 1; x > 0; --x) suf[x - 1] = suf[x] * (x <= t ? sm.al[hw][x] : 1.);
+            const float bt = sm.be[hw][t], gt = (float)(suf[0] * sm.al[hw][0]);
             Coef& cf = sm.coef[buf][hw];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int ii = i0 + i;
-                sm.mn[hw][kind][ii][t] = kind ? (ii <= t ? r[i] * dot[i] : 0.f) : (ii < t ? -bt * (r[i] * dot[i]) : 0.f);
-                if (kind == 0 && t == 0) cf.rest[ii] = e[i];
+                const float r = (float)(i0 ? suf[4 + i] : suf[i]), rd = r * dot[i];
+                sm.mn[hw][kind][ii][t] = kind ? (ii <= t ? rd : 0.f) : (ii < t ? -bt * rd : 0.f);
+                if (kind == 0 && t == kBlk - 1) cf.rest[ii] = r;
             }
             if (i0 == 0) { cf.c1[kind][t] = kind ? 0.f : bt; cf.c2[kind][t] = kind ? gt : -bt * gt; }
-            if (lane == 0) cf.gend = ge;
+            if (kind == 0 && i0 == 0 && t == kBlk - 1) cf.gend = gt;
             __syncwarp();
             {
                 // lanes j, j + 8, ..: column j of the inverse, by forward substitution, and two rows of N times it
