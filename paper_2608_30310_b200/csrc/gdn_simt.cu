@@ -287,7 +287,11 @@ __device__ void helper(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>& 
                     for (int t2 = i + 1; t2 < kBlk; ++t2) x[t2] = fmaf(sm.mn[hw][0][i][t2], x[i], x[t2]);
                 float o0 = 0.f, o1 = 0.f;
 #pragma unroll
-                for (int i = 0; i < kBlk; ++i) { o0 = fmaf(sm.mn[hw][1][i][t0], x[i], o0); o1 = fmaf(sm.mn[hw][1][i][t0 + 4], x[i], o1); }
+                for (int i = 0; i < kBlk; ++i) {
+                    // (up to the token itself: zeros times later tokens' entries would be NaN where those are not finite)
+                    if (i < 4 && i <= t0) o0 = fmaf(sm.mn[hw][1][i][t0], x[i], o0);
+                    if (i <= t0 + 4) o1 = fmaf(sm.mn[hw][1][i][t0 + 4], x[i], o1);
+                }
                 cf.A[1][j][t0] = o0; cf.A[1][j][t0 + 4] = o1;
                 if (t0 == 0) {
 #pragma unroll
