@@ -1,7 +1,8 @@
 // Fast argument path of the Python binding.  A call's tensors are checked and marshalled here instead of in Python, where the
 // checks, the ctypes descriptor and the stream lookup cost some 10 us a call: more than the kernels of a one-request decoding step.
-// Whatever this code does not recognise as a correct call (a wrong type or shape, a workspace that has to grow) is answered with
-// None: the caller then takes the general path in Python, which raises the errors or makes the allocation.
+// Whatever this code does not recognise as a correct call (a wrong type or shape, a workspace that has to grow, a tensor whose sizes or
+// storage torch does not hand out, which it says with a C++ exception: none may pass a C entry) is answered with None: the caller
+// then takes the general path in Python, which raises the errors or makes the allocation.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -53,6 +54,21 @@ inline bool stream_of(PyObject* o, void*& st)
     return true;
 }
 
+using Entry = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
+template <Entry F> PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
+{
+    try {
+        return F(self, a, n);
+    } catch (...) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+}
+struct Ref {                                 // an owned reference, given back on every way out
+    PyObject* o;
+    ~Ref() { Py_XDECREF(o); }
+};
+
 // forward(which, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, init_state, workspace, status_word, kernel, stream, raw)
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
@@ -88,8 +104,8 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
     if (which != 2) {
         // the caller's scratch buffer as it is; growing it is the general path's
         if (a[11] == Py_None) Py_RETURN_NONE;
-        PyObject* b = PyObject_GetAttr(a[11], s_buf);
-        const at::Tensor* buf = b ? tensor(b) : nullptr;
+        const Ref b{PyObject_GetAttr(a[11], s_buf)};      // (the Workspace object keeps it)
+        const at::Tensor* buf = b.o ? tensor(b.o) : nullptr;
         const int64_t need = (int64_t)g_workspace_size(&d);
         const bool ok = buf && buf->is_cuda() && buf->element_size() == 1 && buf->numel() >= need;
         if (ok) {
@@ -97,7 +113,6 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
             d.workspace = (void*)(base + off);
             d.workspace_bytes = (size_t)buf->numel() - off;
         }
-        Py_XDECREF(b);                        // (the Workspace object keeps it)
         PyErr_Clear();
         if (!ok) Py_RETURN_NONE;
     }
@@ -148,8 +163,8 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
 }
 
 PyMethodDef methods[] = {
-    {"forward", (PyCFunction)(void (*)(void))forward, METH_FASTCALL, nullptr},
-    {"decode", (PyCFunction)(void (*)(void))decode, METH_FASTCALL, nullptr},
+    {"forward", (PyCFunction)(void (*)(void))guarded<forward>, METH_FASTCALL, nullptr},
+    {"decode", (PyCFunction)(void (*)(void))guarded<decode>, METH_FASTCALL, nullptr},
     {"bind", (PyCFunction)(void (*)(void))bind, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods};

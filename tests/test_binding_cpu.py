@@ -1,0 +1,60 @@
+"""The binding's native argument path, on the CPU: what it does not take is raised by the Python path behind it."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+# Each case ends in an error of torch's, the binding's or the library's.  They run in a child process: a C++ exception that leaves a C
+# function ends the interpreter.
+ODD_TENSORS = """
+import sys, torch, paper_2608_30310_b200 as gdn
+gdn.load_library()
+T, H, D = 8, 2, 64
+q, k, v = (torch.zeros(T, H, D) for _ in range(3))
+g, beta = torch.zeros(T, H), torch.zeros(T, H)
+cu = torch.tensor([0, T], dtype=torch.int32)
+
+def static(q=q, k=k, v=v, g=g, beta=beta, cu=cu, o=None):
+    gdn.gdn_tail_replay_static_scratch(q, k, v, g, beta, cu, 64, o, None)
+
+def nested():
+    n = torch.nested.nested_tensor([torch.zeros(3, D), torch.zeros(5, D)])
+    gdn.gdn_tail_replay(n, k, v, g, beta, cu, 64, None, None)
+
+def sparse():
+    static(q=q.to_sparse(), k=k.to_sparse(), v=v.to_sparse())
+
+def fake():
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        x = torch.empty(T, H, D)
+        static(x, x, x, torch.empty(T, H), torch.empty(T, H), torch.empty(2, dtype=torch.int32))
+
+def fake_decode():
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        x, s = torch.empty(T, H, D, device="cuda"), torch.empty(T, H, D, D, device="cuda")
+        y = torch.empty(T, H, device="cuda")
+        gdn.gdn_decode_step(x, x, x, y, y, s, x, s)
+
+def vmap():
+    torch.func.vmap(lambda x: static(x, x, x) or x)(torch.zeros(3, T, H, D))
+
+def host_memory():
+    static()                                   # no driver: no current stream; with one: the entry takes device memory only
+
+try:
+    {case}()
+except (RuntimeError, ValueError):
+    print("raised")
+"""
+
+
+@pytest.mark.parametrize("case", ["nested", "sparse", "fake", "fake_decode", "vmap", "host_memory"])
+def test_tensors_without_sizes_or_storage_raise(case):
+    r = subprocess.run([sys.executable, "-c", ODD_TENSORS.replace("{case}", case)], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.strip() == "raised", r.stdout + r.stderr[-2000:]
