@@ -64,6 +64,16 @@ template <Entry F> PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssiz
         Py_RETURN_NONE;
     }
 }
+// The library's call, with the other Python threads running: it may copy pageable memory, or wait for room in a launch queue that
+// only empties when a host callback of another thread's has run.  (The caller's frame holds the arguments.)
+template <typename F> PyObject* without_gil(F call)
+{
+    int32_t rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = call();
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
+}
 struct Ref {                                 // an owned reference, given back on every way out
     PyObject* o;
     ~Ref() { Py_XDECREF(o); }
@@ -101,10 +111,11 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
     d.kernel = (int32_t)kernel;
     d.input_stage = raw ? GDN_INPUT_RAW : GDN_INPUT_READY;
     d.init_state = (const float*)ptr(init);
+    Ref b{nullptr};
     if (which != 2) {
         // the caller's scratch buffer as it is; growing it is the general path's
         if (a[11] == Py_None) Py_RETURN_NONE;
-        const Ref b{PyObject_GetAttr(a[11], s_buf)};      // (the Workspace object keeps it)
+        b.o = PyObject_GetAttr(a[11], s_buf);              // (held over the call: another thread may let the Workspace grow)
         const at::Tensor* buf = b.o ? tensor(b.o) : nullptr;
         const int64_t need = (int64_t)g_workspace_size(&d);
         const bool ok = buf && buf->is_cuda() && buf->element_size() == 1 && buf->numel() >= need;
@@ -118,9 +129,9 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
     }
     d.status_word = (int32_t*)ptr(status);
     if (!stream_of(a[14], d.stream)) Py_RETURN_NONE;
-    const int32_t rc = g_forward[which](&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), (const float*)g->data_ptr(), (const float*)beta->data_ptr(),
-                                        (const int32_t*)cu->data_ptr(), (int32_t)chunk, ptr(o), (float*)ptr(st));
-    return PyLong_FromLong(rc);
+    const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr(), *pg = g->data_ptr(), *pb = beta->data_ptr(), *pc = cu->data_ptr();
+    void *po = ptr(o), *ps = ptr(st);
+    return without_gil([&]() { return g_forward[which](&d, pq, pk, pv, (const float*)pg, (const float*)pb, (const int32_t*)pc, (int32_t)chunk, po, (float*)ps); });
 }
 
 // decode(q, k, v, g, beta, state_in, out_o, state_out, stream)
@@ -144,9 +155,9 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n)
     d.num_seqs = (int32_t)N; d.total_tokens = N;
     d.memory = GDN_MEM_DEVICE; d.kernel = GDN_KERNEL_AUTO;
     if (!stream_of(a[8], d.stream)) Py_RETURN_NONE;
-    const int32_t rc = g_decode(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), (const float*)g->data_ptr(), (const float*)beta->data_ptr(),
-                                (const float*)in->data_ptr(), ptr(o), (float*)out->data_ptr());
-    return PyLong_FromLong(rc);
+    const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr(), *pg = g->data_ptr(), *pb = beta->data_ptr(), *pi = in->data_ptr();
+    void *po = ptr(o), *ps = out->data_ptr();
+    return without_gil([&]() { return g_decode(&d, pq, pk, pv, (const float*)pg, (const float*)pb, (const float*)pi, po, (float*)ps); });
 }
 
 // bind(gdn_tail_replay, gdn_full_prefill, gdn_tail_replay_static_scratch, gdn_decode_step, gdn_workspace_size): their addresses

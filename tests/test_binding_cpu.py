@@ -58,3 +58,28 @@ def test_tensors_without_sizes_or_storage_raise(case):
     r = subprocess.run([sys.executable, "-c", ODD_TENSORS.replace("{case}", case)], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert r.stdout.strip() == "raised", r.stdout + r.stderr[-2000:]
+
+
+# PyGILState_Check stands in for the library's entry points: it answers whether its thread holds the interpreter lock (1) or not (0,
+# which is also GDN_OK).
+LOCK = """
+import ctypes, torch, paper_2608_30310_b200 as gdn
+from paper_2608_30310_b200 import _binding as B
+gdn.load_library()
+check = ctypes.cast(ctypes.pythonapi.PyGILState_Check, ctypes.c_void_p).value
+size = ctypes.cast(gdn.load_library().gdn_workspace_size, ctypes.c_void_p).value
+B._native.bind(check, check, check, check, size)
+class Stream: cuda_stream = 0
+x, y = torch.zeros(8, 2, 64), torch.zeros(8, 2)
+cu = torch.tensor([0, 8], dtype=torch.int32)
+print(B._native.forward(2, x, x, x, y, y, cu, 64, x, None, None, None, None, 0, Stream(), False))
+if torch.cuda.is_available():
+    x, y, s = x.cuda(), y.cuda(), torch.zeros(8, 2, 64, 64, device="cuda")
+    print(B._native.decode(x, x, x, y, y, s, x, s, Stream()))
+"""
+
+
+def test_the_library_is_called_without_the_interpreter_lock():
+    r = subprocess.run([sys.executable, "-c", LOCK], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert set(r.stdout.split()) == {"0"}, r.stdout
