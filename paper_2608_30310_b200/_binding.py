@@ -156,6 +156,12 @@ def _forward(fn_name, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, *
         raise ValueError("out_o must be [T, Hv, dv] in the io dtype")
     if out_state is not None and (tuple(out_state.shape) != (N, Hv, dk, dv) or out_state.dtype != torch.float32):
         raise ValueError("out_state must be [N, Hv, dk, dv] fp32")
+    # (what the kernels read and write out of bounds otherwise; larger buffers serve)
+    if init_state is not None and (init_state.dtype != torch.float32 or init_state.numel() < N * Hv * dk * dv):
+        raise ValueError("init_state must be [N, Hv, dk, dv] fp32")
+    if status_word is not None and (status_word.numel() * status_word.element_size() < 4 or
+                                    not (status_word.is_cuda or status_word.is_pinned())):
+        raise ValueError("status_word must be an int32 that the device can write")
     desc = GdnDesc()
     desc.num_qk_heads, desc.num_v_heads, desc.head_k_dim, desc.head_v_dim = Hq, Hv, dk, dv
     desc.io_dtype, desc.num_seqs = io, N

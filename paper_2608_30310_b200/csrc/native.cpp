@@ -100,8 +100,10 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
         !fits_or_none(a[8], o, dt, cuda, T, Hv, dv) || !fits_or_none(a[9], st, at::kFloat, cuda, N, Hv, dk, dv))
         Py_RETURN_NONE;
     init = status = nullptr;
-    if (a[10] != Py_None && (!(init = tensor(a[10])) || init->is_cuda() != cuda || !init->is_contiguous())) Py_RETURN_NONE;
-    if (a[12] != Py_None && !(status = tensor(a[12]))) Py_RETURN_NONE;
+    if (a[10] != Py_None && (!(init = tensor(a[10])) || init->is_cuda() != cuda || !init->is_contiguous() || init->scalar_type() != at::kFloat ||
+                             init->numel() < N * Hv * dk * dv))
+        Py_RETURN_NONE;
+    if (a[12] != Py_None && (!(status = tensor(a[12])) || !status->is_cuda() || status->nbytes() < 4)) Py_RETURN_NONE;
 
     gdn_desc d = {};
     d.num_qk_heads = (int32_t)Hq; d.num_v_heads = (int32_t)Hv; d.head_k_dim = (int32_t)dk; d.head_v_dim = (int32_t)dv;

@@ -83,3 +83,14 @@ def test_the_library_is_called_without_the_interpreter_lock():
     r = subprocess.run([sys.executable, "-c", LOCK], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert set(r.stdout.split()) == {"0"}, r.stdout
+
+
+@pytest.mark.parametrize("name,value", [("init_state", "torch.zeros(1, 2, 64, 63)"), ("init_state", "torch.zeros(1, 2, 64, 64).double()"),
+                                        ("status_word", "torch.zeros(1, dtype=torch.int16)"), ("status_word", "torch.zeros(1, dtype=torch.int32)")])
+def test_start_state_and_status_word_are_checked(name, value):
+    """Too short, of another type, or not for the device to write (host memory that is not pinned)."""
+    import torch
+    import paper_2608_30310_b200 as gdn
+    x, y, cu = torch.zeros(8, 2, 64), torch.zeros(8, 2), torch.tensor([0, 8], dtype=torch.int32)
+    with pytest.raises(ValueError, match=name):
+        gdn.gdn_tail_replay_static_scratch(x, x, x, y, y, cu, 64, None, None, **{name: eval(value)})
