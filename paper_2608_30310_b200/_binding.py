@@ -261,8 +261,9 @@ def gdn_decode_step(q, k, v, g, beta, state_in, out_o, state_out, *, stream=None
                                ("state_out", state_out, (N, Hv, dk, dv), torch.float32)):
         if tuple(t.shape) != shape or t.dtype != dt or not t.is_contiguous() or not t.is_cuda:
             raise ValueError("%s must be a contiguous device tensor of shape %s and dtype %s" % (name, shape, dt))
-    if out_o is not None and (tuple(out_o.shape) != (N, Hv, dv) or out_o.dtype != q.dtype or not out_o.is_cuda):
-        raise ValueError("out_o must be [N, Hv, dv] in the io dtype on the device")
+    if out_o is not None and (tuple(out_o.shape) != (N, Hv, dv) or out_o.dtype != q.dtype or not out_o.is_cuda or
+                              not out_o.is_contiguous()):
+        raise ValueError("out_o must be a contiguous [N, Hv, dv] in the io dtype on the device")
     desc = GdnDesc()
     desc.num_qk_heads, desc.num_v_heads, desc.head_k_dim, desc.head_v_dim = Hq, Hv, dk, dv
     desc.io_dtype, desc.num_seqs, desc.total_tokens = io, N, N

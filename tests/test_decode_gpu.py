@@ -61,3 +61,13 @@ def test_replay_then_decode_equals_one_pass():
         o, st = _decode(tok, st)
         assert np.abs(o - ro[rows]).max() <= TOL["bf16"]["o_max_abs"]
     assert state_rel_fro(st, rst)[0] <= TOL["bf16"]["state_rel_fro"]
+
+
+def test_decode_step_refuses_a_strided_output():
+    """The kernel writes packed rows: a view with gaps would be filled wrongly, an expanded one out of bounds."""
+    import torch
+    import paper_2608_30310_b200 as gdn
+    x, y, s = torch.zeros(3, 2, 64, device="cuda"), torch.zeros(3, 2, device="cuda"), torch.zeros(3, 2, 64, 64, device="cuda")
+    for o in (torch.empty(3, 2, 128, device="cuda")[..., ::2], torch.empty(1, 2, 64, device="cuda").expand(3, 2, 64)):
+        with pytest.raises(ValueError, match="out_o"):
+            gdn.gdn_decode_step(x, x, x, y, y, s, o, s)
