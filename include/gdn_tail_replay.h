@@ -114,7 +114,10 @@ typedef struct gdn_desc {
 /*
  * Device scratch the two forward calls need for this descriptor (scheduler work list;
  * staging for every input and output when desc->memory == GDN_MEM_HOST; and, for calls with up to 37 chains on the tensor-core
- * path, some 300 KB per chain through which CTAs hand each other operands).
+ * path, some 300 KB per chain through which CTAs hand each other operands; a workspace without that last part still serves).
+ * A call may write the whole of its workspace until it has ended on the GPU.  Two calls that can overlap there (on different
+ * streams, or as replays of captured graphs) must not be given the same one, and it must stay allocated as long as a call, or a
+ * graph that captured one, can still run.
  * Returns 0 for an invalid descriptor.  Host-only; no CUDA call.
  */
 GDN_API size_t gdn_workspace_size(const gdn_desc* desc);

@@ -1,6 +1,7 @@
 """Binding of libgdn_tail_replay.so: argument marshalling only (csrc/native.cpp, with ctypes as the general path)."""
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from typing import Optional
@@ -81,7 +82,8 @@ def _bind_native(lib):
     import torch  # noqa: F401  (its libraries first)
     from . import _native as ext
     ext.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in
-               ("gdn_tail_replay", "gdn_full_prefill", "gdn_tail_replay_static_scratch", "gdn_decode_step", "gdn_workspace_size")))
+               ("gdn_tail_replay", "gdn_full_prefill", "gdn_tail_replay_static_scratch", "gdn_decode_step", "gdn_workspace_size")),
+             Workspace)
     _native = ext
 
 
@@ -107,20 +109,70 @@ def workspace_size(desc: GdnDesc) -> int:
     return int(load_library().gdn_workspace_size(ctypes.byref(desc)))
 
 
+def _on_stream(stream):
+    """Context in which torch allocates for ``stream`` (a torch stream, or any object with a ``cuda_stream`` handle)."""
+    import torch
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream.cuda_stream))
+    return torch.cuda.stream(stream)
+
+
 class Workspace:
-    """A caller-owned device scratch buffer (a torch uint8 tensor), grown on demand."""
+    """Device scratch of the calls that are given it: torch uint8 tensors, grown on demand, one per stream.
+
+    The CTAs of a call hand each other operands through the buffer, so that calls which may overlap on the GPU need one each: every
+    stream has its own, allocated for that stream.  ``buf`` is that of the stream that came first.  A captured call keeps the
+    address of its capture stream's buffer; buffers that device calls can have used are therefore kept when they are outgrown, as
+    long as the object lives.  Keep it as long as the graph, and let no replay overlap another, or a call on the capture stream."""
+
+    # More than any call on device memory needs (37 chains x 9 slots x 33,280 bytes and the request list); such a call takes a
+    # buffer of this size or, without the operand ring, a small one, so that few are ever outgrown.
+    SMALL, DEVICE = 64 << 10, 12 << 20
 
     def __init__(self, device="cuda"):
         self.device = device
-        self.buf = None
+        self.by_stream = {}                  # stream handle -> buffer; read by the native argument path
+        self.outgrown = []
 
-    def ensure(self, nbytes: int):
+    @property
+    def buf(self):
+        return next(iter(self.by_stream.values()), None)
+
+    @buf.setter
+    def buf(self, t):
+        """Takes ``t`` as the buffer of the current stream in place of all others (None: gives them back)."""
+        self.by_stream.clear()
+        self.outgrown.clear()
+        if t is not None:
+            import torch
+            self.by_stream[int(torch.cuda.current_stream().cuda_stream)] = t
+
+    def reserve(self, nbytes: int, stream, current: bool = False):
+        """The buffer of ``stream`` (``current``: known to be the current one), of at least ``nbytes`` bytes."""
         import torch
-        if self.buf is None or self.buf.numel() < nbytes:
-            self.buf = torch.empty(max(int(nbytes), 256) + 256, dtype=torch.uint8, device=self.device)
-        base = self.buf.data_ptr()
-        off = (-base) % 256
-        return base + off, self.buf.numel() - off
+        handle = int(stream.cuda_stream)
+        buf = self.by_stream.get(handle)
+        if buf is None or buf.numel() < nbytes:
+            if buf is not None and buf.numel() <= self.DEVICE + 256:
+                self.outgrown.append(buf)
+            size = max(int(nbytes), 256 if nbytes <= self.SMALL else self.DEVICE) + 256
+            with contextlib.nullcontext() if current else _on_stream(stream):
+                buf = torch.empty(size, dtype=torch.uint8, device=self.device)
+            self.by_stream[handle] = buf
+        return buf
+
+    def ensure(self, nbytes: int, stream=None):
+        """Address and size of the buffer of ``stream`` (default: the current one), of at least ``nbytes`` bytes."""
+        current = stream is None
+        if current:
+            import torch
+            stream = torch.cuda.current_stream()
+        return _aligned(self.reserve(nbytes, stream, current))
+
+
+def _aligned(buf):
+    off = (-buf.data_ptr()) % 256
+    return buf.data_ptr() + off, buf.numel() - off
 
 
 def _ptr(t) -> Optional[int]:
@@ -170,17 +222,23 @@ def _forward(fn_name, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, *
     desc.kernel = kernel
     desc.input_stage = GDN_INPUT_RAW if raw_inputs else GDN_INPUT_READY
     desc.init_state = _ptr(init_state)
+    desc.status_word = _ptr(status_word)
+    current = stream is None
+    if current:
+        stream = torch.cuda.current_stream()
+    desc.stream = int(stream.cuda_stream)
+    buf = None                                                  # (referenced until the call has returned)
     if fn_name == "gdn_tail_replay_static_scratch":
         desc.workspace, desc.workspace_bytes = None, 0          # ignored: the library's built-in scratch is used
     else:
         need = int(lib.gdn_workspace_size(ctypes.byref(desc)))
         if workspace is None:
             workspace = Workspace(device="cuda" if host else q.device)
-        desc.workspace, desc.workspace_bytes = workspace.ensure(need)
-    desc.status_word = _ptr(status_word)
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    desc.stream = int(stream.cuda_stream)
+        if type(workspace) is Workspace:
+            buf = workspace.reserve(need, stream, current)
+            desc.workspace, desc.workspace_bytes = _aligned(buf)
+        else:
+            desc.workspace, desc.workspace_bytes = workspace.ensure(need)
     rc = int(getattr(lib, fn_name)(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
                                    _ptr(cu_tail_lens), int(chunk), _ptr(out_o), _ptr(out_state)))
     if check and rc != GDN_OK:

@@ -18,7 +18,7 @@ using Decode = int32_t (*)(const gdn_desc*, const void*, const void*, const void
 Forward g_forward[3] = {};               // gdn_tail_replay, gdn_full_prefill, gdn_tail_replay_static_scratch
 Decode g_decode = nullptr;
 size_t (*g_workspace_size)(const gdn_desc*) = nullptr;
-PyObject *s_buf = nullptr, *s_cuda_stream = nullptr;
+PyObject *s_by_stream = nullptr, *s_cuda_stream = nullptr, *g_workspace_type = nullptr;
 
 inline const at::Tensor* tensor(PyObject* o) { return THPVariable_Check(o) ? &THPVariable_Unpack(o) : nullptr; }
 // contiguous, of type dt, on the side given by `cuda`, of shape {s...}
@@ -113,11 +113,14 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
     d.kernel = (int32_t)kernel;
     d.input_stage = raw ? GDN_INPUT_RAW : GDN_INPUT_READY;
     d.init_state = (const float*)ptr(init);
+    if (!stream_of(a[14], d.stream)) Py_RETURN_NONE;
     Ref b{nullptr};
     if (which != 2) {
-        // the caller's scratch buffer as it is; growing it is the general path's
-        if (a[11] == Py_None) Py_RETURN_NONE;
-        b.o = PyObject_GetAttr(a[11], s_buf);              // (held over the call: another thread may let the Workspace grow)
+        // the Workspace's buffer for this stream as it is; making or growing it is the general path's
+        if ((PyObject*)Py_TYPE(a[11]) != g_workspace_type) Py_RETURN_NONE;
+        const Ref map{PyObject_GetAttr(a[11], s_by_stream)}, key{PyLong_FromVoidPtr(d.stream)};
+        if (map.o && key.o && PyDict_Check(map.o)) b.o = PyDict_GetItemWithError(map.o, key.o);
+        Py_XINCREF(b.o);                                  // (held over the call: another thread may let the Workspace grow)
         const at::Tensor* buf = b.o ? tensor(b.o) : nullptr;
         const int64_t need = (int64_t)g_workspace_size(&d);
         const bool ok = buf && buf->is_cuda() && buf->element_size() == 1 && buf->numel() >= need;
@@ -130,7 +133,6 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n)
         if (!ok) Py_RETURN_NONE;
     }
     d.status_word = (int32_t*)ptr(status);
-    if (!stream_of(a[14], d.stream)) Py_RETURN_NONE;
     const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr(), *pg = g->data_ptr(), *pb = beta->data_ptr(), *pc = cu->data_ptr();
     void *po = ptr(o), *ps = ptr(st);
     return without_gil([&]() { return g_forward[which](&d, pq, pk, pv, (const float*)pg, (const float*)pb, (const int32_t*)pc, (int32_t)chunk, po, (float*)ps); });
@@ -162,16 +164,19 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n)
     return without_gil([&]() { return g_decode(&d, pq, pk, pv, (const float*)pg, (const float*)pb, (const float*)pi, po, (float*)ps); });
 }
 
-// bind(gdn_tail_replay, gdn_full_prefill, gdn_tail_replay_static_scratch, gdn_decode_step, gdn_workspace_size): their addresses
+// bind(gdn_tail_replay, gdn_full_prefill, gdn_tail_replay_static_scratch, gdn_decode_step, gdn_workspace_size, Workspace): the addresses of
+// the library's functions, and the class whose buffers are looked up here
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    if (n != 5) { PyErr_SetString(PyExc_TypeError, "five addresses"); return nullptr; }
+    if (n != 6) { PyErr_SetString(PyExc_TypeError, "five addresses and a class"); return nullptr; }
     void* p[5];
     for (int i = 0; i < 5; ++i) p[i] = PyLong_AsVoidPtr(a[i]);
     if (PyErr_Occurred()) return nullptr;
     for (int i = 0; i < 3; ++i) g_forward[i] = (Forward)p[i];
     g_decode = (Decode)p[3];
     g_workspace_size = (size_t (*)(const gdn_desc*))p[4];
+    Py_INCREF(a[5]);
+    Py_XSETREF(g_workspace_type, a[5]);
     Py_RETURN_NONE;
 }
 
@@ -186,7 +191,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods};
 
 PyMODINIT_FUNC PyInit__native()
 {
-    s_buf = PyUnicode_InternFromString("buf");
+    s_by_stream = PyUnicode_InternFromString("by_stream");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
     return PyModule_Create(&module);
 }

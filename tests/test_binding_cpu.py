@@ -68,7 +68,7 @@ from paper_2608_30310_b200 import _binding as B
 gdn.load_library()
 check = ctypes.cast(ctypes.pythonapi.PyGILState_Check, ctypes.c_void_p).value
 size = ctypes.cast(gdn.load_library().gdn_workspace_size, ctypes.c_void_p).value
-B._native.bind(check, check, check, check, size)
+B._native.bind(check, check, check, check, size, gdn.Workspace)
 class Stream: cuda_stream = 0
 x, y = torch.zeros(8, 2, 64), torch.zeros(8, 2)
 cu = torch.tensor([0, 8], dtype=torch.int32)
@@ -94,3 +94,30 @@ def test_start_state_and_status_word_are_checked(name, value):
     x, y, cu = torch.zeros(8, 2, 64), torch.zeros(8, 2), torch.tensor([0, 8], dtype=torch.int32)
     with pytest.raises(ValueError, match=name):
         gdn.gdn_tail_replay_static_scratch(x, x, x, y, y, cu, 64, None, None, **{name: eval(value)})
+
+
+class _Stream:
+    def __init__(self, handle):
+        self.cuda_stream = handle
+
+
+def test_every_stream_has_a_buffer_of_its_own(monkeypatch):
+    import contextlib
+    import paper_2608_30310_b200 as gdn
+    from paper_2608_30310_b200 import _binding as B
+    entered = []
+    monkeypatch.setattr(B, "_on_stream", lambda s: entered.append(s.cuda_stream) or contextlib.nullcontext())
+    ws = gdn.Workspace(device="cpu")
+    a = ws.reserve(512, _Stream(0))
+    b = ws.reserve(512, _Stream(7))
+    assert entered == [0, 7] and a.data_ptr() != b.data_ptr()                  # allocated for the stream that uses it
+    assert ws.reserve(500, _Stream(7)) is b and ws.buf is a and len(entered) == 2
+    ring = ws.reserve(9 << 20, _Stream(7))
+    assert ring.numel() >= 12 << 20 and ws.by_stream == {0: a, 7: ring}
+    assert any(x is b for x in ws.outgrown)                                    # (a captured call may have its address)
+    big = ws.reserve(30 << 20, _Stream(7))
+    assert any(x is ring for x in ws.outgrown) and ws.reserve(1 << 20, _Stream(7)) is big
+    ws.reserve(60 << 20, _Stream(7))
+    assert not any(x is big for x in ws.outgrown)                              # staging of host-memory calls is given back
+    base, size = ws.ensure(512, _Stream(0))
+    assert base % 256 == 0 and a.data_ptr() <= base and base + size == a.data_ptr() + a.numel()
