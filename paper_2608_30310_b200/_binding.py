@@ -77,10 +77,21 @@ def load_library():
 
 
 def _bind_native(lib):
-    """The extension that checks and marshals a call's tensors; it takes the library's entry points by address."""
+    """The extension that checks and marshals a call's tensors; it takes the library's entry points by address.  It is built for one
+    version of torch; with another, calls are marshalled in Python (the CUDA library itself knows nothing of torch)."""
     global _native
-    import torch  # noqa: F401  (its libraries first)
-    from . import _native as ext
+    import torch
+    try:
+        from . import _native as ext
+        why = "" if ext.built_for_torch == torch.__version__ else "it was built for torch %s" % ext.built_for_torch
+    except (ImportError, AttributeError) as exc:
+        why = str(exc)
+    if why:
+        import warnings
+        warnings.warn("the native argument path is not used (%s), which costs some 10 us a call: run "
+                      "`python -m paper_2608_30310_b200.build`" % why, RuntimeWarning, stacklevel=3)
+        _native = False
+        return
     ext.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in
                ("gdn_tail_replay", "gdn_full_prefill", "gdn_tail_replay_static_scratch", "gdn_decode_step", "gdn_workspace_size")),
              Workspace)
@@ -255,7 +266,7 @@ def _call(which, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, *, tot
     if _native is None:
         load_library()
     rc = None
-    if total_tokens is None:
+    if total_tokens is None and _native:
         rc = _native.forward(which, q, k, v, g, beta, cu_tail_lens, chunk, out_o, out_state, init_state, workspace, status_word,
                              kernel, stream, raw_inputs)
     if rc is None:
@@ -299,7 +310,7 @@ def gdn_decode_step(q, k, v, g, beta, state_in, out_o, state_out, *, stream=None
     same tensor), out_o [N, Hv, dv] or None.  Device tensors only."""
     if _native is None:
         load_library()
-    rc = _native.decode(q, k, v, g, beta, state_in, out_o, state_out, stream)
+    rc = _native.decode(q, k, v, g, beta, state_in, out_o, state_out, stream) if _native else None
     if rc is not None:
         if rc != GDN_OK and check:
             raise GdnError(rc, "gdn_decode_step")

@@ -21,20 +21,26 @@ NATIVE_SRC = os.path.join(CSRC, "native.cpp")
 
 
 def build_native(force: bool = False) -> str:
-    """Compile the binding's argument path (a CPython extension on torch's C++ tensors; host code only)."""
-    deps = [NATIVE_SRC, os.path.join(ROOT, "include", "gdn_tail_replay.h")]
-    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
-        return NATIVE
+    """Compile the binding's argument path (a CPython extension on torch's C++ tensors; host code only), for the torch and Python at hand."""
     import sysconfig
     import torch
+    deps = [NATIVE_SRC, os.path.join(ROOT, "include", "gdn_tail_replay.h")]
+    stamp, built_for = os.path.join(ROOT, "build", "native.txt"), "%s %s" % (torch.__version__, sys.version)
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps) and \
+            os.path.exists(stamp) and open(stamp).read() == built_for:
+        return NATIVE
     from torch.utils.cpp_extension import include_paths
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     tmp = NATIVE + ".tmp.%d" % os.getpid()
     inc = [x for d in include_paths("cuda") + [sysconfig.get_paths()["include"]] for x in ("-isystem", d)]
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+                           '-DBUILT_FOR_TORCH="%s"' % torch.__version__, "-I", os.path.join(ROOT, "include"),
                            *inc, NATIVE_SRC, "-o", tmp, "-L" + lib, "-Wl,-rpath," + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
     os.replace(tmp, NATIVE)
+    os.makedirs(os.path.dirname(stamp), exist_ok=True)
+    with open(stamp, "w") as f:
+        f.write(built_for)
     return NATIVE
 
 

@@ -193,5 +193,7 @@ PyMODINIT_FUNC PyInit__native()
 {
     s_by_stream = PyUnicode_InternFromString("by_stream");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
-    return PyModule_Create(&module);
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for_torch", BUILT_FOR_TORCH) < 0) { Py_DECREF(m); return nullptr; }
+    return m;
 }

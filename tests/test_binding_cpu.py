@@ -121,3 +121,34 @@ def test_every_stream_has_a_buffer_of_its_own(monkeypatch):
     assert not any(x is big for x in ws.outgrown)                              # staging of host-memory calls is given back
     base, size = ws.ensure(512, _Stream(0))
     assert base % 256 == 0 and a.data_ptr() <= base and base + size == a.data_ptr() + a.numel()
+
+
+OTHER_TORCH = """
+import sys, types, warnings, torch, paper_2608_30310_b200 as gdn
+from paper_2608_30310_b200 import _binding as B
+ext = {ext}
+sys.modules["paper_2608_30310_b200._native"] = ext
+if ext is not None: gdn._native = ext
+with warnings.catch_warnings(record=True) as seen:
+    warnings.simplefilter("always")
+    assert gdn.tail_select(100, 0.07) == 7
+assert any("native argument path" in str(w.message) for w in seen)
+x, y = torch.zeros(8, 2, 64), torch.zeros(8, 2)
+class Stream: cuda_stream = 0
+try:
+    gdn.gdn_tail_replay_static_scratch(x, x, x, y, y, torch.tensor([0, 8], dtype=torch.int32), 64, None, None, stream=Stream())
+except gdn.GdnError as e:
+    print(e.status)
+try:
+    gdn.gdn_decode_step(x, x, x, y, y, x, None, x)
+except ValueError:
+    print("checked")
+"""
+
+
+@pytest.mark.parametrize("ext", ["types.SimpleNamespace(built_for_torch='1.0')", "types.SimpleNamespace()", "None"])
+def test_an_extension_for_another_torch_is_not_used(ext):
+    """The library still loads and the Python path takes the calls (host memory: unsupported by that entry, -2)."""
+    r = subprocess.run([sys.executable, "-c", OTHER_TORCH.replace("{ext}", ext)], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == ["-2", "checked"], r.stdout + r.stderr[-2000:]
