@@ -248,22 +248,24 @@ struct Ctx {
     // A ready barrier costs a few cycles, a try_wait that has to wait returns about 90 cycles after the last arrival.  It does not
     // sleep all that time: waiting warps poll, and half of the instructions of a fused CTA were polls.  There, one warp of a
     // group waits for the group, and the others at a named barrier, which does sleep.
-    __device__ __forceinline__ void wait(int i, uint32_t parity) const
+    // False where the wait gave up.
+    __device__ __forceinline__ bool wait(int i, uint32_t parity) const
     {
         const uint32_t b = bar(i);
-        if (!mbar_try_wait(b, parity)) wait_slow(b, parity, misc);
+        return mbar_try_wait(b, parity) || wait_slow(b, parity, misc);
     }
     // kept out of line: the kernel has many wait sites and its static code size matters
-    __device__ __noinline__ static void wait_slow(uint32_t b, uint32_t parity, Misc* misc)
+    __device__ __noinline__ static bool wait_slow(uint32_t b, uint32_t parity, Misc* misc)
     {
         uint64_t t0 = 0;
         for (uint32_t n = 0; !mbar_try_wait(b, parity); ++n) {
             if ((n & 15u) != 0u) continue;
-            if (misc->abort) return;
+            if (misc->abort) return false;
             const uint64_t t = globaltimer_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > misc->timeout_ns) { misc->abort = 1u; return; }
+            if (t - t0 > misc->timeout_ns) { misc->abort = 1u; return false; }
         }
+        return true;
     }
     // for barriers that the other CTAs of the cluster arrive on
     __device__ __forceinline__ void wait_cluster(int i, uint32_t parity) const
@@ -285,10 +287,17 @@ struct Ctx {
 
 // Hand-overs from the epilogue warps of a chain CTA to its MMA warp, on named barriers (a hardware barrier wakes its
 // waiter sooner than an mbarrier does, and these sit on the serial path of a chain).  The waits cannot outlast
-// the bounded mbarrier waits: the arriving warps run through their loop whatever happens.
+// the bounded mbarrier waits: the arriving warps run through their loop whatever happens.  They must not run ahead of the MMA
+// warp, though: a second arrival on a barrier before the MMA warp's first would complete it without that warp, and leave it waiting
+// for arrivals that have been used up.  The mbarrier waits between two arrivals see to that until one of them gives up; from
+// then on (`dead`) a warp stays at every hand-over until the MMA warp has come.  Both sides pass the hand-overs in the same order.
 enum HandOver { HB_SBF0 = 8, HB_SBF1 = 9, HB_DP = 10, HB_D = 11 };
-template <int WARPS> __device__ __forceinline__ void hand_over_arrive(int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(WARPS * 32 + 32) : "memory"); }
 template <int WARPS> __device__ __forceinline__ void hand_over_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(WARPS * 32 + 32) : "memory"); }
+template <int WARPS> __device__ __forceinline__ void hand_over_arrive(int id, bool dead)
+{
+    if (dead) hand_over_sync<WARPS>(id);
+    else asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(WARPS * 32 + 32) : "memory");
+}
 
 // One arrival per warp: every lane has fenced its own TMEM / shared-memory accesses, the warp converges,
 // lane 0 arrives.  (A full-warp arrive is 32 serialized shared-memory atomics on one address.)
@@ -1154,6 +1163,7 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
     const uint32_t tl = cx.tmem + ((uint32_t)(w4 * 32) << 16);
     Misc* misc = cx.misc;
     const bool has_init = p.init_state != nullptr;
+    bool dead = false;                                    // a wait of this warp (fused CTA: of its group) has given up
 
     uint32_t j = 0;
 #pragma unroll 1
@@ -1173,7 +1183,7 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
         // ---- chain start: the previous chain's final state has been read out (below); a start state, if given, goes
         // into tensor memory as the first chunk's bf16 operand and, multiplied by the chunk's decay, as the fp32 state
         if (has_init) init_chain<CL>(cx, p.init_state + st_off, j, tl, cs, dv);
-        hand_over_arrive<WH>(HB_SBF0 + cs);                  // the start state of step j is in place
+        hand_over_arrive<WH>(HB_SBF0 + cs, dead);            // the start state of step j is in place
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c, ++j) {
             const bool last = c == nchunks - 1;
@@ -1183,9 +1193,10 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
             const uint32_t acc1 = tl + TM_ACC1 + 32 * cs;
             if (CL || w4 == 0) {
                 cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);   // factors of this chunk are published
-                cx.wait(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)(j & 1u), CL ? j & 1u : (j >> 1) & 1u);
+                dead |= !cx.wait(CL ? (int)CB_MMA1 : FB_MMA1_0 + (int)(j & 1u), CL ? j & 1u : (j >> 1) & 1u);
             }
-            if (!CL) half_sync();
+            if (CL) dead = __any_sync(0xffffffffu, dead);
+            else { half_sync(); dead = misc->abort != 0u; }
             const float cfin = dc.cfin;
             tc_fence_after();
             // The accumulator holds Delta~^T = Delta^T diag(beta)^-1: times beta e^(G_C - G) / c it is the A operand of the
@@ -1211,7 +1222,7 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
                 }
                 tmem_st_wait();
                 tc_fence_before();
-                hand_over_arrive<WA>(HB_DP);
+                hand_over_arrive<WA>(HB_DP, dead);
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
 #pragma unroll
@@ -1220,16 +1231,17 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
                 }
                 tmem_st_wait();
                 tc_fence_before();
-                hand_over_arrive<WA>(HB_D);
+                hand_over_arrive<WA>(HB_D, dead);
             }
 
             // ---- state: bf16 copy for the next chunk's MMAs, or the final state ------------------------------
             // if the next chunk starts from a rescaled state, the stored state is multiplied by wb on the way
             if (CL || w4 == 0) {
                 if (!last) cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)((j + 1) & 3u), ((j + 1) >> 2) & 1u);
-                cx.wait((CL ? CB_STATE0 : FB_STATE0) + cs, j & 1u);
+                dead |= !cx.wait((CL ? CB_STATE0 : FB_STATE0) + cs, j & 1u);
             }
-            if (!CL) half_sync();
+            if (CL) dead = __any_sync(0xffffffffu, dead);
+            else { half_sync(); dead = misc->abort != 0u; }
             float wb = 1.f;
             bool rescale = false;
             if (!last) {
@@ -1253,7 +1265,7 @@ __device__ void chain_epilogue(const Ctx& cx, const TcParams* prm, int warp, int
             }
             tmem_st_wait();
             tc_fence_before();
-            if (!last) hand_over_arrive<WH>(HB_SBF0 + cs);    // (a chain's first chunk is announced at the chain start)
+            if (!last) hand_over_arrive<WH>(HB_SBF0 + cs, dead);    // (a chain's first chunk is announced at the chain start)
         }
     }
 }
