@@ -26,7 +26,6 @@
 namespace gdn {
 namespace {
 
-using ptx::fma_f32x2;
 using ptx::mul_f32x2;
 
 template <typename T> __device__ __forceinline__ T from_f32(float x);
@@ -593,8 +592,10 @@ cudaError_t launch_shape(const Problem& p, const Sched& s, cudaStream_t stream)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // Rows per warp: 16 have the lowest cost per row, 8 and 4 the lowest time per token.  The finer splits pay while they find idle
-    // SMs: 4 rows (16 per CTA) up to one CTA per SM, 8 (32 per CTA) up to one and a half.  us for 1,000 tokens at d = 128:
-    // 1,024 rows 138 / 193 / 282 (4 / 8 / 16 rows a warp), 4,096 rows 358 / 195 / 279, 8,192 rows 714 / 305 / 281.
+    // SMs: 4 rows (8 per CTA) up to two CTAs per SM, 8 (32 per CTA) up to one and a half.  us for one request of 1,000 tokens at
+    // d = 128 with 4 / 8 / 16 rows a warp: 1,024 rows 128 / 193 / 275, 2,304 rows 175 / 194 / 276, 2,432 rows 300 / 194 / 276, 4,096 rows
+    // 347 / 195 / 276, 5,120 to 7,040 rows 474-527 / 310 / 277, 8,192 rows 700 / 310 / 278.  (With equal lengths the second line could
+    // lie at one CTA per SM, 4,736 rows.)
     const long long rows = (long long)p.num_seqs * p.Hv * DV;
     // Requests that do not fill a block on average: the instance that leaves out tokens past the end (1,000 requests of 1-8 tokens,
     // 32 heads: 443 -> 365 us at d = 64, 1,565 -> 1,232 us at d = 128; where blocks are full its branches cost 2 %).

@@ -948,6 +948,9 @@ __device__ void chain_receiver(const Ctx& cx, const TcParams* prm)
         const uint32_t slot = j % NSLOT;
         if (j >= NSLOT) {
             cx.wait(CB_DONE0 + (int)((j - NSLOT) & 3u), ((j - NSLOT) >> 2) & 1u);      // (its operands have landed long ago)
+            // A relaxed arrival suffices for the credit: it hands over nothing that was written here.  All that the prep CTA's next
+            // store into the ring slot must not overtake is the bulk load out of it, and that is over: the chunk is done, its
+            // products have read the operands, which they could only after all of the load's bytes had been counted in.
             const uint32_t f = j - NSLOT;
             if (leader) mbar_arrive_remote(map_to_rank(cx.bar(PB_CREDIT0 + (int)((f / R) % (kRingSlots / R))), 1u + f % R));
         }
@@ -1590,20 +1593,23 @@ cudaError_t launch(TcParams& prm, Maps& m, cudaStream_t stream)
     int dev = 0, cap = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const long long items = (long long)prm.p.num_seqs * prm.p.Hv;
+    const Problem& p = prm.p;
+    auto out_map = [&](uint32_t halves) { return make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, halves); };
+    const long long items = (long long)p.num_seqs * p.Hv;
     if (prm.s.ring && items <= kRingClusters) {
         e = capacity<RAW, true>(dev, &cap);
         if (e != cudaSuccess) return e;
         if (items <= cap) {
-            const Problem& p = prm.p;
             if (!make_map(&m.qt, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) || !make_map(&m.kt, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 2) ||
-                !make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2))
+                !out_map(2))
                 return cudaErrorUnknown;
             return launch_as<RAW, true>(prm, items, m, stream);
         }
     }
     e = capacity<RAW, false>(dev, &cap);
     if (e != cudaSuccess) return e;
+    if (!out_map(1)) return cudaErrorUnknown;
+    m.qt = m.q; m.kt = m.k;                                     // (not used by this form)
     return launch_as<RAW, false>(prm, items < cap ? items : cap, m, stream);
 }
 
@@ -1629,10 +1635,8 @@ cudaError_t launch_tcgen05(const Problem& p, const Sched& s, cudaStream_t stream
     if (!tcgen05_supported(p)) return cudaErrorNotSupported;
     Maps m;
     if (!make_map(&m.q, p.q, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 1) || !make_map(&m.k, p.k, (uint64_t)p.total_tokens, (uint64_t)p.Hq, 1) ||
-        !make_map(&m.v, p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2) ||
-        !make_map(&m.o, p.out_o ? p.out_o : p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 1))
+        !make_map(&m.v, p.v, (uint64_t)p.total_tokens, (uint64_t)p.Hv, 2))
         return cudaErrorUnknown;
-    m.qt = m.q; m.kt = m.k;
     TcParams prm;
     prm.p = p; prm.s = s;
     prm.wait_timeout_ns = g_wait_timeout_ns; prm.skip_kq_load = g_skip_kq_load;

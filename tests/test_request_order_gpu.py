@@ -27,3 +27,14 @@ def test_order_of_requests(io, d, n, hv):
     assert launches == 2
     np.testing.assert_allclose(o2, o, rtol=0, atol=0)
     np.testing.assert_allclose(st2, st, rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("io,d", [("bf16", 128), ("f32", 64)])
+def test_more_items_than_a_cta_keeps_in_its_table(io, d):
+    """5,000 short requests x 2 heads: 68 rounds of chains on 148 SMs, past the 64 that a CTA of the tensor-core kernel looks up at its
+    start."""
+    lens = [int(x) for x in np.random.default_rng(77).integers(0, 4, size=5000)]
+    inp = make_inputs(lens, 1, 2, d, d, io, seed=91_000)
+    o, st, launches = run_library(inp, canary=True)
+    assert launches == 2
+    assert_parity(inp, o, st, *oracle.gdn_forward_inputs(inp))
