@@ -32,10 +32,12 @@ WORKLOAD = "concurrent_hits_32req_tails_U400-3300_Hq16_Hv32_d128_bf16_chunk64"
 BYTES_PER_TOKEN_HEAD = 776.0        # q,k shared by 2 v-heads + v + o in bf16, g and beta in fp32
 FLOPS_PER_TOKEN_HEAD = 139264.0     # 6 dk dv + C (3 dk + 2 dv), triangular products at half cost
 STATE_BYTES_PER_CHAIN = 128 * 128 * 4
-# DRAM bytes per token*head of the dominant kernel, from the committed ncu capture of the 8-request case
-# (profiles/gdn_tc_kernel_concurrent_hits_8req.md: dram read + write = 252.8 MB for 346,944 token*heads,
-# final states included); traffic grows in proportion to the units a launch processes.
-NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD = 728.6
+# DRAM bytes that the dominant kernel reads per token*head, from the committed ncu capture of the 8-request case
+# (profiles/gdn_tc_kernel_concurrent_hits_8req.md: 183.2 MB for 346,944 token*heads); the bytes read grow in proportion to the units a
+# launch processes.  The capture's written bytes are not used: it ends with part of the outputs still in L2.  Outputs (256 B) and
+# final states are counted once each instead.
+NCU_READ_BYTES_PER_TOKEN_HEAD = 528.0
+OUTPUT_BYTES_PER_TOKEN_HEAD = 256.0
 
 
 def load_peaks():
@@ -353,8 +355,8 @@ def main():
     ms_per_step = total_ms / args.steps
     value = units_all / (ms_per_step * 1e-3)
 
-    # roofline of the dominant kernel (the chunkwise forward); each call = a ~2 us scheduler kernel
-    # + this kernel, timed together with events on the launching stream, so `achieved` is a floor
+    # roofline of the dominant kernel (the chunkwise forward), from the whole call timed with events on the launching stream
+    # (up to 64 requests the call is this kernel alone), so `achieved` is a floor
     peaks = load_peaks()
     kern_ms = statistics.mean(call_ms)
     alg_bytes = units_per_step * BYTES_PER_TOKEN_HEAD + N * Hv * STATE_BYTES_PER_CHAIN
@@ -366,8 +368,8 @@ def main():
         "bound": "hbm" if t_hbm >= t_tc else "tensor",
         "achieved": achieved_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
         "frac": achieved_gbs / peaks["hbm_gbs"], "peak_source": peaks["source"],
-        "traffic": (NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD * units_per_step
-                    if NCU_TRAFFIC_BYTES_PER_TOKEN_HEAD else None),
+        "traffic": ((NCU_READ_BYTES_PER_TOKEN_HEAD + OUTPUT_BYTES_PER_TOKEN_HEAD) * units_per_step
+                    + N * Hv * STATE_BYTES_PER_CHAIN),
         "kernel_ms": kern_ms, "algorithmic_bytes": alg_bytes, "algorithmic_flops": alg_flops,
         "achieved_tflops": alg_flops / (kern_ms * 1e-3) / 1e12, "roofline_ms": max(t_hbm, t_tc) * 1e3,
         "frac_of_nominal_8000_gbs": achieved_gbs / 8000.0,      # context: the nominal HBM3e figure, not the denominator
