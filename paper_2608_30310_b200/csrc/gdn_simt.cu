@@ -9,7 +9,7 @@
 // which is 3 dk dv FMAs per token and head; the rows of S are independent of each other.
 //
 // A CTA owns a slice of 2 RPT NW rows of one chain (request, v-head): NW warps of 2 RPT rows each.  Sixteen lanes share RPT
-// rows, DK / 16 columns per lane, all in registers.  The dot products of a token are reduced over the sixteen lanes by a
+// rows, DK / 16 columns per lane, all in registers (RPT = 1, for calls with few rows: see compute_few).  The dot products of a token are reduced over the sixteen lanes by a
 // reduce-scatter that leaves each lane one of the 2 RPT values (a row's r or p) for all eight tokens, so that the 8 x 8 products run
 // inside a lane; eight tokens share the latency (one token at a time, each waited for a shuffle reduction: 400 ns a token).  NH helper warps
 // run ahead by a stage of 8 NH tokens: they load k, q, g and beta, apply the input stage if asked, and form the 8 x 8
@@ -546,8 +546,140 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
     }
 }
 
+// ---- compute warp of calls with few rows: one row per sixteen lanes (RPT = 1) -------------------------------------------------
+// With a warp to a scheduler nothing but the chain of dependent instructions of a block counts: every lane has all eight r or p of its
+// row, delta goes from lane to lane by shuffles, and k serves the products and the update from registers.  us for one request of 512
+// tokens: d = 64 (256 rows) 50.8 with two rows per sixteen lanes, 34.4 so, 37.3 with the sums scattered until a lane has one token
+// (half the instructions, but one behind the other), 38.5 so and with k and q loaded a block ahead; d = 128: 67.2, 46.3, 47.5, 47.9.
+template <int DK, int DV, typename T, int NW, int NH>
+__device__ void compute_few(const Problem& p, const Sched& s, Smem<DK, 1, NW, NH>& sm, Walk<DV / (2 * NW)> walk, int warp, int lane)
+{
+    constexpr int NTHR = (NW + NH) * 32, R = 2 * NW, NC = DK / 64;
+    const int l = lane & 15, rg = lane >> 4, type = l >> 3;                // type 1: the outputs' lanes, 0: delta's
+    const T* __restrict__ vg = (const T*)p.v;
+    T* __restrict__ og = (T*)p.out_o;
+    float* const vs = &sm.v[warp][0][0];                  // [row][token]
+    uint32_t stage = 0;
+    Item it;
+    while (walk.next(p, s, sm.requests, it)) {
+        const int j0 = it.slice * R + warp * 2;           // first row (value index) of the warp
+        const size_t st_off = ((size_t)it.n * p.Hv + it.h) * DK * DV + j0 + rg;
+        float2 S[2 * NC];                                 // piece c: columns 64 c + 4 l .. + 3
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float x = p.init_state ? p.init_state[st_off + (size_t)(64 * c + 4 * l + e) * DV] : 0.f;
+                if (e & 1) S[2 * c + (e >> 1)].y = x; else S[2 * c + (e >> 1)].x = x;
+            }
+        const size_t vstride = (size_t)p.Hv * DV;
+        // lanes 0-15: v of the next block, token lane / 2, row lane % 2;  lanes 8-15 of either half: a token's output each
+        const T* vp = vg + ((size_t)(it.row_begin + (l >> 1)) * p.Hv + it.h) * DV + j0 + (l & 1);
+        T* op = og ? og + ((size_t)(it.row_begin + (l & 7)) * p.Hv + it.h) * DV + j0 + rg : nullptr;
+        VNext<T, 1> vn;
+        int left = it.row_end - it.row_begin;             // tokens from the current block on
+        vn.load(vp, rg == 0 && (l >> 1) < left);
+#pragma unroll 1
+        for (; left > 0; ++stage) {
+            const int buf = (int)(stage % kBufs);
+            bar_sync<BAR_FULL>(buf, NTHR);
+#pragma unroll 1
+            for (int sb = 0; sb < NH && left > 0; ++sb, left -= kBlk) {
+                const float (*ks)[Smem<DK, 1, NW, NH>::LD] = &sm.k[buf][sb * kBlk];
+                const float (*qs)[Smem<DK, 1, NW, NH>::LD] = &sm.q[buf][sb * kBlk];
+                const Coef& cf = sm.coef[buf][sb];
+                if (rg == 0) vs[(l & 1) * kBlk + (l >> 1)] = vn.get(0);
+                vp += kBlk * vstride;
+                vn.load(vp, rg == 0 && (l >> 1) < left - kBlk);
+                float4 k4[kBlk][NC];
+                float ak[kBlk], aq[kBlk];
+#pragma unroll
+                for (int t = 0; t < kBlk; ++t) {
+                    float2 x = make_float2(0.f, 0.f), y = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        k4[t][c] = *reinterpret_cast<const float4*>(&ks[t][64 * c + 4 * l]);
+                        const float4 q4 = *reinterpret_cast<const float4*>(&qs[t][64 * c + 4 * l]);
+                        ptx::fma_f32x2(x.x, x.y, S[2 * c].x, S[2 * c].y, k4[t][c].x, k4[t][c].y);
+                        ptx::fma_f32x2(y.x, y.y, S[2 * c].x, S[2 * c].y, q4.x, q4.y);
+                        ptx::fma_f32x2(x.x, x.y, S[2 * c + 1].x, S[2 * c + 1].y, k4[t][c].z, k4[t][c].w);
+                        ptx::fma_f32x2(y.x, y.y, S[2 * c + 1].x, S[2 * c + 1].y, q4.z, q4.w);
+                    }
+                    ak[t] = x.x + x.y; aq[t] = y.x + y.y;
+                }
+                __syncwarp();                             // (v is there)
+                float A[kBlk][kBlk], y[kBlk], e[kBlk];
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i)
+#pragma unroll
+                    for (int t4 = i & ~3; t4 < kBlk; t4 += 4) {
+                        const float4 x = *reinterpret_cast<const float4*>(&cf.A[type][i][t4]);
+                        A[i][t4] = x.x; A[i][t4 + 1] = x.y; A[i][t4 + 2] = x.z; A[i][t4 + 3] = x.w;
+                    }
+#pragma unroll
+                for (int t4 = 0; t4 < kBlk; t4 += 4) {
+                    const float4 v4 = *reinterpret_cast<const float4*>(&vs[rg * kBlk + t4]), c1 = *reinterpret_cast<const float4*>(&cf.c1[type][t4]);
+                    y[t4] = c1.x * v4.x; y[t4 + 1] = c1.y * v4.y; y[t4 + 2] = c1.z * v4.z; y[t4 + 3] = c1.w * v4.w;
+                }
+                // r in the lanes of type 0, p in those of type 1
+                float z[kBlk];
+#pragma unroll
+                for (int t = 0; t < kBlk; ++t) z[t] = (type ? aq[t] : ak[t]) + __shfl_xor_sync(0xffffffffu, type ? ak[t] : aq[t], 8);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                    for (int t = 0; t < kBlk; ++t) z[t] += __shfl_xor_sync(0xffffffffu, z[t], o);
+#pragma unroll
+                for (int t4 = 0; t4 < kBlk; t4 += 4) {
+                    const float4 c2 = *reinterpret_cast<const float4*>(&cf.c2[type][t4]);
+                    y[t4] = fmaf(c2.x, z[t4], y[t4]); y[t4 + 1] = fmaf(c2.y, z[t4 + 1], y[t4 + 1]);
+                    y[t4 + 2] = fmaf(c2.z, z[t4 + 2], y[t4 + 2]); y[t4 + 3] = fmaf(c2.w, z[t4 + 3], y[t4 + 3]);
+                }
+                // delta in the lanes of type 0, the outputs in those of type 1: both from the eight y of the row
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i) e[i] = __shfl_sync(0xffffffffu, y[i], lane & ~8);
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i)
+#pragma unroll
+                    for (int t = i; t < kBlk; ++t) y[t] = fmaf(A[i][t], e[i], y[t]);
+                // S = G_8 S + sum_i R(8, i) delta_i k_i^T
+                const float ge = cf.gend;
+#pragma unroll
+                for (int c = 0; c < 2 * NC; ++c) mul_f32x2(S[c].x, S[c].y, ge, ge);
+#pragma unroll
+                for (int i = 0; i < kBlk; ++i) {
+                    const float d = __shfl_sync(0xffffffffu, y[i] * cf.rest[i], lane & ~8);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        ptx::fma_f32x2(S[2 * c].x, S[2 * c].y, d, d, k4[i][c].x, k4[i][c].y);
+                        ptx::fma_f32x2(S[2 * c + 1].x, S[2 * c + 1].y, d, d, k4[i][c].z, k4[i][c].w);
+                    }
+                }
+                if (og) {
+                    // a token's output to each lane of type 1 (all eight have all of them)
+                    float x4[4], x2[2];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) x4[i] = (l & 4) ? y[i + 4] : y[i];
+                    x2[0] = (l & 2) ? x4[2] : x4[0]; x2[1] = (l & 2) ? x4[3] : x4[1];
+                    if (type && (l & 7) < left) *op = from_f32<T>((l & 1) ? x2[1] : x2[0]);
+                    op += kBlk * vstride;
+                }
+                __syncwarp();                             // the scratch may be overwritten
+            }
+            bar_arrive<BAR_EMPTY>(buf, NTHR);
+        }
+        if (p.out_state) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    p.out_state[st_off + (size_t)(64 * c + 4 * l + e) * DV] = (e & 1) ? S[2 * c + (e >> 1)].y : S[2 * c + (e >> 1)].x;
+        }
+    }
+}
+
 template <int DK, int DV, typename T, int RPT, int NW, int NH, bool SHORT>
-__global__ void __launch_bounds__((NW + NH) * 32, 2)
+__global__ void __launch_bounds__((NW + NH) * 32, RPT == 1 ? 1 : 2)
 gdn_simt_kernel(const Problem p, const Sched s, const int sms)
 {
     extern __shared__ __align__(16) uint8_t raw[];
@@ -559,8 +691,10 @@ gdn_simt_kernel(const Problem p, const Sched s, const int sms)
         sort_requests(p.cu, p.num_seqs, sm.requests, warp, NW + NH, lane);
         __syncthreads();
     }
-    if (warp < NW) compute<DK, DV, T, RPT, NW, NH, SHORT>(p, s, sm, walk, warp, lane);
-    else helper<DK, DV / (2 * RPT * NW), T, RPT, NW, NH>(p, s, sm, walk, warp - NW, lane);
+    if (warp < NW) {
+        if constexpr (RPT == 1) compute_few<DK, DV, T, NW, NH>(p, s, sm, walk, warp, lane);
+        else compute<DK, DV, T, RPT, NW, NH, SHORT>(p, s, sm, walk, warp, lane);
+    } else helper<DK, DV / (2 * RPT * NW), T, RPT, NW, NH>(p, s, sm, walk, warp - NW, lane);
     allow_successor();       // at the end: a successor's blocks placed among this kernel's would land on the SMs in another order
 }
 
@@ -591,8 +725,10 @@ cudaError_t launch_shape(const Problem& p, const Sched& s, cudaStream_t stream)
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // Rows per warp: 16 have the lowest cost per row, 8 and 4 the lowest time per token.  The finer splits pay while they find idle
-    // SMs: 4 rows (8 per CTA) up to two CTAs per SM, 8 (32 per CTA) up to one and a half.  us for one request of 1,000 tokens at
+    // Rows per warp: 16 have the lowest cost per row, 8, 4 and 2 the lowest time per token.  The finer splits pay while they find idle
+    // SMs: 2 rows up to one CTA per SM (4 rows a CTA; up to twice that with 8: us for 512 tokens at d = 64, 512 / 592 < rows <= 1,184: 4 rows a
+    // CTA 34.9 / 65.5-66.3, 8 rows 43.4 / 43.8-44.2, 4 rows a warp 50.9 / 51.2-51.6; d = 128: 46.7 / 88.6-89.2, 58.3 / 58.7-59.4, 67.6 / 67.7-68.1),
+    // 4 rows (8 per CTA) up to two CTAs per SM, 8 (32 per CTA) up to one and a half.  us for one request of 1,000 tokens at
     // d = 128 with 4 / 8 / 16 rows a warp: 1,024 rows 128 / 193 / 275, 2,304 rows 175 / 194 / 276, 2,432 rows 300 / 194 / 276, 4,096 rows
     // 347 / 195 / 276, 5,120 to 7,040 rows 474-527 / 310 / 277, 8,192 rows 700 / 310 / 278.  (With equal lengths the second line could
     // lie at one CTA per SM, 4,736 rows.)
@@ -602,7 +738,9 @@ cudaError_t launch_shape(const Problem& p, const Sched& s, cudaStream_t stream)
     if (rows > 48ll * sms && p.total_tokens <= (int64_t)kBlk * p.num_seqs) return launch_one<DK, DV, T, 8, 4, 2, true>(p, s, dev, sms, stream);
     if (rows > 48ll * sms) return launch_one<DK, DV, T, 8, 4, 2>(p, s, dev, sms, stream);
     if (rows > 16ll * sms) return launch_one<DK, DV, T, 4, 4, 2>(p, s, dev, sms, stream);
-    return launch_one<DK, DV, T, 2, 2, 4>(p, s, dev, sms, stream);
+    if (rows > 8ll * sms) return launch_one<DK, DV, T, 2, 2, 4>(p, s, dev, sms, stream);
+    if (rows > 4ll * sms) return launch_one<DK, DV, T, 1, 4, 4>(p, s, dev, sms, stream);
+    return launch_one<DK, DV, T, 1, 2, 6>(p, s, dev, sms, stream);
 }
 
 }  // namespace
