@@ -60,9 +60,9 @@ constexpr uint32_t kClusterCtas = 4, kPrepCtas = kClusterCtas - 1;          // o
 // ---- shared memory of a chain CTA (bytes from a 1024-aligned base) -----------------------------
 constexpr uint32_t C_OPS = 0;                              // NSLOT operand slots                             96 KB
 constexpr uint32_t C_KQ = C_OPS + NSLOT * OPS_BYTES;       // 2 x {K, Q}, each 2 halves x [64 rows] x 128 B  64 KB
-constexpr uint32_t C_V = C_KQ + 2 * 32768;                 // 2 halves x [64 rows] x 128 B                     16 KB
-constexpr uint32_t C_O = C_V + 16384;                      // 2 x outputs of a chunk on their way out, layout of V  32 KB
-constexpr uint32_t C_MISC = C_O + 2 * 16384;
+constexpr uint32_t C_V = C_KQ + 2 * 32768;                 // 2 x V, 2 halves x [64 rows] x 128 B               32 KB
+constexpr uint32_t C_O = C_V + 2 * 16384;                  // outputs of a chunk on their way out, layout of V   16 KB
+constexpr uint32_t C_MISC = C_O + 16384;
 // ---- shared memory of a prep CTA: per team K/Q 32 KB | operands 32 KB (same layout as a slot) | T'' 8 KB ------------
 constexpr uint32_t P_TEAM = 32768 + OPS_BYTES + 8192;
 constexpr uint32_t P_OPS = 32768, P_TPP = 32768 + OPS_BYTES;
@@ -77,7 +77,7 @@ constexpr uint32_t F_MISC = F_V + 16384;
 static_assert(P_MISC % 1024 == 0 && C_MISC <= P_MISC && F_MISC <= P_MISC, "");
 
 enum ChainBar {
-    CB_OPS_FULL0 = 0, CB_KQ_FULL0 = 3, CB_U = 5, CB_DONE0 = 6, CB_MMA1 = 10, CB_STATE0, CB_STATE1, CB_OUT0, CB_OUT1,
+    CB_OPS_FULL0 = 0, CB_KQ_FULL0 = 3, CB_U0 = 5, CB_DONE0 = 7, CB_MMA1 = 11, CB_STATE0, CB_STATE1, CB_OUT0, CB_OUT1,
     CB_ACC_FREE0, CB_ACC_FREE1, CB_DECAY_READY0, CB_DECAY_FREE0 = CB_DECAY_READY0 + 4, CB_RING0 = CB_DECAY_FREE0 + 4,
     CB_NUM = CB_RING0 + kRingSlots
 };
@@ -118,13 +118,13 @@ constexpr int kChainTable = 64;
 struct Misc {
     int4 requests[kSelfSort];          // the requests, longest first (see sort_requests)
     int4 chains[kChainTable];          // the CTA's (cluster's) first work items, see chain_entry
-    unsigned long long bars[40];
+    unsigned long long bars[42];
     uint32_t tmem_base;
     volatile uint32_t abort;
     unsigned long long timeout_ns;
     union { ChainMisc c; PrepMisc p; FusedMisc f; };
 };
-static_assert(CB_NUM <= 40 && PB_NUM <= 40 && FB_NUM <= 40, "");
+static_assert(CB_NUM <= 42 && PB_NUM <= 42 && FB_NUM <= 42, "");
 // the part of the records that a prep team reads / that the chain's epilogues read (CL: the split over a cluster)
 template <bool CL> __device__ __forceinline__ auto& prep_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->p.decay[i]; else return m->f.decay[i]; }
 template <bool CL> __device__ __forceinline__ auto& chain_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->c.decay[i]; else return m->f.decay[i]; }
@@ -911,15 +911,17 @@ __device__ void chain_producer(const Ctx& cx, const TcParams* prm, const CUtenso
         if (leader) {
             const uint32_t bar = cx.bar(CB_OPS_FULL0 + (int)(iv % NSLOT));       // (with the operands of the chunk)
             mbar_arrive_expect_tx(bar, 16384u);
-            load_tile(cx.sb + C_V, tm_v, cv.h, cv.row0(), bar);
+            load_tile(cx.sb + C_V + (iv & 1u) * 16384, tm_v, cv.h, cv.row0(), bar);
         }
         __syncwarp();
         cv.advance(); ++iv;
     };
 #pragma unroll 1
     while (cv.valid && !cx.stop()) {
-        // V of chunk i: its buffer is free once U^T of chunk i - 1 has been formed;  K/Q of chunk i: once chunk i - 2 is done
-        if (iv >= 1) cx.wait(CB_U, (iv - 1) & 1u);
+        // V of chunk i: its buffer is free once U^T of chunk i - 2 has been formed;  K/Q of chunk i: once chunk i - 2 is done.  K and Q
+        // come out of L2, where the prep CTAs' copies have brought them, V out of DRAM: with a single buffer it arrived too late for its
+        // U^T.  Two: 32K prefill 623 -> 550 us, one layer of 1,638 tokens 42.8 -> 39.0 us, 36 layers of 410 tokens 646 -> 623 us.
+        if (iv >= 2) cx.wait(CB_U0 + (int)(iv & 1u), ((iv >> 1) - 1u) & 1u);
         load_v();
         if (ik >= 2) cx.wait(CB_DONE0 + (int)((ik - 2) & 3u), ((ik - 2) >> 2) & 1u);
         load_kq();
@@ -997,12 +999,12 @@ __device__ void chain_mma(const Ctx& cx, const TcParams* prm)
         }
         tc_fence_after();
         if (leader) {
-            const uint64_t d_v = d_mn + (sb16 + ((CL ? C_V : F_V) >> 4));              // V^T, M-major
+            const uint64_t d_v = d_mn + (sb16 + (CL ? C_V / 16 + (j & 1u) * 1024 : F_V / 16));              // V^T, M-major
             const uint64_t d_tp = d_sw + (sb16 + (CL ? (C_OPS + OPS_TP) / 16 + os * (OPS_BYTES / 16) : F_TP / 16 + (j & 1u) * 512));
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
                 mma_ss(acc1 + 16 * ks, desc_add(d_v, ks * 2048), desc_add(d_tp, ks * (2048 + 32)), id_wu(64 - 16 * ks), ks > 0);
-            mma_commit(cx.bar(CL ? (int)CB_U : FB_U0 + (int)(j & 1u)));
+            mma_commit(cx.bar((CL ? CB_U0 : FB_U0) + (int)(j & 1u)));
         }
         __syncwarp();
     };
@@ -1298,13 +1300,14 @@ __device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap*
         const int row0 = cc.row0(), nvalid = cc.nvalid();
         const bool first = cc.first() && p.init_state == nullptr;      // zero start state: S0 Q^T was not computed
         const auto& dc = chain_rec<CL>(cx.misc, j & 3u);
-        const uint32_t o_t = CL ? C_O + (j & 1u) * 16384 : F_KQ + (j & 3u) * 32768 + 8192;
+        const uint32_t o_t = CL ? C_O : F_KQ + (j & 3u) * 32768 + 8192;
         uint8_t* const ot = cx.sm + o_t;
-        if (CL || leader) {
+        if (leader) {
+            if (CL && lane == 0) bulk_wait_read();             // the tile of the chunk before has left its buffer
             cx.wait((CL ? CB_DECAY_READY0 : FB_DECAY_READY0) + (int)(j & 3u), (j >> 2) & 1u);
             cx.wait(CL ? CB_OUT0 + (int)(j & 1u) : (int)FB_OUT, CL ? (j >> 1) & 1u : j & 1u);
         }
-        if (!CL) group_sync();
+        group_sync();
         tc_fence_after();
         const uint32_t ta = cx.tmem + ((uint32_t)(w4 * 32 + (CL ? (warp >> 2) * 16 : 0)) << 16), ta3 = ta + tm_acc3<CL>(j), ta2 = ta + tm_acc2<CL>(j);
 #pragma unroll 1
@@ -1347,7 +1350,6 @@ __device__ void chain_out(const Ctx& cx, const TcParams* prm, const CUtensorMap*
         }
         warp_arrive(cx.bar((CL ? CB_DECAY_FREE0 : FB_DECAY_FREE0) + (int)(j & 3u)), lane);    // last read of this chunk's factors
         fence_proxy_async_smem();
-        if (CL && leader && lane == 0) bulk_wait_read();           // the tile of the chunk before has left: the next may take its buffer
         group_sync();
         if (p.out_o) {
             if (nvalid == 64) {
@@ -1447,7 +1449,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     } else if (warp == 3) {
         tmem_alloc(cx.sb + SM_MISC + (uint32_t)offsetof(Misc, tmem_base), 512);
         tmem_relinquish();
-    } else if (tid >= 128 && tid < 128 + 40) {
+    } else if (tid >= 128 && tid < 128 + 42) {
         // Arrivals per phase: one per warp of the arriving group, one where a single thread or an MMA commit completes it
         const int i = tid - 128;
         uint32_t count = 1;
