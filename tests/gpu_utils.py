@@ -78,6 +78,18 @@ def run_library(inp, kernel=0, host=False, fn="gdn_tail_replay", want_o=True, in
     return o_np, st.cpu().numpy().astype(np.float64), launches
 
 
+# The fp32 kernel's instances (RPT, NW, NH), and up to how many value rows (requests x v-heads x dv) per SM a call takes them.  A warp
+# has 2 RPT rows, a stage of the helper warps is 8 NH tokens.  (test_boundary_cpu.py holds this to the dispatch in csrc/gdn_simt.cu.)
+SIMT_INSTANCES = [(4, (1, 2, 6)), (8, (1, 4, 4)), (16, (2, 2, 4)), (48, (4, 4, 2)), (None, (8, 4, 2))]
+
+
+def simt_instance(rows):
+    """The instance that a call with this many value rows takes on this device."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return next(instance for line, instance in SIMT_INSTANCES if line is None or rows <= line * sms)
+
+
 def state_rel_fro(got, ref):
     """Worst per-(request, head) relative Frobenius error and the whole-tensor one."""
     N, H = ref.shape[:2]

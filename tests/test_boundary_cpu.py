@@ -139,3 +139,13 @@ def test_workspace_size(lib):
     assert lib.gdn_workspace_size(ctypes.byref(d)) > dev
     assert lib.gdn_workspace_size(ctypes.byref(_desc(num_v_heads=3))) == 0
     assert lib.gdn_workspace_size(None) == 0
+
+
+def test_fp32_sizes_in_the_gpu_tests_follow_the_dispatch():
+    """The GPU tests choose their sizes by SIMT_INSTANCES, so that they reach every instance of the fp32 kernel."""
+    from gpu_utils import SIMT_INSTANCES
+    text = open(os.path.join(ROOT, "paper_2608_30310_b200", "csrc", "gdn_simt.cu")).read()
+    calls = re.findall(r"^    (?:if \(rows > (\d+)ll \* sms\) )?return launch_one<DK, DV, T, (\d+), (\d+), (\d+)>\(", text, flags=re.M)
+    lower = [int(line or 0) for line, *_ in calls]                        # from the largest calls down
+    upper = [None] + lower[:-1]
+    assert [(u, tuple(map(int, c[1:]))) for u, c in zip(upper, calls)][::-1] == SIMT_INSTANCES

@@ -1,10 +1,10 @@
-"""The fp32 path's blocks of eight tokens, its stages of 16 and 32, and its three splits of the value rows."""
+"""The fp32 path's blocks of eight tokens, its stages of 16 and 32 (48: test_simt_few_rows_gpu.py), its splits of the value rows."""
 import numpy as np
 import pytest
 
 import oracle
-from gdn_workloads import make_inputs, make_raw_inputs
-from gpu_utils import run_library, assert_parity
+from gdn_workloads import make_inputs
+from gpu_utils import run_library, assert_parity, simt_instance
 
 pytestmark = pytest.mark.gpu
 
@@ -12,9 +12,10 @@ LENS = [1, 7, 8, 9, 15, 16, 17, 31, 0, 33, 64, 100]       # around the block, bo
 
 
 @pytest.mark.parametrize("io", ["f32", "bf16"])
-@pytest.mark.parametrize("hv", [1, 2, 8])                 # 4, 8 and 16 rows per warp on a 148-SM device
+@pytest.mark.parametrize("hv", [1, 2, 8, 16])             # rows per warp on a 148-SM device: 4, 8, 16, 16; at dv = 64: 2, 4, 8, 16
 @pytest.mark.parametrize("dk,dv", [(64, 128), (128, 128), (128, 64)])
 def test_block_edges(dk, dv, hv, io):
+    assert 2 * simt_instance(len(LENS) * hv * dv)[0] == {1: 4, 2: 8, 8: 16, 16: 16}[hv] // (2 if dv == 64 and hv < 16 else 1)
     inp = make_inputs(LENS, 1, hv, dk, dv, io, seed=800 + hv + dk + dv)
     rng = np.random.default_rng(5)
     st0 = rng.standard_normal((len(LENS), hv, dk, dv)).astype(np.float32)

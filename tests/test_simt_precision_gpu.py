@@ -4,9 +4,12 @@ import pytest
 
 import oracle
 from gdn_workloads import make_inputs
-from gpu_utils import run_library
+from gpu_utils import run_library, simt_instance
 
 pytestmark = pytest.mark.gpu
+
+# v-heads of a request at dv = 128 -> instance of the kernel on a 148-SM device
+INSTANCES = {2: (1, 2, 6), 8: (1, 4, 4), 16: (2, 2, 4), 32: (4, 4, 2), 64: (8, 4, 2)}
 
 
 def token_by_token_f32(inp):
@@ -25,10 +28,11 @@ def token_by_token_f32(inp):
     return o, S[None]
 
 
-@pytest.mark.parametrize("hv", [2, 16, 32])                # 4, 8 and 16 rows per warp on a 148-SM device
+@pytest.mark.parametrize("hv", list(INSTANCES))
 @pytest.mark.parametrize("decay", ["recipe", "slow"])
 def test_error_is_that_of_the_plain_recurrence(hv, decay):
     """Eight decays enter a block as one factor; their rounding must not add to that of eight single steps."""
+    assert simt_instance(hv * 128) == INSTANCES[hv]
     inp = make_inputs([512], hv, hv, 128, 128, "f32", seed=860 + hv)
     if decay == "slow":
         inp.g[:] = np.random.default_rng(hv).uniform(-0.02, -0.0001, inp.g.shape)
@@ -39,7 +43,7 @@ def test_error_is_that_of_the_plain_recurrence(hv, decay):
         assert np.linalg.norm(got - ref) <= np.linalg.norm(plain - ref)
 
 
-@pytest.mark.parametrize("hv", [2, 16, 32])
+@pytest.mark.parametrize("hv", list(INSTANCES))
 def test_equal_decays_do_not_add_up(hv):
     """The same decay in every block: a rounding of its products would point the same way each time.  Independent roundings leave
     the state with some sqrt(n) of them, n = 9 per block over the 1 / (8 * 0.02) blocks that a decay of e^-0.08 a block remembers;

@@ -4,7 +4,7 @@ import pytest
 
 import oracle
 from gdn_workloads import make_inputs
-from gpu_utils import run_library, assert_parity, to_torch
+from gpu_utils import run_library, assert_parity, simt_instance, to_torch
 
 pytestmark = pytest.mark.gpu
 
@@ -21,10 +21,11 @@ def test_short_requests(dk, dv, io, lens):
 
 
 @pytest.mark.parametrize("off", [0, 4])                    # floats: a state on a 32-byte boundary, and on a 16-byte one only
-@pytest.mark.parametrize("n", [3, 80])
+@pytest.mark.parametrize("n", [3, 6, 12, 20, 80])          # every instance of the kernel on a 148-SM device, that of short requests last
 def test_state_buffers_of_either_alignment(n, off):
     import torch
     import paper_2608_30310_b200 as gdn
+    assert simt_instance(n * 2 * 64) == {3: (1, 2, 6), 6: (1, 4, 4), 12: (2, 2, 4), 20: (4, 4, 2), 80: (8, 4, 2)}[n]
     inp = make_inputs([5 + i % 3 for i in range(n)], 1, 2, 64, 64, "f32", seed=930)
     q, k, v, g, beta, cu = to_torch(inp, "cuda")
     size = n * 2 * 64 * 64
