@@ -4,20 +4,22 @@ import pytest
 
 import oracle
 from gdn_workloads import make_inputs, make_raw_inputs
-from gpu_utils import run_library, assert_parity
+from gpu_utils import run_library, assert_parity, simt_instance
 
 pytestmark = pytest.mark.gpu
 
-LENS = [17, 0, 50, 1]              # blocks and stages of 32 and 48 tokens begun and full, three stages in flight, empty, one token
 
-
+# Blocks and stages begun and full, empty, one token.  203: five stages of 48 tokens or seven of 32, of which three are in flight, so
+# that every buffer is used again.
 @pytest.mark.parametrize("io", ["f32", "bf16"])
 @pytest.mark.parametrize("dk,dv", [(64, 64), (64, 128), (128, 64), (128, 128)])
 @pytest.mark.parametrize("rows", [4 * 128, 8 * 128])          # either split on a 148-SM device (up to 592 and 1,184 rows)
 @pytest.mark.parametrize("raw", [False, True])
-def test_few_rows(dk, dv, rows, raw, io):
-    lens = LENS + [170] if rows == 8 * 128 and dv == 64 else LENS
+@pytest.mark.parametrize("longest", [50, 203])
+def test_few_rows(longest, dk, dv, rows, raw, io):
+    lens = [17, 0, longest, 1] + ([170] if rows == 8 * 128 and dv == 64 else [])
     hv = max(1, rows // dv // len(lens))
+    assert simt_instance(len(lens) * hv * dv) == {4 * 128: (1, 2, 6), 8 * 128: (1, 4, 4)}[rows]
     inp = (make_raw_inputs if raw else make_inputs)(lens, 1, hv, dk, dv, io, seed=880 + dk + dv + hv)
     st0 = np.random.default_rng(6).standard_normal((len(lens), hv, dk, dv)).astype(np.float32)
     o, st, _ = run_library(inp, kernel=1, canary=True, init_state=st0, raw_inputs=raw)
