@@ -115,16 +115,17 @@ struct PrepMisc { PrepDecay decay[4]; };
 struct __align__(16) FusedDecay { float G2[64], beta[64], eG[64], colfb[32], norms[128]; float G2mid, wb, cfin; int rescale; float bRest[64], eGk[64]; };
 struct FusedMisc { FusedDecay decay[4]; };
 constexpr int kChainTable = 64;
+constexpr int kBars = 40;              // every kind of CTA initialises as many
 struct Misc {
     int4 requests[kSelfSort];          // the requests, longest first (see sort_requests)
     int4 chains[kChainTable];          // the CTA's (cluster's) first work items, see chain_entry
-    unsigned long long bars[42];
+    unsigned long long bars[kBars];
     uint32_t tmem_base;
     volatile uint32_t abort;
     unsigned long long timeout_ns;
     union { ChainMisc c; PrepMisc p; FusedMisc f; };
 };
-static_assert(CB_NUM <= 42 && PB_NUM <= 42 && FB_NUM <= 42, "");
+static_assert(CB_NUM <= kBars && PB_NUM <= kBars && FB_NUM <= kBars, "");
 // the part of the records that a prep team reads / that the chain's epilogues read (CL: the split over a cluster)
 template <bool CL> __device__ __forceinline__ auto& prep_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->p.decay[i]; else return m->f.decay[i]; }
 template <bool CL> __device__ __forceinline__ auto& chain_rec(Misc* m, uint32_t i) { if constexpr (CL) return m->c.decay[i]; else return m->f.decay[i]; }
@@ -1449,7 +1450,7 @@ gdn_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CUte
     } else if (warp == 3) {
         tmem_alloc(cx.sb + SM_MISC + (uint32_t)offsetof(Misc, tmem_base), 512);
         tmem_relinquish();
-    } else if (tid >= 128 && tid < 128 + 42) {
+    } else if (tid >= 128 && tid < 128 + kBars) {
         // Arrivals per phase: one per warp of the arriving group, one where a single thread or an MMA commit completes it
         const int i = tid - 128;
         uint32_t count = 1;
