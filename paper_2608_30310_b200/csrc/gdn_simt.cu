@@ -9,15 +9,17 @@
 // which is 3 dk dv FMAs per token and head; the rows of S are independent of each other.
 //
 // A CTA owns a slice of 2 RPT NW rows of one chain (request, v-head): NW warps of 2 RPT rows each.  Sixteen lanes share RPT
-// rows, DK / 16 columns per lane, all in registers (RPT = 1, for calls with few rows: see compute_few).  The dot products of a token are reduced over the sixteen lanes by a
+// rows, DK / 16 columns per lane, all in registers.  The dot products of a token are reduced over the sixteen lanes by a
 // reduce-scatter that leaves each lane one of the 2 RPT values (a row's r or p) for all eight tokens, so that the 8 x 8 products run
-// inside a lane; eight tokens share the latency (one token at a time, each waited for a shuffle reduction: 400 ns a token).  NH helper warps
-// run ahead by a stage of 8 NH tokens: they load k, q, g and beta, apply the input stage if asked, and form the 8 x 8
+// inside a lane; eight tokens share the latency (one token at a time, each waited for a shuffle reduction: 400 ns a token).
+// Calls with few rows have RPT = 1: eight lanes each have all of a row's r, the other eight its p (see compute_few).  NH helper
+// warps run ahead by a stage of 8 NH tokens: they load k, q, g and beta, apply the input stage if asked, and form the 8 x 8
 // coefficients.
 //
 // What bounds it: with RPT = 8 the FMA pipe (240 of its cycles per token and 16 rows, 192 of them the 3 dk dv) and, nearly as
 // much, the shared-memory loads: a 16-byte load occupies the SM's load path for four cycles whatever it broadcasts, so a loaded
-// k or q value has to serve many rows (8 lanes to RPT = 4 rows: 340 cycles a token, bound by the loads; RPT = 1: four times as many).
+// k or q value has to serve many rows (8 lanes to 4 rows: 340 cycles a token, bound by the loads; to one row: four times as many).
+// Where warps are few, the chain of dependent instructions of a block.
 //
 // This path serves fp32 io (tolerance 1e-4 rules out tf32/bf16 tensor cores) and every shape the tensor-core path does not cover.
 #include "common.cuh"
@@ -43,6 +45,10 @@ struct __align__(16) Coef {
     float gend; float pad[3];             // G_8
 };
 
+// what each compute warp keeps of the block: R(8, i) delta_i and v, [token][row];  RPT = 1: v, [row][token]
+template <int RPT, int NW> struct __align__(16) Scratch { float dr[NW][kBlk][2 * RPT], v[NW][kBlk][2 * RPT]; };
+template <int NW> struct __align__(16) Scratch<1, NW> { float v[NW][2][kBlk]; };
+
 template <int DK, int RPT, int NW, int NH>
 struct Smem {
     static constexpr int LD = DK + 4;     // row stride: 16-byte aligned, and eight rows at one column fall into different banks
@@ -51,8 +57,7 @@ struct Smem {
     __align__(16) double al[NH][kBlk];                   // helpers: alpha and beta of the block at hand
     float be[NH][kBlk];
     __align__(16) float mn[NH][2][kBlk][kBlk];           // helpers: [0][i][t] -M, [1][i][t] N
-    __align__(16) float dr[NW][kBlk][2 * RPT];           // R(8, i) delta_i by token
-    __align__(16) float v[NW][kBlk][2 * RPT];            // v of the block
+    Scratch<RPT, NW> own;
     int4 requests[kSelfSort];                            // the requests, longest first (see sort_requests)
 };
 
@@ -415,7 +420,7 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
                 const float (*qs)[Smem<DK, RPT, NW, NH>::LD] = &sm.q[buf][sb * kBlk];
                 const Coef& cf = sm.coef[buf][sb];
 #pragma unroll
-                for (int i = 0; i < VPL; ++i) sm.v[warp][vtok][vrow + i] = vn.get(i);
+                for (int i = 0; i < VPL; ++i) sm.own.v[warp][vtok][vrow + i] = vn.get(i);
                 vp += kBlk * vstride;
                 vn.load(vp, vtok < left - kBlk);
                 __syncwarp();
@@ -483,7 +488,7 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
                         for (int x = 0; x < TB; ++x) z[x][0] += __shfl_xor_sync(0xffffffffu, z[x][0], o);
 #pragma unroll
                     for (int x = 0; x < TB; ++x)
-                        y[t0 + x] = fmaf(cf.c2[type][t0 + x], z[x][0], cf.c1[type][t0 + x] * sm.v[warp][t0 + x][wrow]);
+                        y[t0 + x] = fmaf(cf.c2[type][t0 + x], z[x][0], cf.c1[type][t0 + x] * sm.own.v[warp][t0 + x][wrow]);
                 }
                 // delta in the lanes of type 0, the outputs in those of type 1: both from the eight y of the row
                 float e[kBlk];
@@ -497,7 +502,7 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
                 }
                 if (l % (8 / RPT) == 0 && type == 0) {
 #pragma unroll
-                    for (int i = 0; i < kBlk; ++i) sm.dr[warp][i][wrow] = y[i] * rest[i];
+                    for (int i = 0; i < kBlk; ++i) sm.own.dr[warp][i][wrow] = y[i] * rest[i];
                 }
                 __syncwarp();
                 if (og) {
@@ -518,7 +523,7 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
                 for (int i = 0; i < (SHORT ? min(left, kBlk) : kBlk); ++i) {
                     float dv[RPT];
 #pragma unroll
-                    for (int r = 0; r < RPT; ++r) dv[r] = sm.dr[warp][i][rg * RPT + (row ^ r)];
+                    for (int r = 0; r < RPT; ++r) dv[r] = sm.own.dr[warp][i][rg * RPT + (row ^ r)];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
                         const float4 k4 = *reinterpret_cast<const float4*>(&ks[i][64 * c + 4 * l]);
@@ -549,8 +554,9 @@ __device__ void compute(const Problem& p, const Sched& s, Smem<DK, RPT, NW, NH>&
 // ---- compute warp of calls with few rows: one row per sixteen lanes (RPT = 1) -------------------------------------------------
 // With a warp to a scheduler nothing but the chain of dependent instructions of a block counts: every lane has all eight r or p of its
 // row, delta goes from lane to lane by shuffles, and k serves the products and the update from registers.  us for one request of 512
-// tokens: d = 64 (256 rows) 50.8 with two rows per sixteen lanes, 34.4 so, 37.3 with the sums scattered until a lane has one token
-// (half the instructions, but one behind the other), 38.5 so and with k and q loaded a block ahead; d = 128: 67.2, 46.3, 47.5, 47.9.
+// tokens and four heads, the mean of five calls that start on an idle GPU: d = 64 50.8 with two rows per sixteen lanes, 34.4 so, 37.3
+// with the sums scattered until a lane has one token (half the instructions, but one behind the other), 38.5 so and with k and q
+// loaded a block ahead; d = 128: 67.2, 46.3, 47.5, 47.9.  In a long row of calls d = 64 takes 49.8, 33.1, 36.0, 37.5.
 template <int DK, int DV, typename T, int NW, int NH>
 __device__ void compute_few(const Problem& p, const Sched& s, Smem<DK, 1, NW, NH>& sm, Walk<DV / (2 * NW)> walk, int warp, int lane)
 {
@@ -558,7 +564,7 @@ __device__ void compute_few(const Problem& p, const Sched& s, Smem<DK, 1, NW, NH
     const int l = lane & 15, rg = lane >> 4, type = l >> 3;                // type 1: the outputs' lanes, 0: delta's
     const T* __restrict__ vg = (const T*)p.v;
     T* __restrict__ og = (T*)p.out_o;
-    float* const vs = &sm.v[warp][0][0];                  // [row][token]
+    float* const vs = &sm.own.v[warp][0][0];              // [row][token]
     uint32_t stage = 0;
     Item it;
     while (walk.next(p, s, sm.requests, it)) {
@@ -726,12 +732,22 @@ cudaError_t launch_shape(const Problem& p, const Sched& s, cudaStream_t stream)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // Rows per warp: 16 have the lowest cost per row, 8, 4 and 2 the lowest time per token.  The finer splits pay while they find idle
-    // SMs: 2 rows up to one CTA per SM (4 rows a CTA; up to twice that with 8: us for 512 tokens at d = 64, 512 / 592 < rows <= 1,184: 4 rows a
-    // CTA 34.9 / 65.5-66.3, 8 rows 43.4 / 43.8-44.2, 4 rows a warp 50.9 / 51.2-51.6; d = 128: 46.7 / 88.6-89.2, 58.3 / 58.7-59.4, 67.6 / 67.7-68.1),
-    // 4 rows (8 per CTA) up to two CTAs per SM, 8 (32 per CTA) up to one and a half.  us for one request of 1,000 tokens at
-    // d = 128 with 4 / 8 / 16 rows a warp: 1,024 rows 128 / 193 / 275, 2,304 rows 175 / 194 / 276, 2,432 rows 300 / 194 / 276, 4,096 rows
-    // 347 / 195 / 276, 5,120 to 7,040 rows 474-527 / 310 / 277, 8,192 rows 700 / 310 / 278.  (With equal lengths the second line could
-    // lie at one CTA per SM, 4,736 rows.)
+    // SMs (us a call; tests/gpu_utils.py has the same lines).
+    // 2 rows a warp up to one CTA per SM, CTAs of 4 rows and then of 8.  512 tokens, 512 / 592 < rows <= 1,184, d = 64: CTAs of 4 rows
+    //   34.9 / 65.5-66.3, of 8 rows 43.4 / 43.8-44.2, 4 rows a warp 50.9 / 51.2-51.6; d = 128: 46.7 / 88.6-89.2, 58.3 / 58.7-59.4,
+    //   67.6 / 67.7-68.1.  Short calls gain less and lose nothing, 4 rows a warp -> now, 512 and 1,152 rows: one token 3.3 -> 3.1 and
+    //   3.4 -> 3.3 at d = 64, 4.5 -> 4.0 and 4.8 -> 4.2 at d = 128; 64 tokens 8.4 -> 6.5, 8.5 -> 7.4, 11.2 -> 8.4, 11.5 -> 9.7.
+    // 4 rows (8 per CTA) up to two CTAs per SM, 8 (32 per CTA) up to one and a half.  One request of 1,000 tokens at d = 128 with
+    //   4 / 8 / 16 rows a warp: 1,024 rows 128 / 193 / 275, 2,304 rows 175 / 194 / 276, 2,432 rows 300 / 194 / 276, 4,096 rows
+    //   347 / 195 / 276, 5,120 to 7,040 rows 474-527 / 310 / 277, 8,192 rows 700 / 310 / 278.  So requests of one length would have
+    //   the second line at one CTA per SM, 4,736 rows; it lies higher for ragged ones.  4,737 to 7,104 rows, 8 against 16 rows a
+    //   warp: lengths equal or a single request 10-14 % longer; three requests of 60-500 or 250-500 tokens 16 % shorter to 9 %
+    //   longer, five to 25 requests 16 % shorter to 2 % longer (d = 128: 113-129 against 135, 25 requests 119 / 135).
+    // All this is for a call that has the GPU to itself.  A finer split costs more issue slots per row (every slice has its own
+    // helpers), and a CTA with 2 rows a warp fills an SM, so calls on other streams wait once the CTAs outnumber the SMs.  A call of 4
+    // heads on each of 2 / 4 / 8 streams, 4 rows a warp -> now: 196 / 201 / 264 -> 129 / 222 / 460 (2,048 tokens, d = 64), 134 / 183 /
+    // 313 -> 154 / 302 / 610 (1,024 tokens, d = 128).  With room for two CTAs an SM (four helpers) 133 / 195 / 332 and 149 / 253 / 501,
+    // but single calls 2.6 and 12 % longer.  The same requests in one call: 126 / 160 / 254 and 112 / 177 / 198.
     const long long rows = (long long)p.num_seqs * p.Hv * DV;
     // Requests that do not fill a block on average: the instance that leaves out tokens past the end (1,000 requests of 1-8 tokens,
     // 32 heads: 443 -> 365 us at d = 64, 1,565 -> 1,232 us at d = 128; where blocks are full its branches cost 2 %).
